@@ -32,57 +32,141 @@ namespace dpf {
 __device__ __forceinline__ float round_bf16(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
 
 // On the tensor cores (tcgen05):
-// One CTA of 128 threads per 128-row x npad-column tile of C (npad <= 64 columns of a
-// TMEM accumulator in FP32; blockIdx.y picks the column tile) and one slice of K
-// (blockIdx.z; the slices of a long K add their partial products into C, which the
-// caller has zeroed, with atomic adds: the plain-store epilogue only). K is taken in
-// chunks of 128 bytes a row (64 BF16 or 32 TF32 values): the threads load op(A) and
-// op(B)^T from global memory, round them to the operand format and write them in the
-// K-major layout without swizzle; one thread issues the MMAs (four 32-byte K steps a
-// chunk) and commits them to an mbarrier that every thread waits on (bounded; the CTA
-// agrees on the outcome before it reuses the tiles); thread r then reads row r of the
-// accumulator for the epilogue.
+// One CTA of 256 threads per 128-row x npad-column tile of C (npad <= 64 columns of a
+// TMEM accumulator in FP32) and one slice of K (the slices of a long K add their partial
+// products into C, which the caller has zeroed: the plain-store epilogue only). The
+// threads load op(A) and op(B)^T of a chunk of K from global memory, round them to the
+// operand format and write them in the K-major layout without swizzle; one thread issues
+// the MMAs (one per 32 bytes of K) and commits them to an mbarrier that every thread waits
+// on (bounded; the CTA agrees on the outcome before it reuses the tiles); a warp then reads
+// its 32 rows of the accumulator for the epilogue.
 // PREC 0: BF16 operands (kind::f16), the forward pass's own rounding; PREC 1: 3xTF32
 // (A_hi B_hi + A_hi B_lo + A_lo B_hi, kind::tf32), about FP32 accuracy.
-constexpr int TG_NT = 128;
-constexpr int TG_ROWB = 128;        // bytes of one K chunk of a row
-constexpr int TG_KC16 = TG_ROWB / 16;
+//
+// What bounds it: the latency of staging. A training minibatch (1024 rows, width 256) is
+// 0.13 GFLOP a product, a microsecond of MMA work, so a CTA's time is the loads of its
+// operands from L2. A thread therefore moves units of 8 consecutive K values of one row: two
+// 16-byte loads (or, for an operand that is contiguous along its rows, 8 loads each coalesced
+// over the warp's 32 rows), one rounding, one 16-byte store, which the 8 x 16-byte core
+// matrices of consecutive rows take without bank conflicts; four units are in flight at once,
+// and a chunk is as long as shared memory holds twice on an SM (256 BF16 or 64 TF32 values of
+// K), so that a forward product is one round of loads, one of MMAs and one epilogue.
+constexpr int TG_NT = 256;
 constexpr int TG_SPIN = 1 << 22;
+constexpr int TG_UNITS = 4;  // staging units a thread holds in flight
 
 template <int PREC>
-__device__ __forceinline__ void tg_put(unsigned char* hi, unsigned char* lo, int r, int c, float v) {
-  if (PREC == 0) {
-    *(__nv_bfloat16*)(hi + tc::kmajor_offset(r, 2 * c, TG_KC16)) = __float2bfloat16_rn(v);
-  } else {
-    float h, l;
-    tc::split_tf32(v, h, l);
-    *(float*)(hi + tc::kmajor_offset(r, 4 * c, TG_KC16)) = h;
-    *(float*)(lo + tc::kmajor_offset(r, 4 * c, TG_KC16)) = l;
+__host__ __device__ constexpr int tg_chunk() { return PREC == 0 ? 256 : 64; }  // K values a chunk at most
+template <int PREC>
+__host__ __device__ constexpr int tg_kstep() { return PREC == 0 ? 16 : 8; }    // K values an MMA
+
+// One product of a launch.
+struct TgProb {
+  const float* A;
+  const float* B;
+  float* C;
+  const float* bias;
+  const float* mask;
+  float* asum;  // or null: asum[m] += sum_k op(A)(m, k), from the unrounded values (TA only)
+  int M, N, K, lda, ldb, ldc;
+  int ta, tb, epi, round;
+  int npad, mt, nt, ks, kslice;  // column tile, tiles, slices of K
+  int va, vb, vc;                // rows of A, B, C start on 16 bytes
+};
+// Up to two independent products in one launch: CTAs below `first` serve p[0].
+struct TgLaunch {
+  TgProb p[2];
+  int first;
+  int kc;          // K values a chunk (a multiple of the MMA's), for both
+  uint32_t ncols;  // TMEM columns
+  int* err;
+};
+
+// Stage R rows (row0 .. ; `rows` of them real) of op(X) for K values k0 .. k0 + kc - 1, where X
+// is contiguous along its rows' index when `trans`, else along K. RS: R rounded up to a power
+// of two that divides the block's threads, so that a thread stages one row. Returns the sum of
+// the values this thread staged.
+template <int PREC, int RS>
+__device__ __forceinline__ float tg_stage(const float* __restrict__ X, int ld, bool trans, bool vec, int row0, int R,
+                                          int rows, int k0, int kend, int kc, unsigned char* hi, unsigned char* lo) {
+  constexpr int KS = tg_kstep<PREC>();
+  const int left = kend - k0 < kc ? kend - k0 : kc;
+  const int r = threadIdx.x % RS, step = TG_NT / RS, nu = (left + KS - 1) / KS * KS / 8;
+  const int kc16 = PREC == 0 ? kc / 8 : kc / 4;
+  const long long row = (long long)row0 + r;
+  const bool live = row < rows;
+  float sum = 0.f;
+  if (r >= R) return sum;
+  for (int u0 = threadIdx.x / RS; u0 < nu; u0 += step * TG_UNITS) {
+    float v[TG_UNITS][8];
+#pragma unroll
+    for (int q = 0; q < TG_UNITS; ++q) {
+      const int k = k0 + 8 * (u0 + q * step);
+      const bool on = live && u0 + q * step < nu;
+      if (!trans && vec && k + 8 <= kend) {
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+        if (on) {
+          const float4* src = reinterpret_cast<const float4*>(X + row * ld + k);
+          a = src[0];
+          b = src[1];
+        }
+        v[q][0] = a.x; v[q][1] = a.y; v[q][2] = a.z; v[q][3] = a.w;
+        v[q][4] = b.x; v[q][5] = b.y; v[q][6] = b.z; v[q][7] = b.w;
+      } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          v[q][j] = on && k + j < kend ? (trans ? X[(long long)(k + j) * ld + row] : X[row * ld + k + j]) : 0.f;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < TG_UNITS; ++q) {
+      const int u = u0 + q * step;
+      if (u >= nu) break;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) sum += v[q][j];
+      if (PREC == 0) {
+        __nv_bfloat162 h[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) h[j] = __floats2bfloat162_rn(v[q][2 * j], v[q][2 * j + 1]);
+        *reinterpret_cast<uint4*>(hi + tc::kmajor_offset(r, 16 * u, kc16)) = *reinterpret_cast<const uint4*>(h);
+      } else {
+        float h[8], l[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) tc::split_tf32(v[q][j], h[j], l[j]);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const uint32_t o = tc::kmajor_offset(r, 32 * u + 16 * j, kc16);
+          *reinterpret_cast<float4*>(hi + o) = make_float4(h[4 * j], h[4 * j + 1], h[4 * j + 2], h[4 * j + 3]);
+          *reinterpret_cast<float4*>(lo + o) = make_float4(l[4 * j], l[4 * j + 1], l[4 * j + 2], l[4 * j + 3]);
+        }
+      }
+    }
   }
+  return sum;
 }
 
-template <bool TA, bool TB, int EPI, int PREC>
-__global__ void __launch_bounds__(TG_NT)
-    tgemm_kernel(int M, int N, int K, const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
-                 float* __restrict__ C, int ldc, const float* __restrict__ bias, const float* __restrict__ mask,
-                 int round, int npad, uint32_t ncols, int kslice, int* err) {
+template <int PREC>
+__global__ void __launch_bounds__(TG_NT, 2) tgemm_kernel(const __grid_constant__ TgLaunch g) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ __align__(8) uint64_t bar;
   __shared__ uint32_t s_taddr;
-  constexpr int KC = PREC == 0 ? TG_ROWB / 2 : TG_ROWB / 4;  // K values a chunk
+  constexpr int KB = PREC == 0 ? 2 : 4;  // bytes of an operand value
   const int tid = threadIdx.x, w = tid >> 5;
-  const uint32_t a_bytes = 128u * TG_ROWB, b_bytes = (uint32_t)npad * TG_ROWB;
+  const bool second = (int)blockIdx.x >= g.first;
+  const TgProb& p = g.p[second ? 1 : 0];
+  const int bid = (int)blockIdx.x - (second ? g.first : 0);
+  const int tm = bid % p.mt, tn = bid / p.mt % p.nt, tk = bid / p.mt / p.nt;
+  const int npad = p.npad, kc = g.kc, kc16 = kc * KB / 16;
+  const uint32_t a_bytes = 128u * kc * KB, b_bytes = (uint32_t)npad * kc * KB;
   unsigned char* a_hi = sm;
   unsigned char* b_hi = sm + a_bytes;
-  unsigned char* a_lo = sm + a_bytes + b_bytes;  // 3xTF32 only
+  unsigned char* a_lo = b_hi + b_bytes;  // 3xTF32 only
   unsigned char* b_lo = a_lo + a_bytes;
-  const long long m0 = (long long)blockIdx.x * 128;
-  const int n0 = blockIdx.y * npad;                      // this CTA's first column
-  const int kbeg = blockIdx.z * kslice;                  // and its slice of K
-  const int kend = kbeg + kslice < K ? kbeg + kslice : K;
-  const bool split = gridDim.z > 1;
+  const int m0 = tm * 128, n0 = tn * npad;  // this CTA's first row and column
+  const int kbeg = tk * p.kslice;           // and its slice of K
+  const int kend = kbeg + p.kslice < p.K ? kbeg + p.kslice : p.K;
   if (w == 0) {
-    tc::tmem_alloc(&s_taddr, ncols);
+    tc::tmem_alloc(&s_taddr, g.ncols);
     tc::tmem_relinquish();
   }
   if (tid == 0) {
@@ -96,40 +180,26 @@ __global__ void __launch_bounds__(TG_NT)
   const uint32_t idesc = tc::instr_desc(PREC == 0 ? tc::FMT_BF16 : tc::FMT_TF32, 128, npad);
   int ok = 1;
   uint32_t phase = 0;
-  for (int k0 = kbeg; k0 < kend && ok; k0 += KC) {
-    // op(A) rows m0 .. m0 + 127 and op(B)^T rows 0 .. npad - 1, K columns k0 .. k0 + KC - 1;
-    // the index runs fastest along the operand's contiguous dimension
-    for (int e = tid; e < 128 * KC; e += TG_NT) {
-      const int r = TA ? e % 128 : e / KC, c = TA ? e / 128 : e % KC;
-      const long long m = m0 + r;
-      const int k = k0 + c;
-      float v = 0.f;
-      if (m < M && k < kend) v = TA ? A[(long long)k * lda + m] : A[m * lda + k];
-      tg_put<PREC>(a_hi, a_lo, r, c, v);
-    }
-    for (int e = tid; e < npad * KC; e += TG_NT) {
-      const int nl = TB ? e / KC : e % npad, c = TB ? e % KC : e / npad;
-      const int n = n0 + nl, k = k0 + c;
-      float v = 0.f;
-      if (n < N && k < kend) v = TB ? B[(long long)n * ldb + k] : B[(long long)k * ldb + n];
-      tg_put<PREC>(b_hi, b_lo, nl, c, v);
-    }
+  float asum = 0.f;  // of row m0 + tid % 128
+  for (int k0 = kbeg; k0 < kend && ok; k0 += kc) {
+    asum += tg_stage<PREC, 128>(p.A, p.lda, p.ta, p.va, m0, 128, p.M, k0, kend, kc, a_hi, a_lo);
+    tg_stage<PREC, 64>(p.B, p.ldb, !p.tb, p.vb, n0, npad, p.N, k0, kend, kc, b_hi, b_lo);
     tc::fence_proxy_async();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
     if (tid == 0) {
       const uint32_t sah = smem_addr(a_hi), sbh = smem_addr(b_hi), sal = smem_addr(a_lo), sbl = smem_addr(b_lo);
-#pragma unroll
-      for (int ks = 0; ks < TG_ROWB / 32; ++ks) {
+      const int left = kend - k0, steps = ((left < kc ? left : kc) + tg_kstep<PREC>() - 1) / tg_kstep<PREC>();
+      for (int ks = 0; ks < steps; ++ks) {
         const uint32_t off = (uint32_t)ks * 256;
         const uint32_t acc = (k0 > kbeg || ks > 0) ? 1u : 0u;
         if (PREC == 0) {
-          tc::mma_f16(taddr, tc::smem_desc(sah + off, TG_KC16), tc::smem_desc(sbh + off, TG_KC16), idesc, acc);
+          tc::mma_f16(taddr, tc::smem_desc(sah + off, kc16), tc::smem_desc(sbh + off, kc16), idesc, acc);
         } else {  // small terms first, then the leading one
-          tc::mma_tf32(taddr, tc::smem_desc(sal + off, TG_KC16), tc::smem_desc(sbh + off, TG_KC16), idesc, acc);
-          tc::mma_tf32(taddr, tc::smem_desc(sah + off, TG_KC16), tc::smem_desc(sbl + off, TG_KC16), idesc, 1);
-          tc::mma_tf32(taddr, tc::smem_desc(sah + off, TG_KC16), tc::smem_desc(sbh + off, TG_KC16), idesc, 1);
+          tc::mma_tf32(taddr, tc::smem_desc(sal + off, kc16), tc::smem_desc(sbh + off, kc16), idesc, acc);
+          tc::mma_tf32(taddr, tc::smem_desc(sah + off, kc16), tc::smem_desc(sbl + off, kc16), idesc, 1);
+          tc::mma_tf32(taddr, tc::smem_desc(sah + off, kc16), tc::smem_desc(sbh + off, kc16), idesc, 1);
         }
       }
       tc::commit(&bar);
@@ -140,73 +210,113 @@ __global__ void __launch_bounds__(TG_NT)
     ok = __syncthreads_and(done ? 1 : 0);  // every thread saw the MMAs finish before the tiles change
   }
   if (!ok) {
-    if (tid == 0) atomicOr(err, ERR_TIMEOUT);
+    if (tid == 0) atomicOr(g.err, ERR_TIMEOUT);
     tc::bar_wait(&bar, phase ^ 1u, TG_SPIN);  // give MMAs still in flight a second bound
   } else {
-    const long long m = m0 + tid;
-    for (int c0 = 0; c0 < npad; c0 += 16) {
+    if (p.asum && tn == 0 && m0 + tid % 128 < p.M) atomicAdd(p.asum + m0 + tid % 128, asum);
+    // warp w holds rows 32 (w mod 4) .. + 31, 16 columns at a time, every other block of 16
+    const long long m = m0 + tid % 128;
+    const bool split = p.ks > 1;
+    for (int c0 = 16 * (w >> 2); c0 < npad; c0 += 32) {
       float v[16];
-      tc::ld16(taddr + ((uint32_t)(32 * w) << 16) + (uint32_t)c0, v);
-      if (m < M) {
+      tc::ld16(taddr + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)c0, v);
+      if (m >= p.M) continue;
+      const int n = n0 + c0;
+      float* c = p.C + m * p.ldc + n;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        if (n + j >= p.N) break;
+        float x = v[j];
+        if (p.epi == 1) {
+          x = fmaxf(x + p.bias[n + j], 0.f);
+          if (p.round) x = round_bf16(x);
+        } else if (p.epi == 2) {
+          x += p.bias[n + j];
+        } else if (p.epi == 3) {
+          x = p.mask[m * p.ldc + n + j] > 0.f ? x : 0.f;
+        }
+        v[j] = x;
+      }
+      if (p.vc && n + 16 <= p.N) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float4 x = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+          if (split)
+            atomicAdd(reinterpret_cast<float4*>(c) + j, x);
+          else
+            reinterpret_cast<float4*>(c)[j] = x;
+        }
+      } else {
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-          const int n = n0 + c0 + j;
-          if (n >= N) break;
-          float x = v[j];
-          if (EPI == 1) {
-            x = fmaxf(x + bias[n], 0.f);
-            if (round) x = round_bf16(x);
-          } else if (EPI == 2) {
-            x += bias[n];
-          } else if (EPI == 3) {
-            x = mask[m * ldc + n] > 0.f ? x : 0.f;
-          }
+          if (n + j >= p.N) break;
           if (split)
-            atomicAdd(C + m * ldc + n, x);
+            atomicAdd(c + j, v[j]);
           else
-            C[m * ldc + n] = x;
+            c[j] = v[j];
         }
       }
     }
   }
   tc::fence_before();
   __syncthreads();
-  if (w == 0) tc::tmem_dealloc(taddr, ncols);
+  if (w == 0) tc::tmem_dealloc(taddr, g.ncols);
 }
 
-// C = op(A) op(B) with the epilogue EPI on the tensor cores: BF16 operands when the
-// proposal trains in its BF16 form, 3xTF32 otherwise. Column tiles of up to 64; a long
-// K (the batch dimension of a weight gradient) is split over CTAs that accumulate into C.
-template <bool TA, bool TB, int EPI>
-static void tgemm(cudaStream_t s, int prec_bf16, int* err, int M, int N, int K, const float* A, int lda,
-                  const float* B, int ldb, float* C, int ldc, const float* bias = nullptr,
-                  const float* mask = nullptr, int round = 0) {
-  const int npad = std::min(64, (N + 15) / 16 * 16);
-  const uint32_t ncols = npad <= 32 ? 32u : 64u;
-  const int mt = (M + 127) / 128, nt = (N + npad - 1) / npad;
-  const int kc = prec_bf16 ? TG_ROWB / 2 : TG_ROWB / 4;
-  // slices of at least 4 chunks, enough of them for about 152 CTAs (plain-store products)
-  int ks = 1;
-  if (EPI == 0)
-    while (ks < 16 && (long long)mt * nt * ks * 2 <= 152 && K / (2 * ks) >= 4 * kc) ks *= 2;
-  const int kslice = (K + ks - 1) / ks / kc * kc + ((K + ks - 1) / ks % kc ? kc : 0);
-  ks = (K + kslice - 1) / kslice;  // every slice holds part of K
-  if (ks > 1) cudaMemsetAsync(C, 0, sizeof(float) * (size_t)M * ldc, s);
-  const dim3 grid((unsigned)mt, (unsigned)nt, (unsigned)ks);
+// C = op(A) op(B) with the epilogue epi. A weight gradient (TA, epi 0) has the minibatch as its
+// K and few tiles, so its K is split over CTAs that accumulate into C (zeroed by the caller).
+static TgProb tg_prob(bool ta, bool tb, int epi, int M, int N, int K, const float* A, int lda, const float* B, int ldb,
+                      float* C, int ldc, const float* bias = nullptr, const float* mask = nullptr, int round = 0,
+                      float* asum = nullptr) {
+  TgProb p{};
+  p.A = A; p.B = B; p.C = C; p.bias = bias; p.mask = mask; p.asum = asum;
+  p.M = M; p.N = N; p.K = K; p.lda = lda; p.ldb = ldb; p.ldc = ldc;
+  p.ta = ta; p.tb = tb; p.epi = epi; p.round = round;
+  p.npad = std::min(64, (N + 15) / 16 * 16);
+  p.mt = (M + 127) / 128;
+  p.nt = (N + p.npad - 1) / p.npad;
+  auto rows16 = [](const float* q, int ld) { return (int)(((uintptr_t)q | (uintptr_t)(4 * (size_t)ld)) % 16 == 0); };
+  p.va = rows16(A, lda);
+  p.vb = rows16(B, ldb);
+  p.vc = rows16(C, ldc);
+  // slices of at least 128 rows, enough of them for about 96 CTAs: a longer slice leaves SMs
+  // idle at minibatch sizes, a shorter one adds as many partial tiles into C as it saves loads
+  p.ks = 1;
+  if (epi == 0)
+    while (p.ks < 64 && (long long)p.mt * p.nt * p.ks * 2 <= 96 && K / (2 * p.ks) >= 128) p.ks *= 2;
+  p.kslice = ((K + p.ks - 1) / p.ks + 15) / 16 * 16;
+  p.ks = (K + p.kslice - 1) / p.kslice;  // every slice holds part of K
+  return p;
+}
+
+template <int PREC>
+static void tg_launch(cudaStream_t s, int* err, const TgProb& a, const TgProb* b) {
+  TgLaunch g{};
+  g.p[0] = a;
+  g.p[1] = b ? *b : a;
+  g.err = err;
+  const long long n0 = (long long)a.mt * a.nt * a.ks, n1 = b ? (long long)b->mt * b->nt * b->ks : 0;
+  g.first = (int)n0;
+  const int longest = b ? std::max(std::min(a.K, a.kslice), std::min(b->K, b->kslice)) : std::min(a.K, a.kslice);
+  const int step = tg_kstep<PREC>();
+  g.kc = std::min(tg_chunk<PREC>(), (longest + step - 1) / step * step);
+  const int npad = std::max(a.npad, b ? b->npad : 0);
+  g.ncols = npad <= 32 ? 32u : 64u;
   // at most 512 / ncols CTAs can hold TMEM on an SM at once: a CTA asks for enough shared
   // memory that no more become resident (they would wait inside the allocation)
-  const size_t floor_smem = ncols >= 64 ? 29 * 1024 : 0;
-  if (prec_bf16) {
-    const size_t smem = std::max((size_t)(128 + npad) * TG_ROWB, floor_smem);
-    auto k = tgemm_kernel<TA, TB, EPI, 0>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<grid, TG_NT, smem, s>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, mask, round, npad, ncols, kslice, err);
-  } else {
-    const size_t smem = std::max((size_t)2 * (128 + npad) * TG_ROWB, floor_smem);
-    auto k = tgemm_kernel<TA, TB, EPI, 1>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<grid, TG_NT, smem, s>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, mask, round, npad, ncols, kslice, err);
-  }
+  const size_t floor_smem = g.ncols >= 64 ? 29 * 1024 : 0;
+  const size_t smem = std::max((size_t)(128 + npad) * g.kc * (PREC == 0 ? 2 : 8), floor_smem);
+  cudaFuncSetAttribute(tgemm_kernel<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  tgemm_kernel<PREC><<<(unsigned)(n0 + n1), TG_NT, smem, s>>>(g);
+}
+
+// BF16 operands when the proposal trains in its BF16 form, 3xTF32 otherwise; b: a second,
+// independent product in the same launch, or null.
+static void tgemm(cudaStream_t s, bool bf16, int* err, const TgProb& a, const TgProb* b = nullptr) {
+  if (bf16)
+    tg_launch<0>(s, err, a, b);
+  else
+    tg_launch<1>(s, err, a, b);
 }
 
 // ---- the mixture head: loss and d(loss)/d(out) per row ----
@@ -220,8 +330,21 @@ struct HeadArgs {
   int n, d2, C, dout_n;
 };
 
+// *loss += the sum of v over the warp's first `live` lanes (the calling ones): one atomic a warp.
+__device__ __forceinline__ void add_loss(double* loss, double v, int live) {
+  const int lane = threadIdx.x & 31;
+  const unsigned mask = live >= 32 ? FULL : (1u << live) - 1u;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double n = __shfl_down_sync(mask, v, o);
+    if (lane + o < live) v += n;
+  }
+  if (lane == 0) atomicAdd(loss, v);
+}
+
 __global__ void head_loss_kernel(HeadArgs a) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  const int live = __popc(__ballot_sync(FULL, b < a.n));  // the warp's rows: its first lanes
   if (b >= a.n) return;
   const int C = a.C, d2 = a.d2, D = a.dout_n;
   const float* o = a.out + (long long)b * D;
@@ -251,7 +374,7 @@ __global__ void head_loss_kernel(HeadArgs a) {
   for (int c = 0; c < C; ++c) sc += expf(lc[c] - cmax);
   const float lq = cmax + logf(sc);
   const float wn = (float)((double)a.w[b] / *a.wsum);
-  atomicAdd(a.loss, -(double)wn * (double)lq);
+  add_loss(a.loss, -(double)wn * (double)lq, live);
   for (int c = 0; c < C; ++c) {
     const float gam = expf(lc[c] - lq);
     const float pi = expf(o[c] - lse_a);
@@ -283,41 +406,65 @@ struct AffineArgs {
   float half_logdet;
 };
 
-__global__ void head_affine_kernel(AffineArgs a) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= a.n) return;
-  const int d2 = a.d2;
+// One warp a row, a lane for every 32nd coordinate; Q_z^-1 is staged in shared memory (rows one
+// word longer, so that the lanes' rows fall on distinct banks). A thread a row kept its five
+// d2-long arrays in local memory and walked d2 x d2 products alone.
+constexpr int HA_WARPS = 8;
+__global__ void __launch_bounds__(32 * HA_WARPS) head_affine_kernel(AffineArgs a) {
+  __shared__ float q[kMaxD2Amortised * (kMaxD2Amortised + 1)];
+  __shared__ float rs[HA_WARPS][kMaxD2Amortised];
+  constexpr int NC = kMaxD2Amortised / 32;
+  const int d2 = a.d2, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int e = threadIdx.x; e < d2 * d2; e += blockDim.x) q[e / d2 * (d2 + 1) + e % d2] = a.qinv[e];
+  __syncthreads();
+  const int b = blockIdx.x * HA_WARPS + w;
+  if (b >= a.n) return;  // whole warps
   const float* o = a.out + (long long)b * 2 * d2;
   const float* zr = a.Z + (long long)b * 3 * d2;
   float* g = a.dout + (long long)b * 2 * d2;
-  float r[kMaxD2Amortised], u[kMaxD2Amortised], ls[kMaxD2Amortised];
-  float sum_ls = 0.f;
-  for (int d = 0; d < d2; ++d) {
-    ls[d] = fminf(fmaxf(o[d], kLogSigMin), kLogSigMax);
-    u[d] = zr[d] - zr[2 * d2 + d] - o[d2 + d];  // z - m - c
-    const float zhat = zr[2 * d2 + d] + u[d] * expf(-ls[d]);
-    r[d] = zhat - zr[d2 + d];
-    sum_ls += ls[d];
+  float u[NC], ls[NC], raw[NC], r[NC];
+  float sum_ls = 0.f, quad = 0.f;
+#pragma unroll
+  for (int p = 0; p < NC; ++p) {
+    const int d = lane + 32 * p;
+    u[p] = ls[p] = raw[p] = r[p] = 0.f;
+    if (d < d2) {
+      raw[p] = o[d];
+      ls[p] = fminf(fmaxf(raw[p], kLogSigMin), kLogSigMax);
+      u[p] = zr[d] - zr[2 * d2 + d] - o[d2 + d];  // z - m - c
+      r[p] = zr[2 * d2 + d] + u[p] * expf(-ls[p]) - zr[d2 + d];
+      rs[w][d] = r[p];
+      sum_ls += ls[p];
+    }
   }
-  float quad = 0.f;
-  float gz[kMaxD2Amortised];
-  for (int d = 0; d < d2; ++d) {
-    float v = 0.f;
-    for (int e = 0; e < d2; ++e) v += a.qinv[d * d2 + e] * r[e];
-    gz[d] = v;
-    quad += r[d] * v;
-  }
+  __syncwarp();
   const float wn = (float)((double)a.w[b] / *a.wsum);
-  atomicAdd(a.loss, (double)wn * (0.5 * (double)quad + (double)sum_ls + (double)a.half_logdet));
-  for (int d = 0; d < d2; ++d) {
-    const float is = expf(-ls[d]);
-    const bool inside = o[d] > kLogSigMin && o[d] < kLogSigMax;
-    g[d] = inside ? wn * (-gz[d] * u[d] * is + 1.f) : 0.f;
-    g[d2 + d] = -wn * gz[d] * is;
+#pragma unroll
+  for (int p = 0; p < NC; ++p) {
+    const int d = lane + 32 * p;
+    if (d < d2) {
+      float v = 0.f;
+      for (int e = 0; e < d2; ++e) v += q[d * (d2 + 1) + e] * rs[w][e];
+      quad += r[p] * v;
+      const float is = expf(-ls[p]);
+      const bool inside = raw[p] > kLogSigMin && raw[p] < kLogSigMax;
+      g[d] = inside ? wn * (-v * u[p] * is + 1.f) : 0.f;
+      g[d2 + d] = -wn * v * is;
+    }
   }
+  quad = warp_sum(quad);
+  sum_ls = warp_sum(sum_ls);
+  if (lane == 0) atomicAdd(a.loss, (double)wn * (0.5 * (double)quad + (double)sum_ls + (double)a.half_logdet));
 }
 
-__global__ void wsum_kernel(const float* w, int n, double* out) {
+// What a minibatch needs before its products: the sum of its weights (block 0, in a fixed
+// order), the gradient set to zero (split products and the bias sums add into it) and, when
+// `loss` is given, the loss too. One launch in the place of a launch and five memsets.
+__global__ void __launch_bounds__(256)
+    batch_prologue_kernel(const float* w, int n, double* wsum, float* grad, long long ngrad, double* loss) {
+  const long long e = blockIdx.x * 256ll + threadIdx.x;
+  if (grad && e < ngrad) grad[e] = 0.f;
+  if (blockIdx.x) return;
   __shared__ double sh[256];
   double s = 0.0;
   for (int b = threadIdx.x; b < n; b += 256) s += (double)w[b];
@@ -327,21 +474,10 @@ __global__ void wsum_kernel(const float* w, int n, double* out) {
     if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
     __syncthreads();
   }
-  if (threadIdx.x == 0) *out = sh[0];
-}
-
-// db[n] = sum_b d[b][n] (rows in order)
-__global__ void colsum_kernel(const float* d, int rows, int cols, float* db) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= cols) return;
-  float s = 0.f;
-  for (int b = 0; b < rows; ++b) s += d[(long long)b * cols + n];
-  db[n] = s;
-}
-
-__global__ void round_rows_kernel(const float* src, float* dst, long long n, int round) {
-  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (e < n) dst[e] = round ? round_bf16(src[e]) : src[e];
+  if (threadIdx.x == 0) {
+    *wsum = sh[0];
+    if (loss) *loss = 0.0;
+  }
 }
 
 // minibatch gather: rows perm[b] of F, Z, w
@@ -441,50 +577,49 @@ static dpf_status workspace(dpf_proposal& p, int nb) {
   return DPF_OK;
 }
 
-// Forward and backward over the nb rows already in Fb/Zb/wb: loss into *loss_dev
-// (accumulated), gradients into grad (nparams floats).
-static dpf_status fwd_bwd(dpf_proposal& p, int nb, double* loss_dev, float* grad) {
+// Forward and backward over nb rows (features F, targets Z, weights w): loss into *loss_dev
+// (accumulated, from zero when zero_loss), gradients into grad (nparams floats).
+static dpf_status fwd_bwd(dpf_proposal& p, const float* F, const float* Z, const float* w, int nb, double* loss_dev,
+                          bool zero_loss, float* grad) {
   cudaStream_t s = p.stream;
   const int H = p.hidden, din = p.din, dO = p.dout;
   const float* Wq = p.Wq;
-  const int rd = p.bf16 ? 1 : 0;
+  const bool bf = p.bf16;
+  const int rd = bf ? 1 : 0;
   const float *W1 = Wq + p.offW[0], *W2 = Wq + p.offW[1], *W3 = Wq + p.offW[2], *W4 = Wq + p.offW[3];
   const float *b1 = Wq + p.offB[0], *b2 = Wq + p.offB[1], *b3 = Wq + p.offB[2], *b4 = Wq + p.offB[3];
+  const unsigned zb = grad ? (unsigned)((p.nparams + 255) / 256) : 1u;
+  batch_prologue_kernel<<<zb, 256, 0, s>>>(w, nb, p.wsum_d, grad, p.nparams, zero_loss ? loss_dev : nullptr);
   // forward: h_l = round(relu(h_{l-1} W_l^T + b_l)), out = h3 W4^T + b4
-  tgemm<false, true, 1>(s, p.bf16 ? 1 : 0, p.err_d, nb, H, din, p.Fb, din, W1, din, p.h1, H, b1, nullptr, rd);
-  tgemm<false, true, 1>(s, p.bf16 ? 1 : 0, p.err_d, nb, H, H, p.h1, H, W2, H, p.h2, H, b2, nullptr, rd);
-  tgemm<false, true, 1>(s, p.bf16 ? 1 : 0, p.err_d, nb, H, H, p.h2, H, W3, H, p.h3, H, b3, nullptr, rd);
-  tgemm<false, true, 2>(s, p.bf16 ? 1 : 0, p.err_d, nb, dO, H, p.h3, H, W4, H, p.ob, dO, b4);
-  wsum_kernel<<<1, 256, 0, s>>>(p.wb, nb, p.wsum_d);
+  tgemm(s, bf, p.err_d, tg_prob(false, true, 1, nb, H, din, F, din, W1, din, p.h1, H, b1, nullptr, rd));
+  tgemm(s, bf, p.err_d, tg_prob(false, true, 1, nb, H, H, p.h1, H, W2, H, p.h2, H, b2, nullptr, rd));
+  tgemm(s, bf, p.err_d, tg_prob(false, true, 1, nb, H, H, p.h2, H, W3, H, p.h3, H, b3, nullptr, rd));
+  tgemm(s, bf, p.err_d, tg_prob(false, true, 2, nb, dO, H, p.h3, H, W4, H, p.ob, dO, b4));
   if (p.kind == 0) {
-    HeadArgs ha{p.ob, p.Zb, p.wb, p.wsum_d, p.dO, loss_dev, nb, p.d2, p.C, dO};
+    HeadArgs ha{p.ob, Z, w, p.wsum_d, p.dO, loss_dev, nb, p.d2, p.C, dO};
     head_loss_kernel<<<(nb + 127) / 128, 128, 0, s>>>(ha);
   } else {
     AffineArgs aa{};
-    aa.out = p.ob; aa.Z = p.Zb; aa.w = p.wb; aa.wsum = p.wsum_d; aa.dout = p.dO; aa.loss = loss_dev;
+    aa.out = p.ob; aa.Z = Z; aa.w = w; aa.wsum = p.wsum_d; aa.dout = p.dO; aa.loss = loss_dev;
     aa.n = nb; aa.d2 = p.d2;
     aa.qinv = p.qinv_d;
     aa.half_logdet = p.half_logdet;
-    head_affine_kernel<<<(nb + 127) / 128, 128, 0, s>>>(aa);
+    head_affine_kernel<<<(nb + HA_WARPS - 1) / HA_WARPS, 32 * HA_WARPS, 0, s>>>(aa);
   }
   if (!grad) return cuda_error(cudaGetLastError(), "proposal forward");
-  float *gW1 = grad + p.offW[0], *gW2 = grad + p.offW[1], *gW3 = grad + p.offW[2], *gW4 = grad + p.offW[3];
-  float *gb1 = grad + p.offB[0], *gb2 = grad + p.offB[1], *gb3 = grad + p.offB[2], *gb4 = grad + p.offB[3];
-  // layer 4: dW4 = dO^T h3, db4 = colsum dO, d3 = (dO W4) * (h3 > 0)
-  tgemm<true, false, 0>(s, p.bf16 ? 1 : 0, p.err_d, dO, H, nb, p.dO, dO, p.h3, H, gW4, H);
-  colsum_kernel<<<(dO + 127) / 128, 128, 0, s>>>(p.dO, nb, dO, gb4);
-  tgemm<false, false, 3>(s, p.bf16 ? 1 : 0, p.err_d, nb, H, dO, p.dO, dO, W4, H, p.dA, H, nullptr, p.h3);
-  // layer 3
-  tgemm<true, false, 0>(s, p.bf16 ? 1 : 0, p.err_d, H, H, nb, p.dA, H, p.h2, H, gW3, H);
-  colsum_kernel<<<(H + 127) / 128, 128, 0, s>>>(p.dA, nb, H, gb3);
-  tgemm<false, false, 3>(s, p.bf16 ? 1 : 0, p.err_d, nb, H, H, p.dA, H, W3, H, p.dB, H, nullptr, p.h2);
-  // layer 2
-  tgemm<true, false, 0>(s, p.bf16 ? 1 : 0, p.err_d, H, H, nb, p.dB, H, p.h1, H, gW2, H);
-  colsum_kernel<<<(H + 127) / 128, 128, 0, s>>>(p.dB, nb, H, gb2);
-  tgemm<false, false, 3>(s, p.bf16 ? 1 : 0, p.err_d, nb, H, H, p.dB, H, W2, H, p.dA, H, nullptr, p.h1);
-  // layer 1
-  tgemm<true, false, 0>(s, p.bf16 ? 1 : 0, p.err_d, H, din, nb, p.dA, H, p.Fb, din, gW1, din);
-  colsum_kernel<<<(H + 127) / 128, 128, 0, s>>>(p.dA, nb, H, gb1);
+  // layer l: dW_l = d_l^T h_{l-1} with db_l = colsum d_l from the same rows as they are staged,
+  // and in the same launch d_{l-1} = (d_l W_l) * (h_{l-1} > 0), which reads the same d_l
+  auto layer = [&](int l, int rows, int cols, const float* d, const float* h, const float* W, float* dprev) {
+    const TgProb gw = tg_prob(true, false, 0, rows, cols, nb, d, rows, h, cols, grad + p.offW[l], cols, nullptr,
+                              nullptr, 0, grad + p.offB[l]);
+    if (!dprev) return tgemm(s, bf, p.err_d, gw);
+    const TgProb gd = tg_prob(false, false, 3, nb, cols, rows, d, rows, W, cols, dprev, cols, nullptr, h);
+    tgemm(s, bf, p.err_d, gd, &gw);
+  };
+  layer(3, dO, H, p.dO, p.h3, W4, p.dA);
+  layer(2, H, H, p.dA, p.h2, W3, p.dB);
+  layer(1, H, H, p.dB, p.h1, W2, p.dA);
+  layer(0, H, din, p.dA, F, W1, nullptr);
   return cuda_error(cudaGetLastError(), "proposal backward");
 }
 
@@ -493,14 +628,15 @@ dpf_status proposal_forward_rows(dpf_proposal& p, const float* F, long long n, f
   if (n < 1) return DPF_OK;
   if (n > (1LL << 30)) return set_error(DPF_E_INVALID, "proposal forward: too many rows");
   const int H = p.hidden, din = p.din, dO = p.dout, m = (int)n;
-  const int pb = p.bf16 ? 1 : 0;
+  const bool bf = p.bf16;
+  const int rd = bf ? 1 : 0;
   const float* Wq = p.Wq;
   float* ha = hidden;
   float* hb = hidden + (size_t)n * H;
-  tgemm<false, true, 1>(s, pb, err, m, H, din, F, din, Wq + p.offW[0], din, ha, H, Wq + p.offB[0], nullptr, pb);
-  tgemm<false, true, 1>(s, pb, err, m, H, H, ha, H, Wq + p.offW[1], H, hb, H, Wq + p.offB[1], nullptr, pb);
-  tgemm<false, true, 1>(s, pb, err, m, H, H, hb, H, Wq + p.offW[2], H, ha, H, Wq + p.offB[2], nullptr, pb);
-  tgemm<false, true, 2>(s, pb, err, m, dO, H, ha, H, Wq + p.offW[3], H, out, dO, Wq + p.offB[3]);
+  tgemm(s, bf, err, tg_prob(false, true, 1, m, H, din, F, din, Wq + p.offW[0], din, ha, H, Wq + p.offB[0], nullptr, rd));
+  tgemm(s, bf, err, tg_prob(false, true, 1, m, H, H, ha, H, Wq + p.offW[1], H, hb, H, Wq + p.offB[1], nullptr, rd));
+  tgemm(s, bf, err, tg_prob(false, true, 1, m, H, H, hb, H, Wq + p.offW[2], H, ha, H, Wq + p.offB[2], nullptr, rd));
+  tgemm(s, bf, err, tg_prob(false, true, 2, m, dO, H, ha, H, Wq + p.offW[3], H, out, dO, Wq + p.offB[3]));
   return cuda_error(cudaGetLastError(), "proposal forward");
 }
 
@@ -568,11 +704,12 @@ static dpf_status proposal_make(int kind, int32_t d1, int32_t d2, int32_t dy, in
   const size_t bytes = sizeof(float) * (size_t)o;
   if (palloc(*p, (void**)&p->W, bytes) || palloc(*p, (void**)&p->Wq, bytes) ||
       palloc(*p, (void**)&p->am, bytes) || palloc(*p, (void**)&p->av, bytes) ||
-      palloc(*p, (void**)&p->grad, bytes) || palloc(*p, (void**)&p->loss_d, sizeof(double)) ||
-      palloc(*p, (void**)&p->wsum_d, sizeof(double)) || palloc(*p, (void**)&p->err_d, sizeof(int))) {
+      palloc(*p, (void**)&p->grad, bytes) || palloc(*p, (void**)&p->loss_d, 2 * sizeof(double)) ||
+      palloc(*p, (void**)&p->wsum_d, sizeof(double))) {
     dpf_proposal_destroy(p);
     return DPF_E_NOMEM;
   }
+  p->err_d = (int*)(p->loss_d + 1);  // after the loss: one copy reads both
   cudaMemsetAsync(p->err_d, 0, sizeof(int), p->stream);
   cudaMemsetAsync(p->W, 0, bytes, p->stream);
   cudaMemsetAsync(p->Wq, 0, bytes, p->stream);
@@ -723,20 +860,18 @@ dpf_status dpf_proposal_loss_grad(dpf_proposal* p, const float* F, const float* 
   dpf_status st = workspace(*p, (int)n);
   if (st) return st;
   cudaStream_t s = p->stream;
-  const int rd = p->bf16 ? 1 : 0;
-  round_rows_kernel<<<(unsigned)((n * p->din + 255) / 256), 256, 0, s>>>(F, p->Fb, n * p->din, rd);
-  cudaMemcpyAsync(p->Zb, Z, sizeof(float) * n * p->zw, cudaMemcpyDeviceToDevice, s);
-  cudaMemcpyAsync(p->wb, w, sizeof(float) * n, cudaMemcpyDeviceToDevice, s);
-  cudaMemsetAsync(p->loss_d, 0, sizeof(double), s);
-  st = fwd_bwd(*p, (int)n, p->loss_d, grad_dev);
+  // the caller's rows are read where they lie (the products round them as they stage them)
+  st = fwd_bwd(*p, F, Z, w, (int)n, p->loss_d, true, grad_dev);
   if (st) return st;
-  double h = 0.0;
-  cudaError_t e = cudaMemcpyAsync(&h, p->loss_d, sizeof(double), cudaMemcpyDeviceToHost, s);
+  struct {
+    double loss;
+    int err;
+  } h = {0.0, 0};
+  cudaError_t e = cudaMemcpyAsync(&h, p->loss_d, sizeof(double) + sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_error(e, "dpf_proposal_loss_grad");
-  st = training_err(*p, "dpf_proposal_loss_grad");
-  if (st) return st;
-  if (loss) *loss = h;
+  if (h.err) return training_err(*p, "dpf_proposal_loss_grad");
+  if (loss) *loss = h.loss;
   return DPF_OK;
 }
 
@@ -788,7 +923,7 @@ dpf_status dpf_proposal_train(dpf_proposal* p, const float* F, const float* Z, c
       const int64_t b0 = bi * nb_max;
       const int nb = (int)std::min<int64_t>(nb_max, n - b0);
       gather_rows_kernel<<<nb, 32, 0, s>>>(F, Z, w, perm_dev + b0, nb, p->din, p->zw, p->Fb, p->Zb, p->wb, rd);
-      st = fwd_bwd(*p, nb, eloss_d + ep, p->grad);
+      st = fwd_bwd(*p, p->Fb, p->Zb, p->wb, nb, eloss_d + ep, false, p->grad);
       if (!st) st = adam(*p, p->grad, lr);
     }
   }
