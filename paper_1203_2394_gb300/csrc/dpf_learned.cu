@@ -32,7 +32,7 @@ namespace dpf {
 __device__ __forceinline__ float round_bf16(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
 
 // On the tensor cores (tcgen05):
-// One CTA of 256 threads per 128-row x npad-column tile of C (npad <= 64 columns of a
+// One CTA of 512 threads per 128-row x npad-column tile of C (npad <= 64 columns of a
 // TMEM accumulator in FP32) and one slice of K (the slices of a long K add their partial
 // products into C, which the caller has zeroed: the plain-store epilogue only). The
 // threads load op(A) and op(B)^T of a chunk of K from global memory, round them to the
@@ -51,7 +51,7 @@ __device__ __forceinline__ float round_bf16(float v) { return __bfloat162float(_
 // matrices of consecutive rows take without bank conflicts; four units are in flight at once,
 // and a chunk is as long as shared memory holds twice on an SM (256 BF16 or 64 TF32 values of
 // K), so that a forward product is one round of loads, one of MMAs and one epilogue.
-constexpr int TG_NT = 256;
+constexpr int TG_NT = 512;
 constexpr int TG_SPIN = 1 << 22;
 constexpr int TG_UNITS = 4;  // staging units a thread holds in flight
 
@@ -73,6 +73,29 @@ struct TgProb {
   int npad, mt, nt, ks, kslice;  // column tile, tiles, slices of K
   int va, vb, vc;                // rows of A, B, C start on 16 bytes
 };
+// Programmatic dependent launch, along the chain of small kernels of one minibatch: a kernel
+// lets the next one start (its launch, its TMEM allocation and barrier set-up) as soon as every
+// CTA of its own is running, and takes the previous one's results only after that one has
+// completed. Without the launch attribute both are no-ops.
+__device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... KA, class... A>
+static void launch_after(cudaStream_t s, bool overlap, unsigned grid, unsigned block, size_t smem,
+                         void (*k)(KA...), A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, k, KA(args)...);
+}
+
 // Up to two independent products in one launch: CTAs below `first` serve p[0].
 struct TgLaunch {
   TgProb p[2];
@@ -177,6 +200,8 @@ __global__ void __launch_bounds__(TG_NT, 2) tgemm_kernel(const __grid_constant__
   __syncthreads();
   tc::fence_after();
   const uint32_t taddr = s_taddr;
+  grid_launch_next();
+  grid_wait_previous();
   const uint32_t idesc = tc::instr_desc(PREC == 0 ? tc::FMT_BF16 : tc::FMT_TF32, 128, npad);
   int ok = 1;
   uint32_t phase = 0;
@@ -214,10 +239,10 @@ __global__ void __launch_bounds__(TG_NT, 2) tgemm_kernel(const __grid_constant__
     tc::bar_wait(&bar, phase ^ 1u, TG_SPIN);  // give MMAs still in flight a second bound
   } else {
     if (p.asum && tn == 0 && m0 + tid % 128 < p.M) atomicAdd(p.asum + m0 + tid % 128, asum);
-    // warp w holds rows 32 (w mod 4) .. + 31, 16 columns at a time, every other block of 16
+    // warp w takes rows 32 (w mod 4) .. + 31 and the w / 4-th block of 16 columns
     const long long m = m0 + tid % 128;
     const bool split = p.ks > 1;
-    for (int c0 = 16 * (w >> 2); c0 < npad; c0 += 32) {
+    for (int c0 = 16 * (w >> 2); c0 < npad; c0 += TG_NT / 8) {
       float v[16];
       tc::ld16(taddr + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)c0, v);
       if (m >= p.M) continue;
@@ -290,7 +315,7 @@ static TgProb tg_prob(bool ta, bool tb, int epi, int M, int N, int K, const floa
 }
 
 template <int PREC>
-static void tg_launch(cudaStream_t s, int* err, const TgProb& a, const TgProb* b) {
+static void tg_launch(cudaStream_t s, bool overlap, int* err, const TgProb& a, const TgProb* b) {
   TgLaunch g{};
   g.p[0] = a;
   g.p[1] = b ? *b : a;
@@ -307,16 +332,17 @@ static void tg_launch(cudaStream_t s, int* err, const TgProb& a, const TgProb* b
   const size_t floor_smem = g.ncols >= 64 ? 29 * 1024 : 0;
   const size_t smem = std::max((size_t)(128 + npad) * g.kc * (PREC == 0 ? 2 : 8), floor_smem);
   cudaFuncSetAttribute(tgemm_kernel<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  tgemm_kernel<PREC><<<(unsigned)(n0 + n1), TG_NT, smem, s>>>(g);
+  launch_after(s, overlap, (unsigned)(n0 + n1), TG_NT, smem, tgemm_kernel<PREC>, g);
 }
 
 // BF16 operands when the proposal trains in its BF16 form, 3xTF32 otherwise; b: a second,
-// independent product in the same launch, or null.
-static void tgemm(cudaStream_t s, bool bf16, int* err, const TgProb& a, const TgProb* b = nullptr) {
+// independent product in the same launch, or null. overlap: the launch before it on the stream
+// is a kernel of the same chain.
+static void tgemm(cudaStream_t s, bool bf16, bool overlap, int* err, const TgProb& a, const TgProb* b = nullptr) {
   if (bf16)
-    tg_launch<0>(s, err, a, b);
+    tg_launch<0>(s, overlap, err, a, b);
   else
-    tg_launch<1>(s, err, a, b);
+    tg_launch<1>(s, overlap, err, a, b);
 }
 
 // ---- the mixture head: loss and d(loss)/d(out) per row ----
@@ -343,6 +369,8 @@ __device__ __forceinline__ void add_loss(double* loss, double v, int live) {
 }
 
 __global__ void head_loss_kernel(HeadArgs a) {
+  grid_launch_next();
+  grid_wait_previous();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   const int live = __popc(__ballot_sync(FULL, b < a.n));  // the warp's rows: its first lanes
   if (b >= a.n) return;
@@ -415,7 +443,9 @@ __global__ void __launch_bounds__(32 * HA_WARPS) head_affine_kernel(AffineArgs a
   __shared__ float rs[HA_WARPS][kMaxD2Amortised];
   constexpr int NC = kMaxD2Amortised / 32;
   const int d2 = a.d2, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  grid_launch_next();
   for (int e = threadIdx.x; e < d2 * d2; e += blockDim.x) q[e / d2 * (d2 + 1) + e % d2] = a.qinv[e];
+  grid_wait_previous();
   __syncthreads();
   const int b = blockIdx.x * HA_WARPS + w;
   if (b >= a.n) return;  // whole warps
@@ -462,6 +492,7 @@ __global__ void __launch_bounds__(32 * HA_WARPS) head_affine_kernel(AffineArgs a
 // `loss` is given, the loss too. One launch in the place of a launch and five memsets.
 __global__ void __launch_bounds__(256)
     batch_prologue_kernel(const float* w, int n, double* wsum, float* grad, long long ngrad, double* loss) {
+  grid_launch_next();
   const long long e = blockIdx.x * 256ll + threadIdx.x;
   if (grad && e < ngrad) grad[e] = 0.f;
   if (blockIdx.x) return;
@@ -591,20 +622,20 @@ static dpf_status fwd_bwd(dpf_proposal& p, const float* F, const float* Z, const
   const unsigned zb = grad ? (unsigned)((p.nparams + 255) / 256) : 1u;
   batch_prologue_kernel<<<zb, 256, 0, s>>>(w, nb, p.wsum_d, grad, p.nparams, zero_loss ? loss_dev : nullptr);
   // forward: h_l = round(relu(h_{l-1} W_l^T + b_l)), out = h3 W4^T + b4
-  tgemm(s, bf, p.err_d, tg_prob(false, true, 1, nb, H, din, F, din, W1, din, p.h1, H, b1, nullptr, rd));
-  tgemm(s, bf, p.err_d, tg_prob(false, true, 1, nb, H, H, p.h1, H, W2, H, p.h2, H, b2, nullptr, rd));
-  tgemm(s, bf, p.err_d, tg_prob(false, true, 1, nb, H, H, p.h2, H, W3, H, p.h3, H, b3, nullptr, rd));
-  tgemm(s, bf, p.err_d, tg_prob(false, true, 2, nb, dO, H, p.h3, H, W4, H, p.ob, dO, b4));
+  tgemm(s, bf, true, p.err_d, tg_prob(false, true, 1, nb, H, din, F, din, W1, din, p.h1, H, b1, nullptr, rd));
+  tgemm(s, bf, true, p.err_d, tg_prob(false, true, 1, nb, H, H, p.h1, H, W2, H, p.h2, H, b2, nullptr, rd));
+  tgemm(s, bf, true, p.err_d, tg_prob(false, true, 1, nb, H, H, p.h2, H, W3, H, p.h3, H, b3, nullptr, rd));
+  tgemm(s, bf, true, p.err_d, tg_prob(false, true, 2, nb, dO, H, p.h3, H, W4, H, p.ob, dO, b4));
   if (p.kind == 0) {
     HeadArgs ha{p.ob, Z, w, p.wsum_d, p.dO, loss_dev, nb, p.d2, p.C, dO};
-    head_loss_kernel<<<(nb + 127) / 128, 128, 0, s>>>(ha);
+    launch_after(s, true, (nb + 127) / 128, 128, 0, head_loss_kernel, ha);
   } else {
     AffineArgs aa{};
     aa.out = p.ob; aa.Z = Z; aa.w = w; aa.wsum = p.wsum_d; aa.dout = p.dO; aa.loss = loss_dev;
     aa.n = nb; aa.d2 = p.d2;
     aa.qinv = p.qinv_d;
     aa.half_logdet = p.half_logdet;
-    head_affine_kernel<<<(nb + HA_WARPS - 1) / HA_WARPS, 32 * HA_WARPS, 0, s>>>(aa);
+    launch_after(s, true, (nb + HA_WARPS - 1) / HA_WARPS, 32 * HA_WARPS, 0, head_affine_kernel, aa);
   }
   if (!grad) return cuda_error(cudaGetLastError(), "proposal forward");
   // layer l: dW_l = d_l^T h_{l-1} with db_l = colsum d_l from the same rows as they are staged,
@@ -612,9 +643,9 @@ static dpf_status fwd_bwd(dpf_proposal& p, const float* F, const float* Z, const
   auto layer = [&](int l, int rows, int cols, const float* d, const float* h, const float* W, float* dprev) {
     const TgProb gw = tg_prob(true, false, 0, rows, cols, nb, d, rows, h, cols, grad + p.offW[l], cols, nullptr,
                               nullptr, 0, grad + p.offB[l]);
-    if (!dprev) return tgemm(s, bf, p.err_d, gw);
+    if (!dprev) return tgemm(s, bf, true, p.err_d, gw);
     const TgProb gd = tg_prob(false, false, 3, nb, cols, rows, d, rows, W, cols, dprev, cols, nullptr, h);
-    tgemm(s, bf, p.err_d, gd, &gw);
+    tgemm(s, bf, true, p.err_d, gd, &gw);
   };
   layer(3, dO, H, p.dO, p.h3, W4, p.dA);
   layer(2, H, H, p.dA, p.h2, W3, p.dB);
@@ -633,10 +664,10 @@ dpf_status proposal_forward_rows(dpf_proposal& p, const float* F, long long n, f
   const float* Wq = p.Wq;
   float* ha = hidden;
   float* hb = hidden + (size_t)n * H;
-  tgemm(s, bf, err, tg_prob(false, true, 1, m, H, din, F, din, Wq + p.offW[0], din, ha, H, Wq + p.offB[0], nullptr, rd));
-  tgemm(s, bf, err, tg_prob(false, true, 1, m, H, H, ha, H, Wq + p.offW[1], H, hb, H, Wq + p.offB[1], nullptr, rd));
-  tgemm(s, bf, err, tg_prob(false, true, 1, m, H, H, hb, H, Wq + p.offW[2], H, ha, H, Wq + p.offB[2], nullptr, rd));
-  tgemm(s, bf, err, tg_prob(false, true, 2, m, dO, H, ha, H, Wq + p.offW[3], H, out, dO, Wq + p.offB[3]));
+  tgemm(s, bf, false, err, tg_prob(false, true, 1, m, H, din, F, din, Wq + p.offW[0], din, ha, H, Wq + p.offB[0], nullptr, rd));
+  tgemm(s, bf, true, err, tg_prob(false, true, 1, m, H, H, ha, H, Wq + p.offW[1], H, hb, H, Wq + p.offB[1], nullptr, rd));
+  tgemm(s, bf, true, err, tg_prob(false, true, 1, m, H, H, hb, H, Wq + p.offW[2], H, ha, H, Wq + p.offB[2], nullptr, rd));
+  tgemm(s, bf, true, err, tg_prob(false, true, 2, m, dO, H, ha, H, Wq + p.offW[3], H, out, dO, Wq + p.offB[3]));
   return cuda_error(cudaGetLastError(), "proposal forward");
 }
 
