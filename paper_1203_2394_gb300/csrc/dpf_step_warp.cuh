@@ -312,6 +312,20 @@ __device__ __forceinline__ void reduce_rows(const T* part, int L, int lane, T* o
   }
 }
 
+// The sum of a row's 32 lane partials, lane 0's first (vector loads, one chain of adds).
+template <typename T>
+__device__ __forceinline__ T lane_sum_in_order(const T* part) {
+  T r = T(0);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    T x[16];
+    vld<T, 16>(part + 16 * h, x);
+#pragma unroll
+    for (int l = 0; l < 16; ++l) r += x[l];
+  }
+  return r;
+}
+
 // Issue the bulk copies of one group's source rows into a warp's stage (lane 0).
 template <typename T, int D1, int D2>
 __device__ __forceinline__ void warp_stage(const StepArgs<T>& a, unsigned char* st, uint64_t* bar,
@@ -447,7 +461,7 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
         T mx = NEG;
 #pragma unroll
         for (int p = 0; p < PPL; ++p) mx = fmax(mx, lqr[p]);
-        sigma = warp_max(mx);
+        sigma = warp_max_redux(mx);
         T se = T(0);
 #pragma unroll
         for (int p = 0; p < PPL; ++p) se += act ? exp2_t((lqr[p] - sigma) * LOG2E) : T(0);
@@ -465,7 +479,7 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
         const bool two = L > 32;
         const T l0 = lane < L ? slwh[lane] : NEG;
         const T l1 = two && lane + 32 < L ? slwh[lane + 32] : NEG;
-        const T mx = warp_max(fmax(l0, l1));
+        const T mx = warp_max_redux(fmax(l0, l1));
         const uint32_t c0 = lane < L ? (uint32_t)floor(exp2_t((l0 - mx) * LOG2E) * a.scaleL) : 0u;
         uint32_t s0 = c0, s1 = 0u;
 #pragma unroll
@@ -540,7 +554,7 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
       T amax = NEG;
 #pragma unroll
       for (int p = 0; p < PPL; ++p) amax = fmax(amax, alpha[p]);
-      amax = warp_max(amax);
+      amax = warp_max_redux(amax);
       // ancestors of the lane's destinations by offspring ranges (sys_local_offspring)
       int bidx[PPL];
       {
@@ -648,7 +662,7 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
         ell[p] = act ? T(-0.5) * ell[p] : NEG;
         lmax = fmax(lmax, ell[p]);
       }
-      lmax = warp_max(lmax);
+      lmax = warp_max_redux(lmax);
       T ls = T(0);
 #pragma unroll
       for (int p = 0; p < PPL; ++p) ls += act ? exp2_t((ell[p] - lmax) * LOG2E) : T(0);
@@ -825,7 +839,7 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
     T B[PPL];  // beta_k up to normalisation
 #pragma unroll
     for (int p = 0; p < PPL; ++p) B[p] = T(0);
-    bool general = XZ;
+    bool general = false;  // a row underflowed: take the robust path
     if (!XZ) {
       // one pass: e(m,k) = 2^(a_k - |c'_m - g'_k|^2), S_m = sum_k e, B_k = sum_m e
 #pragma unroll 4
@@ -877,6 +891,132 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
       for (int m = lane; m < L; m += 32) bad |= rowS[m] < tiny;
       general = __any_sync(FULL, bad);
     }
+    if (XZ) {
+      // The x transition depends on z. v = alpha's exponent, vl = v less the y terms (log2
+      // units); A_m and S_m are their row sums over k. Since pi_m / S_m is proportional to
+      // 1 / A_m, beta_k = sum_m w_m e(m,k) up to normalisation, with w_m known once the A rows
+      // are summed, so the pass that sums the S rows gives beta too.
+      const T tiny = sizeof(T) == 4 ? T(1e-30) : T(1e-290);
+      // the rows of exponents: v alone, or vl
+      auto expo = [&](int m, bool with_y, T (&v)[PPL]) {
+#pragma unroll
+        for (int p = 0; p < PPL; ++p) v[p] = ak[p];
+#pragma unroll
+        for (int c = 0; c < D1; ++c) sub_sq<T, PPL>(xw[m * D1 + c], nfk[c], v);
+        if (with_y) {
+#pragma unroll
+          for (int q = 0; q < DY; ++q) sub_sq<T, PPL>(cw[m * DY + q], ngk[q], v);
+        }
+      };
+      // FP64 first tries without shifts (both exponents are at most 0), like the pass above: two
+      // exponentials a pair in the place of three, on a pipe that gives one FP64 result for 64
+      // FP32 ones. A row that underflows, and FP32 always, take the sums relative to the row
+      // maxima (in FP32 the unshifted sums round differently, and one last-bit change of a
+      // look-ahead weight can move a resampling decision and with it the whole run)
+      bool shifted = sizeof(T) == 4;
+      if (!shifted) {
+        bool bad = false;
+        for (int m = 0; m < L; ++m) {
+          T v[PPL];
+          expo(m, false, v);
+          T pa = T(0);
+#pragma unroll
+          for (int p = 0; p < PPL; ++p) pa += act ? exp2_t(v[p]) : T(0);
+          part[m * PART_STRIDE + lane] = pa;
+        }
+        __syncwarp();
+        reduce_rows<T, false>(part, L, lane, rowA);
+        __syncwarp();
+        for (int m = lane; m < L; m += 32) {
+          bad |= rowA[m] < tiny;
+          coef[m] = T(1) / rowA[m];
+          shS[m] = T(0);
+          shA[m] = T(0);
+        }
+        __syncwarp();
+        for (int m = 0; m < L; ++m) {
+          T v[PPL];
+          expo(m, true, v);
+          T ps = T(0);
+#pragma unroll
+          for (int p = 0; p < PPL; ++p) {
+            const T e = act ? exp2_t(v[p]) : T(0);
+            ps += e;
+            B[p] = fma(coef[m], e, B[p]);
+          }
+          part[m * PART_STRIDE + lane] = ps;
+        }
+        __syncwarp();
+        reduce_rows<T, false>(part, L, lane, rowS);
+        __syncwarp();
+        for (int m = lane; m < L; m += 32) bad |= rowS[m] < tiny;
+        shifted = __any_sync(FULL, bad);
+      }
+      if (shifted) {
+        // row maxima of both exponents
+#pragma unroll 2
+        for (int m = 0; m < L; ++m) {
+          T v[PPL];
+          T pa = NEG, ps = NEG;
+          expo(m, false, v);
+#pragma unroll
+          for (int p = 0; p < PPL; ++p) pa = fmax(pa, v[p]);
+#pragma unroll
+          for (int q = 0; q < DY; ++q) sub_sq<T, PPL>(cw[m * DY + q], ngk[q], v);
+#pragma unroll
+          for (int p = 0; p < PPL; ++p) ps = fmax(ps, v[p]);
+          part[m * PART_STRIDE + lane] = act ? pa : NEG;
+          part[(L + m) * PART_STRIDE + lane] = act ? ps : NEG;
+        }
+        __syncwarp();
+        reduce_rows<T, true>(part, L, lane, shA);
+        reduce_rows<T, true>(part + L * PART_STRIDE, L, lane, shS);
+        __syncwarp();
+        // A_m relative to its maximum, added lane after lane
+#pragma unroll 2
+        for (int m = 0; m < L; ++m) {
+          const T ha = shA[m];
+          T v[PPL], pa = T(0);
+          expo(m, false, v);
+          if (act) {
+#pragma unroll
+            for (int p = 0; p < PPL; ++p) pa += exp2_t(v[p] - ha);
+          }
+          part[m * PART_STRIDE + lane] = pa;
+        }
+        __syncwarp();
+        T wmax = NEG;
+        for (int m = lane; m < L; m += 32) {
+          const T r = lane_sum_in_order<T>(part + m * PART_STRIDE);
+          rowA[m] = r;
+          coef[m] = shS[m] - shA[m] - log2_fast(r);
+          wmax = fmax(wmax, coef[m]);
+        }
+        wmax = warp_max_redux(wmax);
+        for (int m = lane; m < L; m += 32) coef[m] = exp2_t(coef[m] - wmax);
+        __syncwarp();
+#pragma unroll
+        for (int p = 0; p < PPL; ++p) B[p] = T(0);
+        // S_m relative to its maximum, and beta
+#pragma unroll 2
+        for (int m = 0; m < L; ++m) {
+          const T hs = shS[m];
+          T v[PPL], ps = T(0);
+          expo(m, true, v);
+#pragma unroll
+          for (int p = 0; p < PPL; ++p) v[p] = exp2_t(v[p] - hs);
+          axpy<T, PPL>(coef[m], v, B);
+          if (act) {
+#pragma unroll
+            for (int p = 0; p < PPL; ++p) ps += v[p];
+          }
+          part[m * PART_STRIDE + lane] = ps;
+        }
+        __syncwarp();
+        for (int m = lane; m < L; m += 32) rowS[m] = lane_sum_in_order<T>(part + m * PART_STRIDE);
+        __syncwarp();
+      }
+    }
     T gmax = T(0);  // the largest row maximum (robust path without x-z coupling; else 0)
     if (general && !XZ) {
       // robust path of a model whose x transition does not depend on z (a row
@@ -918,68 +1058,12 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
           __syncwarp();
           T g = NEG;
           for (int m = lane; m < L; m += 32) g = fmax(g, shS[m]);
-          gmax = warp_max(g);
+          gmax = warp_max_redux(g);
         } else {
           reduce_rows<T, false>(part, L, lane, rowS);
           for (int m = lane; m < L; m += 32) {
             rowA[m] = SA0;
             shA[m] = T(0);
-          }
-        }
-        __syncwarp();
-      }
-    } else if (general) {
-      // robust path (x transition depends on z): row maxima, row sums relative to them,
-      // then beta with the coefficients pi_m / S_m
-      for (int pass = 0; pass < 2; ++pass) {
-        for (int m = 0; m < L; ++m) {
-          const T ha = pass ? shA[m] : T(0), hs = pass ? shS[m] : T(0);
-          T v[PPL];
-#pragma unroll
-          for (int p = 0; p < PPL; ++p) v[p] = ak[p];
-          if (XZ) {
-#pragma unroll
-            for (int c = 0; c < D1; ++c) sub_sq<T, PPL>(xw[m * D1 + c], nfk[c], v);
-          }
-          T vl[PPL];
-#pragma unroll
-          for (int p = 0; p < PPL; ++p) vl[p] = v[p];
-#pragma unroll
-          for (int q = 0; q < DY; ++q) sub_sq<T, PPL>(cw[m * DY + q], ngk[q], vl);
-          T pa = pass ? T(0) : NEG, ps = pass ? T(0) : NEG;
-          if (act) {
-#pragma unroll
-            for (int p = 0; p < PPL; ++p) {
-              if (pass == 0) {
-                pa = fmax(pa, v[p]);
-                ps = fmax(ps, vl[p]);
-              } else {
-                pa += exp2_t(v[p] - ha);
-                ps += exp2_t(vl[p] - hs);
-              }
-            }
-          }
-          part[m * PART_STRIDE + lane] = pa;
-          part[(L + m) * PART_STRIDE + lane] = ps;
-        }
-        __syncwarp();
-        for (int m = lane; m < L; m += 32) {
-          T ra = pass ? T(0) : NEG, rs = pass ? T(0) : NEG;
-          for (int l = 0; l < 32; ++l) {
-            if (pass == 0) {
-              ra = fmax(ra, part[m * PART_STRIDE + l]);
-              rs = fmax(rs, part[(L + m) * PART_STRIDE + l]);
-            } else {
-              ra += part[m * PART_STRIDE + l];
-              rs += part[(L + m) * PART_STRIDE + l];
-            }
-          }
-          if (pass == 0) {
-            shA[m] = ra;
-            shS[m] = rs;
-          } else {
-            rowA[m] = ra;
-            rowS[m] = rs;
           }
         }
         __syncwarp();
@@ -998,7 +1082,7 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
                                   (log2_fast(rowA[lane + 32]) + shA[lane + 32]));
       a.lwh_new[i * L + lane + 32] = lw1;
     }
-    const T mx = warp_max(two ? fmax(lw0, lw1) : lw0);
+    const T mx = warp_max_redux(two ? fmax(lw0, lw1) : lw0);
     const T p0 = lane < L ? exp2_t((lw0 - mx) * LOG2E) : T(0);
     const T p1 = two && lane + 32 < L ? exp2_t((lw1 - mx) * LOG2E) : T(0);
     const T psum = warp_sum(p0 + p1);
@@ -1019,36 +1103,15 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
         atomicMax(a.lwmax_key, key);
     }
     // ---- z part of the filtered mean: beta_k = sum_m pi_m e(m,k) / S_m ----
-    if (general && XZ) {
+    // normalise sum_m w_m e(m,k) by sum_(m,k) w_m e(m,k); without x-z coupling w_m = 1, and both
+    // sums are relative to the largest row (gmax = 0 and every shS = 0 on the fast path)
+    T tot = T(0);
+    for (int m = lane; m < L; m += 32)
+      tot += general ? rowS[m] * exp2_t(shS[m] - gmax) : (XZ ? rowS[m] * coef[m] : rowS[m]);
+    tot = warp_sum(tot);
+    const T inv = T(1) / tot;
 #pragma unroll
-      for (int p = 0; p < PPL; ++p) B[p] = T(0);
-      if (lane < L) coef[lane] = p0 / psum / rowS[lane];
-      if (lane + 32 < L) coef[lane + 32] = p1 / psum / rowS[lane + 32];
-      __syncwarp();
-      for (int m = 0; m < L; ++m) {
-        const T cf = coef[m], hs = shS[m];
-        T v[PPL];
-#pragma unroll
-        for (int p = 0; p < PPL; ++p) v[p] = ak[p];
-        if (XZ) {
-#pragma unroll
-          for (int c = 0; c < D1; ++c) sub_sq<T, PPL>(xw[m * D1 + c], nfk[c], v);
-        }
-#pragma unroll
-        for (int q = 0; q < DY; ++q) sub_sq<T, PPL>(cw[m * DY + q], ngk[q], v);
-#pragma unroll
-        for (int p = 0; p < PPL; ++p) B[p] += act ? cf * exp2_t(v[p] - hs) : T(0);
-      }
-    } else {
-      // normalise sum_m e(m,k) by sum_(m,k) e(m,k), both relative to the largest row
-      // (gmax = 0 and every shS = 0 on the fast path)
-      T tot = T(0);
-      for (int m = lane; m < L; m += 32) tot += general ? rowS[m] * exp2_t(shS[m] - gmax) : rowS[m];
-      tot = warp_sum(tot);
-      const T inv = T(1) / tot;
-#pragma unroll
-      for (int p = 0; p < PPL; ++p) B[p] *= inv;
-    }
+    for (int p = 0; p < PPL; ++p) B[p] *= inv;
     T acc[D2 + DY];
 #pragma unroll
     for (int c = 0; c < D2; ++c) {
@@ -1096,8 +1159,9 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, warp_min_blocks<PPL, D2>()
   }
   __syncwarp();
   uint32_t phase = 0;
-  warp_run<T, D1, D2, DY, XZ, PPL, MF>(mc, a, (long long)blockIdx.x * WARPS_PER_CTA + wib, a.N,
-                                   (long long)gridDim.x * WARPS_PER_CTA,
+  const int nw = blockDim.x >> 5;  // warps of this CTA (WARPS_PER_CTA, or 1 for a few groups)
+  warp_run<T, D1, D2, DY, XZ, PPL, MF>(mc, a, (long long)blockIdx.x * nw + wib, a.N,
+                                   (long long)gridDim.x * nw,
                                    smem_raw + (size_t)wib * a.stage_bytes, &bars[wib], phase);
 }
 

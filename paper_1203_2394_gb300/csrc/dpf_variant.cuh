@@ -11,6 +11,8 @@
 
 namespace dpf {
 
+constexpr int FEW_GROUPS = 16 * 152;  // one-warp CTAs: 16 fit on an SM at 128 registers a thread
+
 inline int threads_for(int M) { return ((M + 31) / 32) * 32; }
 
 // The outer stage of a step (the outer reduction and the global resampling, in one
@@ -163,6 +165,15 @@ struct VariantImpl {
       attr_done = true;
     }
     const size_t sm = warp_geometry<T, D1, D2, DY, XZ>(x.M, x.L, &a, a.first != 0);
+    // Few groups: a CTA of one warp each, so that they spread over every SM. (Four to a CTA left
+    // the 256 groups of a small filter on 64 of the 152 SMs, four warps sharing each one's FP64
+    // pipe. lg4 in FP64 at N = 256, M = 32, L = 8: 90.8 us a step, 74.5 with the spread and the
+    // two-pass look-ahead.) Above FEW_GROUPS four-warp CTAs fill every
+    // SM anyway.
+    if (x.N <= FEW_GROUPS) {
+      k<<<(unsigned)x.N, 32, sm / WARPS_PER_CTA, stream ? stream : x.stream>>>(cst(x), a);
+      return cuda_error(cudaGetLastError(), "step kernel launch");
+    }
     if (x.grid_step == 0 || x.grid_kernel != (const void*)k) {
       // persistent grid: as many CTAs of this kernel as fit on the device at once
       int nb = 0, dev = 0, nsm = 0;
