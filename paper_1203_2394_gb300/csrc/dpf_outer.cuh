@@ -50,39 +50,15 @@ struct FusedOuterArgs {
   double* host_stats;           // a pinned host mirror of stats[0 .. 4 + d) and the error word, or null
 };
 
-template <typename T>
-__device__ __forceinline__ T pow2_t(int e);
-template <>
-__device__ __forceinline__ float pow2_t<float>(int e) { return __int_as_float((127 + e) << 23); }
-template <>
-__device__ __forceinline__ double pow2_t<double>(int e) {
-  return __longlong_as_double((long long)(1023 + e) << 52);
-}
-
-// K(c) = #{ k in [0, n) : (k 2^32 + u) C < c n 2^32 }, the number of systematic
-// points below the cumulative count c (the quantity points_below computes). The
-// condition falls as k grows, so K is the first k where it fails: an estimate
-// c n / C - u 2^-32 (single precision up to n = 2^24, whose error is a few units;
-// double beyond) is settled by exact 128-bit comparisons.
-__device__ __forceinline__ int points_below_est(unsigned long long c, long long n, uint32_t u,
-                                                unsigned long long C) {
-  if (c == 0) return 0;
-  const u128 X = ((u128)c * (u128)(unsigned long long)n) << 32;
-  long long k;
-  if (n <= (1ll << 24)) {
-    const float e = __fdividef((float)c, (float)C) * (float)n - (float)u * 0x1p-32f;
-    k = e > 0.f ? (long long)ceilf(e) : 0;
-  } else {
-    const double e = (double)c / (double)C * (double)n - (double)u * 0x1p-32;
-    k = e > 0.0 ? (long long)ceil(e) : 0;
-  }
-  if (k > n) k = n;
-  while (k > 0 && !((u128)((unsigned long long)(k - 1) << 32 | u) * C < X)) --k;
-  while (k < n && (u128)((unsigned long long)k << 32 | u) * C < X) ++k;
-  return (int)k;
-}
-
 // ---- A: the partial sums and the count total of CTA `bid` of the `nb` CTAs of one filter ----
+// Whether the sums that came with the step serve (OuterArgs::npre): with the largest weight at
+// least e^-20 of the reference its square is 4e-18, so single precision holds W'^2 and every
+// weight of consequence beside it.
+template <typename T>
+__device__ __forceinline__ bool sums_given(const OuterArgs<T>& o, T lwmax) {
+  return o.npre > 0 && lwmax >= o.lref - T(20) && lwmax <= o.lref + T(20);
+}
+
 template <typename T, int D1, int D2>
 __device__ __forceinline__ void outer_sums(const FusedOuterArgs<T>& a, int bid, int nb, T lwmax) {
   constexpr int NV = 2 + D1 + D2, NW = OF_NT / 32;

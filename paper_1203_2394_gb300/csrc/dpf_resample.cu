@@ -10,31 +10,35 @@
 
 namespace dpf {
 
+constexpr int WQ = 8;  // weights a thread loads at once
+
 // Largest weight as an order-preserving 64-bit key (weights are >= 0, so the
 // IEEE bit pattern orders like the value); flags negative, NaN and inf.
 template <typename T>
-__global__ void wmax_kernel(const T* w, long long n, unsigned long long* maxkey, int* err) {
-  unsigned long long best = 0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    const T W = w[i];
-    if (!(W >= T(0)) || isinf(W)) atomicOr(err, ERR_NUMERIC);
-    const unsigned long long k = sizeof(T) == 8 ? (unsigned long long)__double_as_longlong((double)W)
-                                                : (unsigned long long)__float_as_uint((float)W);
-    best = k > best ? k : best;
-  }
+__global__ void __launch_bounds__(256) wmax_kernel(const T* w, long long n, unsigned long long* maxkey, int* err) {
+  const bool vec = ((uintptr_t)w & 15) == 0;
+  T best = T(0);
+  bool bad = false;
+  for (long long i = (blockIdx.x * 256ll + threadIdx.x) * WQ; i < n; i += (long long)gridDim.x * 256 * WQ) {
+    T W[WQ];
+    load_weights<T, WQ>(w, i, n, vec, W);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long v = __shfl_xor_sync(FULL, best, o);
-    best = v > best ? v : best;
+    for (int q = 0; q < WQ; ++q) {
+      bad |= !(W[q] >= T(0)) || isinf(W[q]);
+      best = fmax(best, W[q]);
+    }
   }
-  if ((threadIdx.x & 31) == 0 && best) atomicMax(maxkey, best);
+  best = warp_max(best);
+  if (__any_sync(FULL, bad) && (threadIdx.x & 31) == 0) atomicOr(err, ERR_NUMERIC);
+  if ((threadIdx.x & 31) == 0 && best > T(0))
+    atomicMax(maxkey, sizeof(T) == 8 ? (unsigned long long)__double_as_longlong((double)best)
+                                     : (unsigned long long)__float_as_uint((float)best));
 }
 
 // C = sum floor(W_i 2^(S - e)) with e from the largest weight; also publishes S - e.
 template <typename T>
-__global__ void sumc_kernel(const T* w, long long n, int S, const unsigned long long* maxkey,
-                            unsigned long long* C, int* shift_out, int* err) {
+__global__ void __launch_bounds__(256) sumc_kernel(const T* w, long long n, int S, const unsigned long long* maxkey,
+                                                   unsigned long long* C, int* shift_out, int* err) {
   const unsigned long long k = *maxkey;
   if (k == 0) {
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(err, ERR_NUMERIC);
@@ -42,12 +46,17 @@ __global__ void sumc_kernel(const T* w, long long n, int S, const unsigned long 
   }
   const int e = sizeof(T) == 8 ? ilogb(__longlong_as_double((long long)k))
                                : ilogbf(__uint_as_float((uint32_t)k));
+  if (e > 2000) return;  // an infinite weight (wmax_kernel has flagged it): C stays 0
   const int shift = S - e;
   if (blockIdx.x == 0 && threadIdx.x == 0) *shift_out = shift;
+  const bool vec = ((uintptr_t)w & 15) == 0;
   unsigned long long s = 0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    s += quantize_u64(w[i], shift);
+  for (long long i = (blockIdx.x * 256ll + threadIdx.x) * WQ; i < n; i += (long long)gridDim.x * 256 * WQ) {
+    T W[WQ];
+    load_weights<T, WQ>(w, i, n, vec, W);
+#pragma unroll
+    for (int q = 0; q < WQ; ++q) s += quantize_u64(W[q], shift);
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
   if ((threadIdx.x & 31) == 0 && s) atomicAdd(C, s);
@@ -106,7 +115,7 @@ template <typename T>
 static void launch_global(const T* w, long long n, const uint32_t* u, int32_t* out, Scratch& sc,
                           cudaStream_t s, long long withhold = -1) {
   const int S = 62 - ceil_log2_i(n);
-  const int grid = (int)std::min<long long>((n + 1023) / 1024, 4 * 152);
+  const int grid = (int)std::min<long long>((n + 256 * WQ - 1) / (256 * WQ), 8 * 152);
   wmax_kernel<T><<<grid, 256, 0, s>>>(w, n, sc.maxkey, sc.err);
   sumc_kernel<T><<<grid, 256, 0, s>>>(w, n, S, sc.maxkey, sc.C, sc.shift, sc.err);
   GlobalArgs<T> a{};

@@ -5,6 +5,7 @@
 #pragma once
 
 #include <cuda/atomic>
+#include <cstring>
 
 #include "dpf_common.cuh"
 #include "dpf_internal.h"
@@ -15,25 +16,36 @@ constexpr int SPIN_LIMIT = 1 << 22;  // bounded look-back wait (~0.3 s with the 
 
 typedef unsigned __int128 u128;
 
-// K(c) = #{ k in [0, n) : (k 2^32 + u) C < c n 2^32 }: the number of systematic
-// points below the cumulative count c (global rule).
-__device__ __forceinline__ long long points_below(unsigned long long c, long long n, uint32_t u,
-                                                  unsigned long long C) {
+template <typename T>
+__device__ __forceinline__ T pow2_t(int e);
+template <>
+__device__ __forceinline__ float pow2_t<float>(int e) { return __int_as_float((127 + e) << 23); }
+template <>
+__device__ __forceinline__ double pow2_t<double>(int e) {
+  return __longlong_as_double((long long)(1023 + e) << 52);
+}
+
+// K(c) = #{ k in [0, n) : (k 2^32 + u) C < c n 2^32 }, the number of systematic
+// points below the cumulative count c (global rule). The
+// condition falls as k grows, so K is the first k where it fails: an estimate
+// c n / C - u 2^-32 (single precision up to n = 2^24, whose error is a few units;
+// double beyond) is settled by exact 128-bit comparisons.
+__device__ __forceinline__ int points_below_est(unsigned long long c, long long n, uint32_t u,
+                                                unsigned long long C) {
   if (c == 0) return 0;
   const u128 X = ((u128)c * (u128)(unsigned long long)n) << 32;
-  const u128 uC = (u128)u * (u128)C;
-  if (X <= uC) return 0;
-  // K = ceil((X - uC) / (C 2^32)) = floor(Y / C) + 1 with Y = (X - uC - 1) >> 32 < 2^94:
-  // a double estimate of the quotient (<= n < 2^31), corrected exactly in 128 bits
-  const u128 Y = (X - uC - 1) >> 32;
-  const double yd = (double)(unsigned long long)(Y >> 64) * 18446744073709551616.0 +
-                    (double)(unsigned long long)Y;
-  long long q = (long long)(yd / (double)C);
-  if (q < 0) q = 0;
-  while (q > 0 && (u128)(unsigned long long)q * C > Y) --q;
-  while ((u128)(unsigned long long)(q + 1) * C <= Y) ++q;
-  const long long k = q + 1;
-  return k >= n ? n : k;
+  long long k;
+  if (n <= (1ll << 24)) {
+    const float e = __fdividef((float)c, (float)C) * (float)n - (float)u * 0x1p-32f;
+    k = e > 0.f ? (long long)ceilf(e) : 0;
+  } else {
+    const double e = (double)c / (double)C * (double)n - (double)u * 0x1p-32;
+    k = e > 0.0 ? (long long)ceil(e) : 0;
+  }
+  if (k > n) k = n;
+  while (k > 0 && !((u128)((unsigned long long)(k - 1) << 32 | u) * C < X)) --k;
+  while (k < n && (u128)((unsigned long long)k << 32 | u) * C < X) ++k;
+  return (int)k;
 }
 
 // Inputs of the scan-and-scatter pass: the weights W_i, with e = floor(log2 max W)
@@ -63,22 +75,40 @@ __device__ __forceinline__ float exp_t<float>(float v) { return expf(v); }
 template <>
 __device__ __forceinline__ double exp_t<double>(double v) { return exp(v); }
 
-// c = floor(W 2^shift) as a 64-bit count (exact: power-of-two scaling, floor).
-__device__ __forceinline__ unsigned long long quantize_u64(float W, int shift) {
-  return (unsigned long long)floorf(ldexpf(W, shift));
+// c = floor(W 2^shift) as a 64-bit count (exact: power-of-two scaling, floor). The scaling is two
+// products by powers of two, each of half the exponent (|shift| <= 211 in FP32, 1136 in FP64, so
+// both factors are normal numbers): where the result is at least 1, W, the product between and the
+// result are ordered in magnitude, so both products are exact, as ldexp is; below 1 the floor is 0.
+template <typename T>
+__device__ __forceinline__ unsigned long long quantize_u64(T W, int shift) {
+  const int h = shift / 2;
+  return (unsigned long long)floor(W * pow2_t<T>(h) * pow2_t<T>(shift - h));
 }
-__device__ __forceinline__ unsigned long long quantize_u64(double W, int shift) {
-  return (unsigned long long)floor(ldexp(W, shift));
+
+// Q consecutive weights from w[i], zeros past n: 16-byte loads where `vec` (w on 16 bytes, i a
+// multiple of Q).
+template <typename T, int Q>
+__device__ __forceinline__ void load_weights(const T* __restrict__ w, long long i, long long n, bool vec, T (&v)[Q]) {
+  if (vec && i + Q <= n) {
+    constexpr int V = 16 / (int)sizeof(T);
+#pragma unroll
+    for (int q = 0; q < Q / V; ++q) {
+      const uint4 b = __ldg(reinterpret_cast<const uint4*>(w + i) + q);
+      memcpy(&v[q * V], &b, 16);
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < Q; ++q) v[q] = i + q < n ? w[i + q] : T(0);
+  }
 }
 
 // One tile of the `ntiles` tiles of one resampling, the tile taken by ticket.
 template <typename T>
 __device__ __forceinline__ void global_scan_scatter_body(const GlobalArgs<T>& a, long long ntiles) {
-  __shared__ unsigned long long cum[SCAN_TILE];
+  __shared__ int ks[SCAN_TILE + 1];  // systematic points below each item's cumulative count
   __shared__ unsigned long long wsum[SCAN_NT / 32];
   __shared__ unsigned long long s_prefix;
   __shared__ long long s_tile;
-  __shared__ long long s_klo, s_khi;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
   if (tid == 0) {
@@ -91,21 +121,21 @@ __device__ __forceinline__ void global_scan_scatter_body(const GlobalArgs<T>& a,
   if (tile < 0) return;
   const long long base = tile * SCAN_TILE;
   const unsigned long long C = *a.C;
+  if (C == 0) return;  // no positive finite weight (flagged): in every tile, so none waits for another
   const int shift = a.shift_dev ? *a.shift_dev : a.shift;
   const uint32_t u = a.u_ptr ? *a.u_ptr : rand_word(a.key, a.t, 0, P_OUTER, 0);
 
   // quantise this thread's items (blocked arrangement) and sum them
   unsigned long long c[SCAN_IPT];
   unsigned long long tsum = 0;
+  {
+    T W[SCAN_IPT];
+    load_weights<T, SCAN_IPT>(a.w, base + (long long)tid * SCAN_IPT, a.n, ((uintptr_t)a.w & 15) == 0, W);
 #pragma unroll
-  for (int q = 0; q < SCAN_IPT; ++q) {
-    const long long i = base + (long long)tid * SCAN_IPT + q;
-    unsigned long long ci = 0;
-    if (i < a.n) {
-      ci = quantize_u64(a.w[i], shift);
+    for (int q = 0; q < SCAN_IPT; ++q) {
+      c[q] = quantize_u64(W[q], shift);
+      tsum += c[q];
     }
-    c[q] = ci;
-    tsum += ci;
   }
   // block exclusive scan of the per-thread sums
   unsigned long long v = tsum;
@@ -181,33 +211,30 @@ __device__ __forceinline__ void global_scan_scatter_body(const GlobalArgs<T>& a,
             .store((ep << 2) | 2u, cuda::memory_order_release);
       }
     }
-    if (lane == 0) {
-      s_prefix = prefix;
-      s_klo = points_below(prefix, a.n, u, C);
-      s_khi = points_below(prefix + agg, a.n, u, C);
-    }
+    if (lane == 0) s_prefix = prefix;
   }
   __syncthreads();
-  // global inclusive cumulative counts of this tile into shared memory
+  // scatter: output k takes the item j of this tile with ks[j] <= k < ks[j + 1]. The exact 128-bit
+  // arithmetic is done once an item (the count of points below its cumulative count) and the
+  // search compares 32-bit counts; a search on cumulative counts took eleven 128-bit products
+  // an output (36 us of a call at n = 1,000,003)
   unsigned long long run = s_prefix + texcl;
+  if (tid == 0) ks[0] = points_below_est(run, a.n, u, C);
 #pragma unroll
   for (int q = 0; q < SCAN_IPT; ++q) {
     run += c[q];
-    cum[tid * SCAN_IPT + q] = run;
+    ks[tid * SCAN_IPT + q + 1] = points_below_est(run, a.n, u, C);
   }
   __syncthreads();
-  // scatter: output k takes the first item of this tile with cum * n 2^32 > (k 2^32 + u) C
-  const long long len = (a.n - base) < SCAN_TILE ? (a.n - base) : SCAN_TILE;
-  const u128 scale = (u128)(unsigned long long)a.n << 32;
-  for (long long k = s_klo + tid; k < s_khi; k += SCAN_NT) {
-    const u128 rhs = ((u128)(unsigned long long)k << 32 | u) * (u128)C;
-    int lo = 0, hi = (int)len - 1;
-    while (lo < hi) {
+  const int khi = ks[SCAN_TILE];
+  for (int k = ks[0] + tid; k < khi; k += SCAN_NT) {
+    int lo = 0, hi = SCAN_TILE;
+    while (hi - lo > 1) {
       const int mid = (lo + hi) >> 1;
-      if ((u128)cum[mid] * scale > rhs)
-        hi = mid;
+      if (ks[mid] <= k)
+        lo = mid;
       else
-        lo = mid + 1;
+        hi = mid;
     }
     a.out[k] = (int32_t)(base + lo);
   }
