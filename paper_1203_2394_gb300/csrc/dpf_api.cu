@@ -400,7 +400,7 @@ dpf_status dpf_create(const dpf_model_desc* model, int32_t d1, int32_t d2, int64
        !dalloc(*x, x->yb, s * 2 * x->dy) && !dalloc(*x, x->anc, 4 * N) && !dalloc(*x, x->sel, 4 * N) &&
        !dalloc(*x, x->stats, ssz) && !dalloc(*x, x->lwmax_t, 8) && !dalloc(*x, x->lwmax_key, 8) &&
        !dalloc(*x, x->Csum, 8) && !dalloc(*x, x->done, 8) && !dalloc(*x, x->err, 8) &&
-       !dalloc(*x, x->partials, sizeof(double) * out_ctas * (4 + d)) &&
+       !dalloc(*x, x->partials, sizeof(double) * 2 * out_ctas * (4 + d)) &&
        !dalloc(*x, x->ctot, sizeof(unsigned long long) * out_ctas);
   if (!ok) {
     std::string msg = g_err;
@@ -788,8 +788,18 @@ dpf_status dpf_read(dpf_ctx* x, const char* which, void* dst, size_t bytes) {
   else if (w == "anc") { src = x->anc; need = 4 * N; }
   else if (w == "sel") { src = x->sel; need = 4 * N; }
   else if (w == "wout") { src = x->wout; need = s * N; }
+  else if (w == "xm" && x->pf && x->pf_rows) {  // a particle's part is the particle: rows of x, by coordinate
+    if (bytes != s * N * x->d1)
+      return set_error(DPF_E_INVALID, "dpf_read: 'xm' needs " + std::to_string(s * N * x->d1) + " bytes");
+    cudaError_t e = cudaSuccess;
+    for (int c = 0; c < x->d1 && e == cudaSuccess; ++c)
+      e = cudaMemcpy2DAsync((char*)dst + s * N * c, s, (const char*)x->x[cur] + s * c, s * x->xp, s, N,
+                            cudaMemcpyDeviceToHost, x->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(x->stream);
+    return cuda_error(e, "dpf_read");
+  }
   else if (w == "xm") { src = x->xm; need = s * N * x->d1; }
-  else if (w == "zm") { src = x->zm; need = s * N * x->d2; }
+  else if (w == "zm") { src = x->pf && x->pf_rows ? x->z[cur] : x->zm; need = s * N * x->d2; }
   else if (w == "x") {  // rows are padded to xp elements on the device; returned packed
     if (bytes != s * N * x->d1)
       return set_error(DPF_E_INVALID, "dpf_read: 'x' needs " + std::to_string(s * N * x->d1) + " bytes");

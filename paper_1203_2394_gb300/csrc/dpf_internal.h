@@ -185,6 +185,7 @@ struct dpf_ctx {
   // reads them after one synchronisation instead of two device-to-host copies
   double* hstats = nullptr;
   double* hstats_dev = nullptr;     // ... its device address
+  int pf_rows = 0;                  // rows of sums the particle filter's last step left in `partials`
   bool host_out = false;            // the coming outer stage writes the mirror
   double* diag_inner = nullptr;     // [sum of the groups' inner ESS, their minimum (as bits)]
   void* lwmax_t = nullptr;          // the largest log-weight of the step, as T

@@ -75,18 +75,24 @@ __device__ __forceinline__ void outer_sums(const FusedOuterArgs<T>& a, int bid, 
 #pragma unroll
   for (int q = 0; q < NV; ++q) v[q] = T(0);
   unsigned long long cc = 0;
-  for (long long i = i0 + tid; i < iend; i += OF_NT) {
-    const T W = exp_t<T>(o.lw[i] - lwmax);
-    cc += (unsigned long long)floor(W * sS);  // exact: a power-of-two scaling, then a floor
-    v[0] += W;
-    v[1] += W * W;
+  const bool given = sums_given(o, lwmax);  // uniform over the grid
+  if (given) {
+    for (long long i = i0 + tid; i < iend; i += OF_NT)
+      cc += (unsigned long long)floor(exp_t<T>(o.lw[i] - lwmax) * sS);
+  } else {
+    for (long long i = i0 + tid; i < iend; i += OF_NT) {
+      const T W = exp_t<T>(o.lw[i] - lwmax);
+      cc += (unsigned long long)floor(W * sS);  // exact: a power-of-two scaling, then a floor
+      v[0] += W;
+      v[1] += W * W;
 #pragma unroll
-    for (int c = 0; c < D1; ++c) v[2 + c] += W * o.xm[(long long)c * N + i];
+      for (int c = 0; c < D1; ++c) v[2 + c] += W * o.xm[c * o.xc + i * o.xi];
 #pragma unroll
-    for (int c = 0; c < D2; ++c) v[2 + D1 + c] += W * o.zm[(long long)c * N + i];
+      for (int c = 0; c < D2; ++c) v[2 + D1 + c] += W * o.zm[(long long)c * N + i];
+    }
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] = warp_sum(v[q]);
   }
-#pragma unroll
-  for (int q = 0; q < NV; ++q) v[q] = warp_sum(v[q]);
   cc = warp_sum(cc);
   if (lane == 0) {
 #pragma unroll
@@ -95,7 +101,7 @@ __device__ __forceinline__ void outer_sums(const FusedOuterArgs<T>& a, int bid, 
   }
   __syncthreads();
   if (tid == 0) {  // one thread publishes the CTA's row (so that one fence covers it)
-    for (int q = 0; q < NV; ++q) {
+    for (int q = 0; q < (given ? 0 : NV); ++q) {
       T s = T(0);
 #pragma unroll
       for (int r = 0; r < NW; ++r) s += sv[q][r];
@@ -220,9 +226,11 @@ __device__ __forceinline__ void outer_stats(const FusedOuterArgs<T>& a, int nb, 
   const OuterArgs<T>& o = a.o;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int D = o.d1 + o.d2, NV = 2 + D;
+  const bool given = sums_given(o, lwmax);
+  const int rows = given ? o.npre : nb;
   for (int q = w; q < NV; q += NW) {
     double s = 0.0;
-    for (int b = lane; b < nb; b += 32) s += __ldcg(o.partials + (long long)b * NV + q);
+    for (int b = lane; b < rows; b += 32) s += __ldcg(o.partials + (long long)b * NV + q);
     s = warp_sum(s);
     if (lane == 0) sd[q] = s;
   }
@@ -237,11 +245,11 @@ __device__ __forceinline__ void outer_stats(const FusedOuterArgs<T>& a, int nb, 
   if (tid == 0) {
     const bool bad = !(lwmax > neg_inf<T>()) || lwmax != lwmax || !(t1 > 0) || C == 0;
     if (bad) atomicOr(o.err, ERR_NUMERIC);
-    const double lz = (double)lwmax + log(t1) - a.logN;
+    const double lz = (given ? (double)o.lref : (double)lwmax) + log(t1) - a.logN;
     o.stats[0] += lz;
     o.stats[1] = lz;
     o.stats[2] = t1 * t1 / sd[1];
-    o.stats[3] = t1;
+    o.stats[3] = given ? t1 * exp((double)o.lref - (double)lwmax) : t1;
     if (o.logz_out) *o.logz_out = o.stats[0];
     *o.lwmax_t = lwmax;
     *o.Csum = C;

@@ -28,6 +28,8 @@ dpf_status check_outer_barrier(cudaStream_t s) {
   o.lw = (const float*)b;
   o.xm = (const float*)(b + fb);
   o.zm = (const float*)(b + 2 * fb);
+  o.xc = n;
+  o.xi = 1;
   a.w_out = (float*)(b + 3 * fb);
   a.anc = (int32_t*)(b + 4 * fb);
   o.N = n;

@@ -1388,10 +1388,15 @@ __global__ void __launch_bounds__(MAXNT)
 template <typename T>
 struct OuterArgs {
   const T* lw;
-  const T* xm;
-  const T* zm;
+  const T* xm;       // x mean of item i, coordinate c: xm[c xc + i xi]
+  const T* zm;       // z means [c][N]
+  long long xc, xi;
   long long N;
   int d1, d2;
+  // npre > 0: `partials` already holds npre rows of the sums, of W' = exp(lw - lref) in the place
+  // of exp(lw - max lw); they are used unless max lw is so far below lref that they lose digits
+  int npre;
+  T lref;
   unsigned long long* lwmax_key;
   T* lwmax_t;
   unsigned long long* Csum;

@@ -26,6 +26,17 @@ void fill_outer_args(Ctx& x, double* mean_out, double* logz_out, unsigned int* a
     o.lw = (const T*)x.lw;
     o.xm = (const T*)x.xm;
     o.zm = (const T*)x.zm;
+    o.xc = x.N;
+    o.xi = 1;
+    if (x.pf && x.pf_rows) {  // the particles themselves are the means, and their step has summed them
+      const int cur = (int)((x.t + 1) % 2);
+      o.xm = (const T*)x.x[cur];
+      o.xc = 1;
+      o.xi = x.xp;
+      o.zm = (const T*)x.z[cur];
+      o.npre = x.pf_rows;
+      o.lref = (T)x.hm.lognorm_y;
+    }
     o.N = x.N;
     o.d1 = x.d1;
     o.d2 = x.d2;
@@ -383,18 +394,26 @@ struct VariantImpl {
     a.y = (const T*)x.yb + (t % 2) * x.dy;
     a.lwmax_key = x.lwmax_key;
     a.Csum = x.Csum;
+    a.partials = x.partials;
     a.N = x.N;
-    a.xp = x.xp;
     a.t = (uint32_t)t;
     a.key = Key{(uint32_t)x.seed, (uint32_t)(x.seed >> 32)};
     const HostModel& h = x.hm;
     a.gcos = h.growth ? (T)(h.gc * std::cos(h.gw * (double)(t - 1))) : T(0);
     a.first = t == 1 ? 1 : 0;
-    const unsigned blocks = (unsigned)std::min<long long>((x.N + 255) / 256, 152 * 8);
-    if (use_xz(x))
-      pf_kernel<T, D1, D2, DY, true><<<blocks, 256, 0, x.stream>>>(cst(x), a);
-    else
-      pf_kernel<T, D1, D2, DY, false><<<blocks, 256, 0, x.stream>>>(cst(x), a);
+    auto k = use_xz(x) ? pf_kernel<T, D1, D2, DY, true> : pf_kernel<T, D1, D2, DY, false>;
+    if (x.grid_step == 0) {  // as many CTAs as fit on the device at once
+      int nb = 0, dev = 0, nsm = 0;
+      cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, PF_NT, 0);
+      if (e == cudaSuccess) e = cudaGetDevice(&dev);
+      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+      if (e != cudaSuccess) return cuda_error(e, "particle filter step occupancy");
+      x.grid_step = std::min((nb > 0 ? nb : 1) * nsm, OF_MAX_CTAS);
+    }
+    // one row of sums a CTA: the context holds two for every 512 particles, up to 2 OF_MAX_CTAS
+    const unsigned blocks = (unsigned)std::min<long long>((x.N + PF_NT - 1) / PF_NT, x.grid_step);
+    x.pf_rows = (int)blocks;
+    k<<<blocks, PF_NT, 0, x.stream>>>(cst(x), a);
     return cuda_error(cudaGetLastError(), "particle filter step launch");
   }
 
