@@ -17,7 +17,7 @@
 // the same normals.
 #pragma once
 
-#include "dpf_step.cuh"
+#include "dpf_step_warp.cuh"
 
 namespace dpf {
 
@@ -270,6 +270,352 @@ __global__ void __launch_bounds__(1024)
       if (lwi == lwi && key > *(volatile unsigned long long*)a.lwmax_key) atomicMax(a.lwmax_key, key);
     }
     __syncthreads();  // the staged rows are free for the next group
+  }
+}
+
+// Sums over the warp of N values a lane, returned to every lane as out[0..N-1]. Halving: a
+// shuffle step exchanges half of the values still held for the other half of its partner's,
+// so a step costs half of the one before it (N = 8: 4 + 2 + 1 + 1 + 1 shuffles and one each to
+// hand out a total, not 40).
+template <int N, typename T>
+__device__ __forceinline__ T warp_sum_vec(const T (&v)[N], int lane) {
+  // lane l returns the total of value l mod NP (NP: N rounded up to a power of two)
+  constexpr int NP = N <= 1 ? 1 : N <= 2 ? 2 : N <= 4 ? 4 : N <= 8 ? 8 : N <= 16 ? 16 : 32;
+  static_assert(N <= 32, "one total a lane");
+  T w[NP];
+#pragma unroll
+  for (int q = 0; q < NP; ++q) w[q] = q < N ? v[q < N ? q : 0] : T(0);
+#pragma unroll
+  for (int h = NP / 2; h > 0; h /= 2) {
+    const bool up = (lane & h) != 0;
+#pragma unroll
+    for (int q = 0; q < h; ++q) {
+      const T give = up ? w[q] : w[q + h];
+      const T keep = up ? w[q + h] : w[q];
+      w[q] = keep + __shfl_xor_sync(FULL, give, h);
+    }
+  }
+#pragma unroll
+  for (int o = NP; o < 32; o <<= 1) w[0] += __shfl_xor_sync(FULL, w[0], o);
+  return w[0];
+}
+
+// The same step with one warp a group (M <= 256, rows of whole 16-byte units): each lane owns
+// PPL consecutive inner particles in registers, every reduction and scan is a warp shuffle, the
+// local resampling takes the offspring ranges (no search), and the ancestor's rows of the next
+// group are bulk-copied into the warp's stage while this one's are used. A group takes 1.9 k warp instructions, not 6.9 k; the growth model's step (N = 65536,
+// M = 128) went from 581 to 197 us, 45% of the copy bandwidth; what bounds it now is the issue of
+// the random numbers and the propagation at four warps a scheduler.
+// The component draw of x_t is made only where it is read (an x transition that depends
+// on z, or debug recording). The Gaussian form of the draw keeps the block kernel.
+template <typename T, int D1, int D2>
+inline size_t std_warp_smem(int M, int xp) {  // bytes a warp
+  return (size_t)D2 * M * sizeof(T) + (size_t)M * sizeof(T) + (size_t)xp * sizeof(T) +
+         ((size_t)M * sizeof(int) + 15) / 16 * 16 + 256 * sizeof(T);
+}
+
+// Sum over the warp of values held PPL consecutive ones a lane, added as a block of one thread a
+// value adds them: 32 neighbours by a butterfly, then the groups of 32 in order (the block-wide
+// form's bits, so that the weights, and every resampling decision after them, do not depend
+// on which form ran). ws: 32 PPL elements of the warp's shared memory.
+template <typename T, int PPL>
+__device__ __forceinline__ T strided_sum(const T (&v)[PPL], T* ws, int k0, int lane) {
+  if constexpr (PPL == 1) {
+    return warp_sum(v[0]);
+  } else {
+    vst<T, PPL>(ws + k0, v);
+    __syncwarp();
+    T r = T(0);
+#pragma unroll
+    for (int p = 0; p < PPL; ++p) {
+      const T s = warp_sum(ws[32 * p + lane]);
+      r = p ? r + s : s;
+    }
+    __syncwarp();
+    return r;
+  }
+}
+
+template <typename T, int D1, int D2, int DY, bool XZ, int PPL>
+__global__ void __launch_bounds__(WARPS_PER_CTA * 32, warp_min_blocks<PPL, D2>())
+    std_warp_kernel(const __grid_constant__ MC<T, D1, D2, DY> mc, const __grid_constant__ StdArgs<T> a,
+                    uint32_t warp_bytes) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t bars[WARPS_PER_CTA];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int M = a.M, k0 = PPL * lane;
+  const bool act = k0 < M;
+  const long long N = a.N, NM = N * (long long)M;
+  T* sz = (T*)(smem_raw + (size_t)wib * warp_bytes);  // [D2][M] the ancestor group's z
+  T* slq = sz + D2 * M;                               // [M]
+  T* sx = slq + M;                                    // [xp]
+  int* slot = (int*)(sx + a.xp);                      // [M] scratch of the local resampling
+  T* ws = (T*)((unsigned char*)slot + ((size_t)M * sizeof(int) + 15) / 16 * 16);  // [32 PPL] sums
+  uint64_t* bar = &bars[wib];
+  uint32_t phase = 0;
+  const T NEG = neg_inf<T>(), LOG2E = (T)LOG2E_D;
+  const RoundKeys rk = round_keys(a.key);
+  if (lane == 0) {
+    mbar_init(bar, 1);
+    mbar_fence_init();
+  }
+  __syncwarp();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *a.Csum = 0ull;
+  const uint32_t row = (uint32_t)(M * sizeof(T));
+  auto stage = [&](long long src) {
+    if (lane == 0) mbar_arrive_tx(bar, (D2 + 1) * row + (uint32_t)(a.xp * sizeof(T)));
+    for (int e = lane; e < D2 + 2; e += 32) {
+      if (e < D2)
+        bulk_load(sz + e * M, a.z_old + e * NM + src * M, row, bar);
+      else if (e == D2)
+        bulk_load(slq, a.lq_old + src * M, row, bar);
+      else
+        bulk_load(sx, a.x_old + src * a.xp, (uint32_t)(a.xp * sizeof(T)), bar);
+    }
+  };
+  const long long W = (long long)gridDim.x * nw;
+  long long i = (long long)blockIdx.x * nw + wib;
+  long long src_next = -1;
+  if (i < N) {
+    stage(a.first ? i : (long long)a.anc[i]);
+    if (i + W < N) src_next = a.first ? i + W : (long long)a.anc[i + W];
+  }
+  for (; i < N; i += W, phase ^= 1u) {
+    {  // wait for this group's rows (bounded)
+      int spins = 0;
+      while (!mbar_test(bar, phase)) {
+        if (++spins > MBAR_SPIN_LIMIT) {
+          if (lane == 0) atomicOr(a.err, ERR_TIMEOUT);
+          break;
+        }
+      }
+    }
+    T xp_[D1], alpha[PPL];
+#pragma unroll
+    for (int c = 0; c < D1; ++c) xp_[c] = sx[c];
+#pragma unroll
+    for (int p = 0; p < PPL; ++p) alpha[p] = NEG;
+    if (act) vld<T, PPL>(slq + k0, alpha);
+    // inclusive cumulative counts of the lane's particles for the log-weights v, and the total
+    auto counts = [&](const T (&v)[PPL], T mx, uint32_t (&loc)[PPL]) {
+      uint32_t run = 0;
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) {
+        run += act ? (uint32_t)floor(exp2_t((v[p] - mx) * LOG2E) * a.scaleM) : 0u;
+        loc[p] = run;
+      }
+      uint32_t s = run;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t n = __shfl_up_sync(FULL, s, o);
+        if (lane >= o) s += n;
+      }
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) loc[p] += s - run;
+      return __shfl_sync(FULL, s, 31);
+    };
+    auto lane_max = [&](const T (&v)[PPL]) {
+      T m = v[0];
+#pragma unroll
+      for (int p = 1; p < PPL; ++p) m = fmax(m, v[p]);
+      return warp_max_redux(m);
+    };
+    // ---- x_t from the mixture: the component, then the Gaussian draw ----
+    T e1[D1], mux[D1], xt[D1];
+    normals_rk<D1>(rk, a.t, (uint32_t)i, P_LA_X, 0u, e1);
+    mu_x(mc, xp_, a.gcos, mux);
+    T w[D1];
+#pragma unroll
+    for (int r = 0; r < D1; ++r) w[r] = e1[r];
+    if (XZ || a.dbg_j) {
+      // the one-draw local rule: the component is the number of particles whose cumulative
+      // count c_k has c_k 2^32 <= u C
+      uint32_t loc[PPL];
+      const uint32_t C = counts(alpha, lane_max(alpha), loc);
+      const uint64_t rhs = (uint64_t)philox_rk(ctr(a.t, (uint32_t)i, P_LA_J, 0u, 0u), rk).x * C;
+      unsigned below = 0;
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) below += act && ((uint64_t)loc[p] << 32) <= rhs ? 1u : 0u;
+      const int jm = min((int)__reduce_add_sync(FULL, below), M - 1);
+      if (a.dbg_j && lane == 0) a.dbg_j[i] = jm;
+      if (XZ) {
+#pragma unroll
+        for (int r = 0; r < D1; ++r) {
+#pragma unroll
+          for (int c = 0; c < D2; ++c) w[r] += mc.WAxz[r][c] * sz[c * M + jm];
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < D1; ++r) {
+      T v = mux[r];
+#pragma unroll
+      for (int c = 0; c < D1; ++c)
+        if (c <= r) v += mc.Lqx[r][c] * w[c];
+      xt[r] = v;
+    }
+    // ---- local resampling by q = qbar p(x_t | x_{t-1}, z) ----
+    if (XZ && act) {
+      T wres[D1], q[PPL];
+#pragma unroll
+      for (int r = 0; r < D1; ++r) {
+        T v = T(0);
+#pragma unroll
+        for (int c = 0; c < D1; ++c)
+          if (c <= r) v += mc.LqxInv[r][c] * (xt[c] - mux[c]);
+        wres[r] = v;
+      }
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) q[p] = T(0);
+#pragma unroll
+      for (int r = 0; r < D1; ++r) {
+        T v[PPL];
+#pragma unroll
+        for (int p = 0; p < PPL; ++p) v[p] = wres[r];
+#pragma unroll
+        for (int c = 0; c < D2; ++c) {
+          T zc[PPL];
+          vld<T, PPL>(sz + c * M + k0, zc);
+          axpy<T, PPL>(-mc.WAxz[r][c], zc, v);
+        }
+#pragma unroll
+        for (int p = 0; p < PPL; ++p) q[p] += v[p] * v[p];
+      }
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) alpha[p] -= T(0.5) * q[p];
+    }
+    int bidx[PPL];
+    {
+      uint32_t loc[PPL];
+      const uint32_t C = counts(alpha, lane_max(alpha), loc);
+      const uint32_t uin = philox_rk(ctr(a.t, (uint32_t)i, P_INNER, 0u, 0u), rk).x;
+      sys_local_offspring<PPL>(loc, C, M, uin >> 16, k0, act, lane, slot, bidx);
+    }
+    if (a.dbg_b && act) vst<int, PPL>(a.dbg_b + i * M + k0, bidx);
+    // ---- propagation from the prior and the weights of y_t ----
+    T yh[DY];
+    {
+      T hx[DY], res[DY];
+      h_x(mc, xt, hx);
+#pragma unroll
+      for (int q = 0; q < DY; ++q) res[q] = a.y[q] - hx[q];
+#pragma unroll
+      for (int q = 0; q < DY; ++q) {
+        T v = T(0);
+#pragma unroll
+        for (int c = 0; c < DY; ++c)
+          if (c <= q) v += mc.LrInv[q][c] * res[c];
+        yh[q] = v;
+      }
+    }
+    T zn[D2][PPL];
+#pragma unroll
+    for (int r = 0; r < D2; ++r) {
+      T v = T(0);
+#pragma unroll
+      for (int c = 0; c < D1; ++c) v += mc.Azx[r][c] * xp_[c];
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) zn[r][p] = v;
+    }
+#pragma unroll
+    for (int c = 0; c < D2; ++c) {
+      T zc[PPL];
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) zc[p] = sz[c * M + bidx[p]];
+#pragma unroll
+      for (int r = 0; r < D2; ++r) axpy<T, PPL>(mc.Azz[r][c], zc, zn[r]);
+    }
+    // the stage is consumed: prefetch the next group's rows into it
+    __syncwarp();
+    if (i + W < N) {
+      stage(src_next);
+      if (i + 2 * W < N) src_next = a.first ? i + 2 * W : (long long)a.anc[i + 2 * W];
+    }
+#pragma unroll
+    for (int b = 0; b < (D2 + 3) / 4; ++b) {
+      T e4[4][PPL];
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) {
+        T e[4];
+        normal_block_rk(rk, a.t, (uint32_t)i, P_PROP, (uint32_t)(k0 + p), b, D2 - 4 * b, e);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) e4[j][p] = e[j];
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c = 4 * b + j;
+        if (c < D2) {
+          if (mc.diag_qz) {
+            axpy<T, PPL>(mc.Lqz[c][c], e4[j], zn[c]);
+          } else {
+#pragma unroll
+            for (int r = 0; r < D2; ++r)
+              if (r >= c) axpy<T, PPL>(mc.Lqz[r][c], e4[j], zn[r]);
+          }
+        }
+      }
+    }
+    T ell[PPL], lmax = NEG;
+    {
+      T qf[PPL];
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) qf[p] = T(0);
+#pragma unroll
+      for (int q = 0; q < DY; ++q) {
+        T v[PPL];
+#pragma unroll
+        for (int p = 0; p < PPL; ++p) v[p] = yh[q];
+#pragma unroll
+        for (int c = 0; c < D2; ++c) axpy<T, PPL>(-mc.LrHz[q][c], zn[c], v);
+#pragma unroll
+        for (int p = 0; p < PPL; ++p) qf[p] += v[p] * v[p];
+      }
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) {
+        ell[p] = act ? mc.lognorm_y - T(0.5) * qf[p] : NEG;
+        lmax = fmax(lmax, ell[p]);
+      }
+    }
+    lmax = warp_max_redux(lmax);
+    T Wp[PPL];
+#pragma unroll
+    for (int p = 0; p < PPL; ++p) Wp[p] = act ? exp_t<T>(ell[p] - lmax) : T(0);
+    const T lsum = strided_sum<T, PPL>(Wp, ws, k0, lane);
+    const T lse = lmax + log_t(lsum);
+    if (act) {
+#pragma unroll
+      for (int c = 0; c < D2; ++c) vst<T, PPL>(a.z_new + c * NM + i * M + k0, zn[c]);
+      T lqn[PPL];
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) lqn[p] = ell[p] - lse;
+      vst<T, PPL>(a.lq_new + i * M + k0, lqn);
+    }
+    // the group's z-mean sum_j qbar z_t (lane c < D2 ends with coordinate c)
+    {
+      T acc[D2];
+#pragma unroll
+      for (int c = 0; c < D2; ++c) {
+        T v = T(0);
+#pragma unroll
+        for (int p = 0; p < PPL; ++p) v += Wp[p] * zn[c][p];
+        acc[c] = act ? v : T(0);
+      }
+      const T tot = warp_sum_vec<D2>(acc, lane) / lsum;
+      if (lane < D2) a.zm[(long long)lane * N + i] = tot;
+    }
+    if (lane == 0) {
+      const T lwi = lse - a.logM;
+#pragma unroll
+      for (int c = 0; c < D1; ++c) {
+        a.x_new[i * a.xp + c] = xt[c];
+        a.xm[(long long)c * N + i] = xt[c];
+      }
+      a.lw[i] = lwi;
+      if (lwi != lwi) atomicOr(a.err, ERR_NUMERIC);
+      const unsigned long long key = order_key(lwi);
+      if (lwi == lwi && key > *(volatile unsigned long long*)a.lwmax_key) atomicMax(a.lwmax_key, key);
+    }
+    __syncwarp();
   }
 }
 

@@ -388,8 +388,6 @@ struct VariantImpl {
     a.x_new = (T*)x.x[sn];
     a.z_new = (T*)x.z[sn];
     a.lw = (T*)x.lw;
-    a.xm = (T*)x.xm;
-    a.zm = (T*)x.zm;
     a.anc = x.anc;
     a.y = (const T*)x.yb + (t % 2) * x.dy;
     a.lwmax_key = x.lwmax_key;
@@ -417,7 +415,38 @@ struct VariantImpl {
     return cuda_error(cudaGetLastError(), "particle filter step launch");
   }
 
-  // The DPF without look-ahead, call t (one CTA a group of M inner particles).
+  template <bool XZ, int PPL>
+  static dpf_status launch_std_warp(Ctx& x, const StdArgs<T>& a) {
+    auto k = std_warp_kernel<T, D1, D2, DY, XZ, PPL>;
+    const size_t wb = std_warp_smem<T, D1, D2>(x.M, x.xp);
+    const int nw = x.N <= FEW_GROUPS ? 1 : WARPS_PER_CTA;
+    if (x.grid_step == 0 || x.grid_kernel != (const void*)k) {  // as many CTAs as fit on the device at once
+      int nb = 0, dev = 0, nsm = 0;
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(wb * WARPS_PER_CTA));
+      if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, WARPS_PER_CTA * 32, wb * WARPS_PER_CTA);
+      if (e == cudaSuccess) e = cudaGetDevice(&dev);
+      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+      if (e != cudaSuccess) return cuda_error(e, "DPF step occupancy");
+      x.grid_step = (nb > 0 ? nb : 1) * nsm;
+      x.grid_kernel = (const void*)k;
+    }
+    const long long want = (x.N + nw - 1) / nw;
+    const unsigned grid = (unsigned)(nw == 1 ? want : std::min<long long>(want, x.grid_step));
+    k<<<grid, 32 * nw, wb * nw, x.stream>>>(cst(x), a, (uint32_t)wb);
+    return cuda_error(cudaGetLastError(), "DPF step launch");
+  }
+  template <bool XZ>
+  static dpf_status launch_std(Ctx& x, const StdArgs<T>& a) {
+    if (x.M <= 32) return launch_std_warp<XZ, 1>(x, a);
+    if (x.M <= 64) return launch_std_warp<XZ, 2>(x, a);
+    if (x.M <= 128) return launch_std_warp<XZ, 4>(x, a);
+    return launch_std_warp<XZ, 8>(x, a);
+  }
+
+  // The DPF without look-ahead, call t: one warp a group where its rows are whole 16-byte
+  // units and fit a stage (as for the step; there is no look-ahead here, so L does not matter),
+  // else one CTA a group of M inner particles.
   static dpf_status std_step(Ctx& x) {
     const long long t = x.t + 1;
     StdArgs<T> a{};
@@ -449,6 +478,10 @@ struct VariantImpl {
     a.gauss = x.std_gauss ? 1 : 0;
     a.dbg_b = x.debug ? x.dbg_b : nullptr;
     a.dbg_j = x.debug ? x.dbg_j : nullptr;
+    if (!a.gauss && warp_path(x.M, 16) && std_warp_smem<T, D1, D2>(x.M, x.xp) * WARPS_PER_CTA <= 200 * 1024) {
+      if constexpr (XZM == 1) return launch_std<true>(x, a);
+      else return use_xz(x) ? launch_std<true>(x, a) : launch_std<false>(x, a);
+    }
     const int nt = (x.M + 31) / 32 * 32;
     const size_t sm = sizeof(T) * (size_t)D2 * x.M + 4 * (size_t)(x.M + 1) + sizeof(T) * 32 + 4 * 64 + 16;
     const unsigned blocks = (unsigned)std::min<long long>(x.N, 152 * 8);
