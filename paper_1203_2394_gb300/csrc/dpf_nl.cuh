@@ -15,7 +15,7 @@
 // noise is B v_z with B = [[1, 0], [1, 1]]; s_0 ~ N(0, I) as the table states.
 #pragma once
 
-#include "dpf_step.cuh"
+#include "dpf_std.cuh"
 
 namespace dpf {
 
@@ -485,6 +485,392 @@ __global__ void __launch_bounds__(1024) nl_step_kernel(const __grid_constant__ N
   }
 }
 
+// The same step with one warp a group (M <= 256, rows of whole 16-byte units): no block barrier,
+// no L x M arrays. The inner update holds PPL consecutive particles a lane (offspring ranges in
+// the place of the searches), the look-ahead particles lane + 32 p, so that its row sums add the
+// pairs in the order of the block form: the log-weights, and with them every resampling
+// decision, keep their bits. A draw's pairs live in registers: both exponents, their row
+// maxima (one warp reduction instruction each), the exponentials, and the lane's partial sums
+// to the table `part`, one row a sum; then a lane adds a row. Bound by issue: model 1 at
+// N = 65536, M = 128, L = 16 went from 806 us a step (10.9 k warp instructions a group, four warps
+// between barriers) to 322.
+// Shared memory of one warp, in floats.
+template <int D1, int D2>
+struct NLWarp {
+  int sz, slq, sx, slwh, sxbb, zk, lqk, fxk, cum, xbs, hxs, rowm, part, total;
+  __host__ __device__ NLWarp(int M, int L, int xp, int ppl) {
+    const int MP = 32 * ppl, L4 = (L + 3) & ~3;
+    int o = 0;
+    sz = o; o += D2 * M;
+    slq = o; o += M;
+    sx = o; o += xp;
+    slwh = o; o += L;
+    sxbb = o; o += L * D1;
+    zk = o; o += D2 * MP;
+    lqk = o; o += MP;
+    fxk = o; o += D1 * MP;
+    cum = o; o += MP;
+    xbs = o; o += L4 * D1;
+    hxs = o; o += L4;
+    rowm = o; o += 2 * L4;
+    part = o; o += (2 + D2) * L * PART_STRIDE;
+    total = o;
+  }
+};
+
+template <class Mod, int PPL>
+__global__ void __launch_bounds__(WARPS_PER_CTA * 32, 4)
+    nl_step_warp_kernel(const __grid_constant__ NLArgs a, const __grid_constant__ NLWarp<Mod::D1, Mod::D2> o) {
+  constexpr int D1 = Mod::D1, D2 = Mod::D2, MP = 32 * PPL;
+  static_assert(Mod::DY == 1, "the look-ahead's pair loop takes a scalar observation");
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t bars[WARPS_PER_CTA];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int M = a.M, L = a.L, k0 = PPL * lane;
+  const bool act = k0 < M;
+  const long long N = a.N, NM = N * (long long)M;
+  float* ws = (float*)smem_raw + (size_t)wib * o.total;
+  float *sz = ws + o.sz, *slq = ws + o.slq, *sx = ws + o.sx, *slwh = ws + o.slwh, *sxbb = ws + o.sxbb;
+  float *zks = ws + o.zk, *lqs = ws + o.lqk, *fxk = ws + o.fxk, *xbs = ws + o.xbs, *hxs = ws + o.hxs;
+  float *rowm = ws + o.rowm, *part = ws + o.part;
+  uint32_t* cum = (uint32_t*)(ws + o.cum);
+  uint64_t* bar = &bars[wib];
+  uint32_t phase = 0;
+  const float NEG = neg_inf<float>(), LOG2E = (float)LOG2E_D;
+  const RoundKeys rk = round_keys(a.key);
+  if (lane == 0) {
+    mbar_init(bar, 1);
+    mbar_fence_init();
+  }
+  __syncwarp();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *a.Csum = 0ull;
+  auto stage = [&](long long src) {
+    if (lane == 0)
+      mbar_arrive_tx(bar, 4u * (uint32_t)((D2 + 1) * M + a.xp + (a.first ? 0 : L + L * D1)));
+    for (int e = lane; e < D2 + 4; e += 32) {
+      if (e < D2)
+        bulk_load(sz + e * M, a.z_old + e * NM + src * M, 4u * M, bar);
+      else if (e == D2)
+        bulk_load(slq, a.lq_old + src * M, 4u * M, bar);
+      else if (e == D2 + 1)
+        bulk_load(sx, a.x_old + src * a.xp, 4u * a.xp, bar);
+      else if (!a.first && e == D2 + 2)
+        bulk_load(slwh, a.lwh_old + src * L, 4u * L, bar);
+      else if (!a.first)
+        bulk_load(sxbb, a.xbb_old + src * L * D1, 4u * L * D1, bar);
+    }
+  };
+  // inclusive cumulative counts of the lane's consecutive particles for the log-weights v
+  auto counts = [&](const float (&v)[PPL], uint32_t (&loc)[PPL]) {
+    float mx = v[0];
+#pragma unroll
+    for (int p = 1; p < PPL; ++p) mx = fmaxf(mx, v[p]);
+    mx = warp_max_redux(mx);
+    uint32_t run = 0;
+#pragma unroll
+    for (int p = 0; p < PPL; ++p) {
+      run += act ? (uint32_t)floor(exp2f((v[p] - mx) * LOG2E) * a.scaleM) : 0u;
+      loc[p] = run;
+    }
+    uint32_t s = run;
+#pragma unroll
+    for (int q = 1; q < 32; q <<= 1) {
+      const uint32_t n = __shfl_up_sync(FULL, s, q);
+      if (lane >= q) s += n;
+    }
+#pragma unroll
+    for (int p = 0; p < PPL; ++p) loc[p] += s - run;
+    return __shfl_sync(FULL, s, 31);
+  };
+  const long long W = (long long)gridDim.x * nw;
+  long long i = (long long)blockIdx.x * nw + wib;
+  long long src_next = -1;
+  if (i < N) {
+    stage(a.first ? i : (long long)a.anc[i]);
+    if (i + W < N) src_next = a.first ? i + W : (long long)a.anc[i + W];
+  }
+  for (; i < N; i += W, phase ^= 1u) {
+    {  // wait for this group's rows (bounded)
+      int spins = 0;
+      while (!mbar_test(bar, phase)) {
+        if (++spins > MBAR_SPIN_LIMIT) {
+          if (lane == 0) atomicOr(a.err, ERR_TIMEOUT);
+          break;
+        }
+      }
+    }
+    float x[D1], zk[D2][PPL], lqk[PPL];
+#pragma unroll
+    for (int p = 0; p < PPL; ++p) {
+      lqk[p] = NEG;
+#pragma unroll
+      for (int c = 0; c < D2; ++c) zk[c][p] = 0.f;
+    }
+    if (a.first) {
+#pragma unroll
+      for (int c = 0; c < D1; ++c) x[c] = sx[c];
+      if (act) {
+#pragma unroll
+        for (int c = 0; c < D2; ++c) vld<float, PPL>(sz + c * M + k0, zk[c]);
+        vld<float, PPL>(slq + k0, lqk);
+      }
+    } else {
+      float xa[D1];
+#pragma unroll
+      for (int c = 0; c < D1; ++c) xa[c] = sx[c];
+      const uint32_t word = philox_rk(ctr(a.t - 1, (uint32_t)i, lane == 0 ? P_SEL : P_INNER, 0u, 0u), rk).x;
+      // ---- x_{t-1}: one of the ancestor's look-ahead draws, by its weight (L <= 32) ----
+      {
+        const float l = lane < L ? slwh[lane] : NEG;
+        const float mx = warp_max_redux(l);
+        uint32_t s = lane < L ? (uint32_t)floor(exp2f((l - mx) * LOG2E) * a.scaleL) : 0u;
+#pragma unroll
+        for (int q = 1; q < 32; q <<= 1) {
+          const uint32_t n = __shfl_up_sync(FULL, s, q);
+          if (lane >= q) s += n;
+        }
+        const uint32_t C = __shfl_sync(FULL, s, 31);
+        const uint64_t rhs = (uint64_t)__shfl_sync(FULL, word, 0) * C;
+        const unsigned b = __ballot_sync(FULL, ((uint64_t)s << 32) > rhs);
+        int m = b ? __ffs(b) - 1 : L - 1;
+        if (C == 0 || m >= L) {
+          if (lane == 0) atomicOr(a.err, ERR_NUMERIC);
+          m = L - 1;
+        }
+        if (lane == 0) a.sel[i] = m;
+#pragma unroll
+        for (int c = 0; c < D1; ++c) x[c] = sxbb[m * D1 + c];
+      }
+      // ---- local resampling by lq + log p(x_{t-1} | x_{t-2}, z) ----
+      int bidx[PPL];
+      {
+        float alpha[PPL];
+#pragma unroll
+        for (int p = 0; p < PPL; ++p) alpha[p] = NEG;
+        if (act) {
+          vld<float, PPL>(slq + k0, alpha);
+          float zz[D2][PPL];
+#pragma unroll
+          for (int c = 0; c < D2; ++c) vld<float, PPL>(sz + c * M + k0, zz[c]);
+#pragma unroll
+          for (int p = 0; p < PPL; ++p) {
+            float z1[D2], fxv[D1], r[D1];
+#pragma unroll
+            for (int c = 0; c < D2; ++c) z1[c] = zz[c][p];
+            Mod::fx(xa, z1, a.tt_prev, fxv);
+#pragma unroll
+            for (int c = 0; c < D1; ++c) r[c] = x[c] - fxv[c];
+            alpha[p] = alpha[p] + nl_quad_x<Mod>(r);
+          }
+        }
+        uint32_t loc[PPL];
+        const uint32_t C = counts(alpha, loc);
+        sys_local_offspring<PPL>(loc, C, M, __shfl_sync(FULL, word, 1) >> 16, k0, act, lane, (int*)cum, bidx);
+      }
+      if (a.dbg_b && act) vst<int, PPL>(a.dbg_b + i * M + k0, bidx);
+      // ---- propagation given x_{t-1} and the update by y_{t-1} ----
+      float ell[PPL], e[PPL], lmax = NEG;
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) {
+        float zb[D2], fxb[D1], fzb[D2], en[D2], zn[D2];
+#pragma unroll
+        for (int c = 0; c < D2; ++c) zb[c] = sz[c * M + bidx[p]];
+        Mod::fx(xa, zb, a.tt_prev, fxb);
+        Mod::fz(xa, zb, a.tt_prev, fzb);
+        normals_rk<D2>(rk, a.t - 1, (uint32_t)i, P_PROP, (uint32_t)(k0 + p), en);
+        nl_zdraw<Mod>(fzb, fxb, x, en, zn);
+        ell[p] = act ? nl_loglik<Mod>(x, zn, a.y_prev) : NEG;
+#pragma unroll
+        for (int c = 0; c < D2; ++c) zk[c][p] = zn[c];
+        lmax = fmaxf(lmax, ell[p]);
+      }
+      lmax = warp_max_redux(lmax);
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) e[p] = act ? expf(ell[p] - lmax) : 0.f;
+      const float lsum = strided_sum<float, PPL>(e, lqs, k0, lane);
+      const float lse = lmax + logf(lsum);
+      if (act) {
+#pragma unroll
+        for (int p = 0; p < PPL; ++p) lqk[p] = ell[p] - lse;
+#pragma unroll
+        for (int c = 0; c < D2; ++c) vst<float, PPL>(a.z_new + c * NM + i * M + k0, zk[c]);
+        vst<float, PPL>(a.lq_new + i * M + k0, lqk);
+      }
+      {
+        float xo = x[0];
+#pragma unroll
+        for (int c = 1; c < D1; ++c)
+          if (lane == c) xo = x[c];
+        if (lane < D1) a.x_new[i * a.xp + lane] = xo;
+      }
+    }
+    // the stage is consumed: prefetch the next group's rows into it
+    __syncwarp();
+    if (i + W < N) {
+      stage(src_next);
+      if (i + 2 * W < N) src_next = a.first ? i + 2 * W : (long long)a.anc[i + 2 * W];
+    }
+    // ======== look-ahead of step t from (x, z, lq) with y_t ========
+    {
+      uint32_t loc[PPL];
+      counts(lqk, loc);
+      vst<uint32_t, PPL>(cum + k0, loc);
+    }
+    // hand the particles over to their look-ahead lanes (lane + 32 p)
+#pragma unroll
+    for (int c = 0; c < D2; ++c) vst<float, PPL>(zks + c * MP + k0, zk[c]);
+    vst<float, PPL>(lqs + k0, lqk);
+    __syncwarp();
+    // per inner particle k: f_x, the base f_z + chol(S) e_k of its draw (the noise e_k shared
+    // by the L draws) and, when the draw is free of x_t, h_z of it
+    float fx[D1][PPL], zb[D2][PPL], hz0[PPL];
+#pragma unroll
+    for (int p = 0; p < PPL; ++p) {
+      const int k = lane + 32 * p;
+      float z1[D2], fxv[D1], fzv[D2], ek[D2], b1[D2];
+#pragma unroll
+      for (int c = 0; c < D2; ++c) z1[c] = zks[c * MP + k];
+      lqk[p] = lqs[k];
+      Mod::fx(x, z1, a.tt_cur, fxv);
+      Mod::fz(x, z1, a.tt_cur, fzv);
+      normals_rk<D2>(rk, a.t, (uint32_t)i, P_LA_Z, (uint32_t)k, ek);
+#pragma unroll
+      for (int r = 0; r < D2; ++r) {
+        float v = fzv[r];
+#pragma unroll
+        for (int c = 0; c < D2; ++c)
+          if (c <= r) v += Mod::LS(r, c) * ek[c];
+        b1[r] = v;
+        zb[r][p] = v;
+      }
+#pragma unroll
+      for (int c = 0; c < D1; ++c) {
+        fx[c][p] = fxv[c];
+        fxk[c * MP + k] = fxv[c];
+      }
+      hz0[p] = Mod::GZERO ? Mod::hz(b1) : 0.f;
+    }
+    __syncwarp();
+    if (lane < L) {  // draw m from the mixture: a component by qbar, then the Gaussian
+      const int m = lane;
+      const int jm = sys_local_pick(cum, M, cum[M - 1], 1, 0,
+                                    philox_rk(ctr(a.t, (uint32_t)i, P_LA_J, (uint32_t)m, 0u), rk).x);
+      if (a.dbg_j) a.dbg_j[i * L + m] = jm;
+      float e1[D1], xb[D1];
+      normals_rk<D1>(rk, a.t, (uint32_t)i, P_LA_X, (uint32_t)m, e1);
+#pragma unroll
+      for (int r = 0; r < D1; ++r) {
+        float v = fxk[r * MP + jm];
+#pragma unroll
+        for (int c = 0; c < D1; ++c)
+          if (c <= r) v += Mod::Lqx(r, c) * e1[c];
+        xb[r] = v;
+        xbs[m * D1 + r] = v;
+        a.xbb_new[((long long)i * L + m) * D1 + r] = v;
+      }
+      hxs[m] = Mod::hx(xb);
+    }
+    __syncwarp();
+    // the L x M pairs: alpha = lq_k + log p(xbb_m | x, z_k), zhat = base_k + G (xbb_m - f_x,k),
+    // ell = log p(y_t | xbb_m, zhat), in log2 units (particles past M weigh nothing: lq = -inf)
+    const float y0 = a.y_cur[0];
+#pragma unroll 2
+    for (int m = 0; m < L; ++m) {
+      float xb[D1], E1[PPL], E2[PPL], zh[D2][PPL];
+#pragma unroll
+      for (int c = 0; c < D1; ++c) xb[c] = xbs[m * D1 + c];
+      const float hxm = hxs[m];
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) {
+        float r[D1], z1[D2];
+#pragma unroll
+        for (int c = 0; c < D1; ++c) r[c] = xb[c] - fx[c][p];
+        const float al = lqk[p] + nl_quad_x<Mod>(r);
+        float hzv = hz0[p];
+#pragma unroll
+        for (int q = 0; q < D2; ++q) {
+          float v = zb[q][p];
+          if (!Mod::GZERO) {
+#pragma unroll
+            for (int c = 0; c < D1; ++c) v += Mod::G(q, c) * r[c];
+          }
+          z1[q] = v;
+          zh[q][p] = v;
+        }
+        if (!Mod::GZERO) hzv = Mod::hz(z1);
+        const float res = (y0 - hxm - hzv) * Mod::LrInv(0, 0);
+        E1[p] = (al + Mod::lognorm_y - 0.5f * res * res) * LOG2E;
+        E2[p] = al * LOG2E;
+      }
+      float m1 = E1[0], m2 = E2[0];
+#pragma unroll
+      for (int p = 1; p < PPL; ++p) {
+        m1 = fmaxf(m1, E1[p]);
+        m2 = fmaxf(m2, E2[p]);
+      }
+      m1 = warp_max_redux(m1);
+      m2 = warp_max_redux(m2);
+      float s1 = 0.f, s2 = 0.f, za[D2];
+#pragma unroll
+      for (int c = 0; c < D2; ++c) za[c] = 0.f;
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) {
+        if (lane + 32 * p < M) {
+          const float e = exp2_t(E1[p] - m1);
+          s1 += e;
+          s2 += exp2_t(E2[p] - m2);
+#pragma unroll
+          for (int c = 0; c < D2; ++c) za[c] += e * zh[c][p];
+        }
+      }
+      part[(2 * m) * PART_STRIDE + lane] = s1;
+      part[(2 * m + 1) * PART_STRIDE + lane] = s2;
+#pragma unroll
+      for (int c = 0; c < D2; ++c) part[(2 * L + m * D2 + c) * PART_STRIDE + lane] = za[c];
+      if (lane == 0) {
+        rowm[2 * m] = m1;
+        rowm[2 * m + 1] = m2;
+      }
+    }
+    __syncwarp();
+    // a lane a row: the sum of its 32 partials as the butterfly over the lanes adds them
+    for (int r = lane; r < (2 + D2) * L; r += 32) {
+      float v[32];
+      vld<float, 32>(part + r * PART_STRIDE, v);
+      const float t = tree_sum<float, 32>(v);
+      part[r * PART_STRIDE] = r < 2 * L ? (rowm[r] + log2f(t)) * (float)LN2_D : t;  // natural-log units
+      if (r < 2 * L && !(r & 1)) part[r * PART_STRIDE + 1] = t;
+    }
+    __syncwarp();
+    {  // per-draw weights, the outer weight and the filtered mean (L <= 32)
+      const float lwm = lane < L ? part[2 * lane * PART_STRIDE] - part[(2 * lane + 1) * PART_STRIDE] : NEG;
+      if (lane < L) a.lwh_new[i * L + lane] = lwm;
+      const float mx = warp_max_redux(lwm);
+      const float p = lane < L ? expf(lwm - mx) : 0.f;
+      const float ps = warp_sum(p);
+#pragma unroll
+      for (int c = 0; c < D1; ++c) {
+        const float v = warp_sum(lane < L ? p * xbs[lane * D1 + c] : 0.f) / ps;
+        if (lane == 0) a.xm[c * N + i] = v;
+      }
+#pragma unroll
+      for (int c = 0; c < D2; ++c) {
+        const float zr = lane < L ? part[(2 * L + lane * D2 + c) * PART_STRIDE] / part[2 * lane * PART_STRIDE + 1] : 0.f;
+        const float v = warp_sum(lane < L ? p * zr : 0.f) / ps;
+        if (lane == 0) a.zm[c * N + i] = v;
+      }
+      if (lane == 0) {
+        const float lwi = mx + logf(ps) - a.logL;
+        a.lw[i] = lwi;
+        if (lwi != lwi) atomicOr(a.err, ERR_NUMERIC);
+        const unsigned long long key = order_key(lwi);
+        if (lwi == lwi && key > *(volatile unsigned long long*)a.lwmax_key) atomicMax(a.lwmax_key, key);
+      }
+    }
+    __syncwarp();  // the group's arrays are free for the next group
+  }
+}
+
 // The bootstrap particle filter for these models: one thread a particle.
 template <class Mod>
 __global__ void __launch_bounds__(256) nl_pf_kernel(const __grid_constant__ NLArgs a) {
@@ -746,6 +1132,28 @@ struct PaperVariant {
     tt[0] = v[0];
     tt[1] = Mod::NT > 1 ? v[Mod::NT > 1 ? 1 : 0] : 0.f;
   }
+  // one warp a group: where a group's rows are whole 16-byte units (bulk copies) and M <= 256
+  template <int PPL>
+  static dpf_status step_warp(Ctx& x, const NLArgs& a) {
+    auto k = nl_step_warp_kernel<Mod, PPL>;
+    const NLWarp<D1, D2> o(x.M, x.L, x.xp, PPL);
+    const size_t wb = 4 * (size_t)o.total;
+    if (x.grid_step == 0) {  // as many CTAs as fit on the device at once
+      int nb = 0, dev = 0, nsm = 0;
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(wb * WARPS_PER_CTA));
+      if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, WARPS_PER_CTA * 32, wb * WARPS_PER_CTA);
+      if (e == cudaSuccess) e = cudaGetDevice(&dev);
+      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+      if (e != cudaSuccess) return cuda_error(e, "paper-model step occupancy");
+      x.grid_step = (nb > 0 ? nb : 1) * nsm;
+    }
+    const int nw = x.N <= FEW_GROUPS ? 1 : WARPS_PER_CTA;
+    const long long want = (x.N + nw - 1) / nw;
+    const unsigned grid = (unsigned)(nw == 1 ? want : std::min<long long>(want, x.grid_step));
+    k<<<grid, 32 * nw, wb * nw, x.stream>>>(a, o);
+    return cuda_error(cudaGetLastError(), "paper-model step launch");
+  }
   static dpf_status step(Ctx& x, int) {
     const long long t = x.t + 1;
     const int so = (int)((t + 2) % 2), sn = (int)((t + 1) % 2);
@@ -785,6 +1193,12 @@ struct PaperVariant {
     a.first = first ? 1 : 0;
     a.dbg_b = x.debug ? x.dbg_b : nullptr;
     a.dbg_j = x.debug ? x.dbg_j : nullptr;
+    if (VariantImpl<float, D1, D2, DY, 1>::warp_path(x.M, x.L)) {
+      if (x.M <= 32) return step_warp<1>(x, a);
+      if (x.M <= 64) return step_warp<2>(x, a);
+      if (x.M <= 128) return step_warp<4>(x, a);
+      return step_warp<8>(x, a);
+    }
     const int big = x.M > x.L ? x.M : x.L;
     const int nt = (big < 32 ? 32 : (big + 31) / 32 * 32);
     const size_t sm = nl_smem_bytes(D1, D2, x.M, x.L);
