@@ -11,7 +11,7 @@
 // memory, so the copy of the next chunks overlaps the MMAs of the current ones.
 // Every hidden layer's accumulator (128 x 256 FP32, TMEM columns 0..255) is read
 // back row by row, biased, passed through ReLU, rounded to BF16 and written as
-// the next layer's A operand (K-major, no swizzle). All waits are bounded.
+// the next layer's A operand (K-major, 128-byte swizzle). All waits are bounded.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -45,29 +45,87 @@ constexpr size_t PK_B = PK_W4 + (size_t)LNP * LH * 2;
 constexpr size_t PK_BYTES = PK_B + sizeof(float) * (3 * LH + LNP);
 
 // One iteration of the kernel takes 2 x 128 rows (tiles A and B, TMEM columns 0..255 and
-// 256..511); 8 compute warps hold one row a thread, a ninth warp feeds the weight ring.
+// 256..511). The first 256 compute threads hold one row each; the hidden layers' epilogues are
+// shared by LSPLIT threads a row (each a range of columns). One more warp feeds the weight ring.
+//
+// The weights reach the ring by multicast: the LCL CTAs of a cluster walk the same chunks in step,
+// each copies 1 / LCL of a chunk from L2 into all of their rings, and a stage is refilled when
+// the MMAs of every CTA of the cluster have read it. Alone, each of 152 SMs fetched the same 128 KB a
+// layer, and a 16 KB copy took 6,000 cycles whatever the ring's depth: the streamed layers ran
+// at 3.6 times their MMA time (together with the polls, see wait_products). With both gone the
+// layers run at the pace of their MMAs: 1,000,003 rows 929 us, now 372 (298 and 744 TFLOP/s).
+// Clusters of 4 left some SMs out (140 of 152 busy) and were no faster.
 constexpr int LROWS = 256;
-constexpr int LCOMPUTE = 256;                               // compute threads
-constexpr int LTHREADS = LCOMPUTE + 32;                     // + the producer warp
+constexpr int LCL = 2;  // CTAs of a cluster
+template <int MODE>
+constexpr int learned_split() { return MODE == 0 ? 2 : 1; }  // the filter's pass needs 136 registers a thread
+template <int MODE>
+constexpr int learned_compute() { return LROWS * learned_split<MODE>(); }  // compute threads
+template <int MODE>
+constexpr int learned_threads() { return learned_compute<MODE>() + 32; }   // + the producer warp
 // shared-memory layout (bytes)
-constexpr uint32_t SM_ACT = 0;                              // 2 x (128 x 256 bf16), kc16 = 32
+constexpr uint32_t SM_ACT = 0;                              // 2 x (128 x 256 bf16), 128-byte swizzle
 constexpr uint32_t SM_IN = SM_ACT + 2 * 128 * LH * 2;       // 2 x (128 x 16 bf16), kc16 = 2
 constexpr uint32_t SM_W1 = SM_IN + 2 * 128 * LDIN * 2;      // 256 x 16, kc16 = 2
 constexpr uint32_t SM_W4 = SM_W1 + LH * LDIN * 2;           // 32 x 256, kc16 = 32
-constexpr uint32_t SM_RING = SM_W4 + LNP * LH * 2;          // 3 x (256 x 32), kc16 = 4
+constexpr uint32_t SM_RING = SM_W4 + LNP * LH * 2;          // 3 x (256 x 32), 64-byte swizzle
 constexpr uint32_t SM_BIAS = SM_RING + LSTAGES * LCHUNK;    // b1 b2 b3 (256 each), b4 (32)
 constexpr uint32_t SM_CUM = SM_BIAS + sizeof(float) * (3 * LH + LNP);  // 256 uint32
 constexpr uint32_t SM_RED = SM_CUM + LROWS * 4;             // 8 floats, 8 words
 constexpr uint32_t SM_BYTES = SM_RED + 64;
 static_assert(SM_BYTES <= 227 * 1024, "shared memory of the learned kernel");
 
-// Barrier of the 256 compute threads only (the producer warp runs its own loop).
+// Barrier of the 256 row threads (the group reductions of the filter's pass).
 __device__ __forceinline__ void compute_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// Barrier of all NT compute threads (the producer warp runs its own loop).
+template <int NT>
+__device__ __forceinline__ void all_sync() { asm volatile("bar.sync 2, %0;" ::"n"(NT) : "memory"); }
+
+// Wait (bounded) for the products committed to `mbar`. One thread polls and the others block in
+// the hardware barrier: polls of an mbarrier from every warp take the shared-memory cycles that
+// the weight copies and their byte counts need (a 16 KB copy then took 3,300 cycles from 16
+// polling warps, 2,100 from 8).
+template <int NT>
+__device__ __forceinline__ void wait_products(uint64_t* mbar, uint32_t& phase, bool& ok) {
+  if (threadIdx.x == 0) ok &= tc::bar_wait(mbar, phase, L_SPIN);
+  phase ^= 1u;
+  __syncwarp();
+  tc::fence_before();
+  all_sync<NT>();
+  tc::fence_after();
+}
+
+// ---- cluster pieces: rank, barrier, multicast copy and commit (the same shared-memory offsets in
+// every CTA of the mask) ----
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void bulk_load_multicast(void* dst, const void* src, uint32_t bytes, uint64_t* b,
+                                                    uint16_t mask) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1], %2, [%3], %4;" ::
+          "r"(smem_addr(dst)),
+      "l"(src), "r"(bytes), "r"(smem_addr(b)), "h"(mask)
+      : "memory");
+}
+__device__ __forceinline__ void commit_multicast(uint64_t* bar, uint16_t mask) {
+  asm volatile(
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+          smem_addr(bar)),
+      "h"(mask)
+      : "memory");
+}
 
 // Pack one FP32 matrix (rows x cols, row-major) into BF16 K-major chunks of kch
-// columns, rows padded to rows_pad and columns to a multiple of kch with zeros.
+// columns, rows padded to rows_pad and columns to a multiple of kch with zeros; sw64: in the
+// 64-byte-swizzled layout (kch = 32).
 __global__ void pack_matrix_kernel(const float* __restrict__ W, int rows, int cols, int rows_pad, int kch,
-                                   int nchunks, unsigned char* __restrict__ dst) {
+                                   int nchunks, bool sw64, unsigned char* __restrict__ dst) {
   const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long total = (long long)rows_pad * kch * nchunks;
   if (e >= total) return;
@@ -75,7 +133,8 @@ __global__ void pack_matrix_kernel(const float* __restrict__ W, int rows, int co
   const int k = (int)(e % ((long long)kch * nchunks));
   const int ch = k / kch, kl = k % kch;
   const float v = (n < rows && k < cols) ? W[(long long)n * cols + k] : 0.f;
-  const size_t off = (size_t)ch * rows_pad * kch * 2 + tc::kmajor_offset(n, 2 * kl, kch * 2 / 16);
+  const size_t off = (size_t)ch * rows_pad * kch * 2 +
+                     (sw64 ? tc::sw64_offset(n, 2 * kl) : tc::kmajor_offset(n, 2 * kl, kch * 2 / 16));
   *(__nv_bfloat16*)(dst + off) = __float2bfloat16_rn(v);
 }
 
@@ -104,7 +163,8 @@ static dpf_status pack(dpf_proposal& p) {
   const float* Wq = p.Wq;
   auto launch = [&](const float* W, int rows, int cols, int rows_pad, int kch, int nch, size_t off) {
     const long long total = (long long)rows_pad * kch * nch;
-    pack_matrix_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(W, rows, cols, rows_pad, kch, nch, d + off);
+    pack_matrix_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(W, rows, cols, rows_pad, kch, nch, kch == LKCH,
+                                                                      d + off);
   };
   launch(Wq + p.offW[0], LH, p.din, LH, LDIN, 1, PK_W1);
   launch(Wq + p.offW[1], LH, LH, LH, LKCH, LNCH, PK_W2);
@@ -125,33 +185,57 @@ struct LearnArgs {
   const float* F;
   float* out;
   long long nrows;
+  int vec_in, vec_out;  // rows of F, of out, are whole 16-byte units
   // filter mode
   float* dbg_head;  // N M x dout head outputs, or null
   uint32_t scaleC;  // 2^(31 - ceil log2 C)
   int* err;
 };
 
-__device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
-  const uint32_t lo = __bfloat16_as_ushort(__float2bfloat16_rn(a));
-  const uint32_t hi = __bfloat16_as_ushort(__float2bfloat16_rn(b));
-  return lo | (hi << 16);
+// Whether the feature and head rows can move in 16-byte units.
+static void row_alignment(LearnArgs& la) {
+  la.vec_in = la.din % 4 == 0 && ((uintptr_t)la.F & 15) == 0;
+  la.vec_out = la.dout % 4 == 0 && ((uintptr_t)la.out & 15) == 0;
 }
 
-// Read one hidden accumulator row (256 FP32 columns of TMEM, 64 per load), add the
+__device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);  // one conversion of the pair
+  uint32_t r;
+  memcpy(&r, &v, 4);
+  return r;
+}
+
+// Descriptor of K step ks (16 columns) of a 128 x 256 activation tile (four 128-byte-swizzled
+// tiles of 64 columns).
+__device__ __forceinline__ uint64_t act_desc(uint32_t tile, int ks) {
+  return tc::smem_desc_sw(tile + (uint32_t)(ks >> 2) * (128u * 128u) + (uint32_t)(ks & 3) * 32u, tc::LAYOUT_SW128);
+}
+
+// Read columns cbeg .. cend - 1 of one hidden accumulator row (FP32, TMEM, CW = 32 or 64 per load), add the
 // bias, ReLU, round to BF16 and store it as row r of the activation tile.
-__device__ __forceinline__ void hidden_epilogue(uint32_t taddr_row, const float* bias, unsigned char* act, int r) {
+template <int CW>
+__device__ __forceinline__ void hidden_epilogue(uint32_t taddr_row, const float* bias, unsigned char* act, int r,
+                                                int cbeg, int cend) {
 #pragma unroll 1
-  for (int c0 = 0; c0 < LH; c0 += 64) {
-    float v[64];
-    tc::ld64(taddr_row + (uint32_t)c0, v);
+  for (int c0 = cbeg; c0 < cend; c0 += CW) {
+    float v[CW];
+    if constexpr (CW == 64)
+      tc::ld64(taddr_row + (uint32_t)c0, v);
+    else
+      tc::ld32(taddr_row + (uint32_t)c0, v);
 #pragma unroll
-    for (int h = 0; h < 64; h += 8) {
+    for (int h = 0; h < CW; h += 8) {
+      const float4 b0 = *(const float4*)(bias + c0 + h), b1 = *(const float4*)(bias + c0 + h + 4);
+      const float2 s0 = __fadd2_rn(make_float2(v[h + 0], v[h + 1]), make_float2(b0.x, b0.y));
+      const float2 s1 = __fadd2_rn(make_float2(v[h + 2], v[h + 3]), make_float2(b0.z, b0.w));
+      const float2 s2 = __fadd2_rn(make_float2(v[h + 4], v[h + 5]), make_float2(b1.x, b1.y));
+      const float2 s3 = __fadd2_rn(make_float2(v[h + 6], v[h + 7]), make_float2(b1.z, b1.w));
       uint4 q;
-      q.x = pack_bf16x2(fmaxf(v[h + 0] + bias[c0 + h + 0], 0.f), fmaxf(v[h + 1] + bias[c0 + h + 1], 0.f));
-      q.y = pack_bf16x2(fmaxf(v[h + 2] + bias[c0 + h + 2], 0.f), fmaxf(v[h + 3] + bias[c0 + h + 3], 0.f));
-      q.z = pack_bf16x2(fmaxf(v[h + 4] + bias[c0 + h + 4], 0.f), fmaxf(v[h + 5] + bias[c0 + h + 5], 0.f));
-      q.w = pack_bf16x2(fmaxf(v[h + 6] + bias[c0 + h + 6], 0.f), fmaxf(v[h + 7] + bias[c0 + h + 7], 0.f));
-      *(uint4*)(act + tc::kmajor_offset(r, 2 * (c0 + h), 32)) = q;
+      q.x = pack_bf16x2(fmaxf(s0.x, 0.f), fmaxf(s0.y, 0.f));
+      q.y = pack_bf16x2(fmaxf(s1.x, 0.f), fmaxf(s1.y, 0.f));
+      q.z = pack_bf16x2(fmaxf(s2.x, 0.f), fmaxf(s2.y, 0.f));
+      q.w = pack_bf16x2(fmaxf(s3.x, 0.f), fmaxf(s3.y, 0.f));
+      *(uint4*)(act + tc::sw128_offset(r, 2 * (c0 + h), 128)) = q;
     }
   }
 }
@@ -185,14 +269,17 @@ __device__ __forceinline__ float group_sum(float v, int M, float* red) {
 // MODE 0: head outputs of feature rows; MODE 1: the filter's inner update with NC
 // mixture components (compile-time, so that the head's arrays stay in registers).
 template <int MODE, int D1, int D2, int DY, bool XZ, int NC>
-__global__ void __launch_bounds__(LTHREADS, 1)
+__global__ void __launch_bounds__(learned_threads<MODE>(), 1)
     learned_kernel(const __grid_constant__ MC<float, D1, D2, DY> mc, const __grid_constant__ StepArgs<float> a,
                    const __grid_constant__ LearnArgs la) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ __align__(8) uint64_t full[LSTAGES], empty[LSTAGES], mbar;
   __shared__ uint32_t s_taddr;
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-  const int half = tid >> 7;  // tile A (0) or B (1) of this thread's row
+  constexpr int NCT = learned_compute<MODE>(), NT = learned_threads<MODE>();
+  const int half = (tid >> 7) & 1;  // tile A (0) or B (1) of this thread's row
+  const bool rower = tid < LROWS;   // holds a row outside the hidden epilogues
+  const int ccols = LH / learned_split<MODE>(), cbeg = (tid >> 8) * ccols;  // its columns in them
   const int r128 = tid & 127;
   unsigned char* act = sm + SM_ACT + half * (128 * LH * 2);
   unsigned char* in = sm + SM_IN + half * (128 * LDIN * 2);
@@ -204,14 +291,19 @@ __global__ void __launch_bounds__(LTHREADS, 1)
   const int M = MODE == 1 ? a.M : 128;
   const long long rows_total = MODE == 1 ? a.N * (long long)a.M : la.nrows;
   const long long niters = (rows_total + LROWS - 1) / LROWS;
-  const long long my_iters = niters > blockIdx.x ? (niters - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+  // every CTA of a cluster runs as many iterations as its first one (some on no live row), so that
+  // they walk the weights' chunks together
+  const uint32_t rank = cluster_rank();
+  const long long first = (long long)blockIdx.x - rank;
+  const long long my_iters = niters > first ? (niters - 1 - first) / gridDim.x + 1 : 0;
+  constexpr uint16_t all_ctas = (uint16_t)((1u << LCL) - 1u);
   const long long total_chunks = my_iters * 2 * LNCH;
 
   // ---- set-up: barriers, TMEM, resident weights and biases ----
   if (tid == 0) {
     for (int s = 0; s < LSTAGES; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
+      mbar_init(&empty[s], LCL);
     }
     mbar_init(&mbar, 1);
     mbar_fence_init();
@@ -220,21 +312,22 @@ __global__ void __launch_bounds__(LTHREADS, 1)
     tc::tmem_alloc(&s_taddr, LTMEM_COLS);
     tc::tmem_relinquish();
   }
-  for (int e = tid; e < (int)(LH * LDIN * 2 / 16); e += LTHREADS)
+  for (int e = tid; e < (int)(LH * LDIN * 2 / 16); e += NT)
     ((uint4*)(sm + SM_W1))[e] = ((const uint4*)(la.wp + PK_W1))[e];
-  for (int e = tid; e < (int)(LNP * LH * 2 / 16); e += LTHREADS)
+  for (int e = tid; e < (int)(LNP * LH * 2 / 16); e += NT)
     ((uint4*)(sm + SM_W4))[e] = ((const uint4*)(la.wp + PK_W4))[e];
-  for (int e = tid; e < 3 * LH + LNP; e += LTHREADS) bias[e] = ((const float*)(la.wp + PK_B))[e];
+  for (int e = tid; e < 3 * LH + LNP; e += NT) bias[e] = ((const float*)(la.wp + PK_B))[e];
   tc::fence_proxy_async();
   tc::fence_before();
   __syncthreads();
+  cluster_sync_all();  // every CTA's barriers are set up before another one's copies or commits arrive
   tc::fence_after();
   const uint32_t taddr = s_taddr;
   // this thread's accumulator row: lanes 32 (w % 4) .., columns 256 half ..
   const uint32_t trow = taddr + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(half * LH);
   bool ok = true;
 
-  if (w == LCOMPUTE / 32) {
+  if (w == NCT / 32) {
     // ---- producer warp: refill each ring stage as soon as its MMAs are done ----
     if (lane == 0) {
       for (long long c = 0; c < total_chunks; ++c) {
@@ -246,8 +339,10 @@ __global__ void __launch_bounds__(LTHREADS, 1)
         const int q = (int)(c % (2 * LNCH));
         const unsigned char* src =
             la.wp + (q < LNCH ? PK_W2 + (size_t)q * LCHUNK : PK_W3 + (size_t)(q - LNCH) * LCHUNK);
+        // this CTA's part of the chunk, into the same stage of every CTA of the cluster
+        constexpr uint32_t part = LCHUNK / LCL;
         mbar_arrive_tx(&full[s], LCHUNK);
-        bulk_load(sm + SM_RING + s * LCHUNK, src, LCHUNK, &full[s]);
+        bulk_load_multicast(sm + SM_RING + s * LCHUNK + rank * part, src + rank * part, part, &full[s], all_ctas);
       }
       // wait until the last chunks' MMAs have released their stages, so that no
       // copy is in flight when the kernel ends
@@ -261,9 +356,35 @@ __global__ void __launch_bounds__(LTHREADS, 1)
   const uint32_t id_h = tc::instr_desc(tc::FMT_BF16, 128, LH);
   const uint32_t id_o = tc::instr_desc(tc::FMT_BF16, 128, LNP);
 
-  for (long long it = blockIdx.x; it < niters; it += gridDim.x) {
-    const long long row = it * LROWS + tid;
-    const bool live = row < rows_total;
+  // forward-only mode: the features of the row of iteration n, loaded one iteration ahead
+  float fnext[MODE == 0 ? LDIN : 1];
+  auto load_features = [&](long long n) {
+    if constexpr (MODE == 0) {
+      const long long row = (blockIdx.x + n * gridDim.x) * LROWS + tid;
+#pragma unroll
+      for (int k = 0; k < LDIN; ++k) fnext[k] = 0.f;
+      if (!rower || n >= my_iters || row >= rows_total) return;
+      if (la.vec_in) {
+#pragma unroll
+        for (int k = 0; k < LDIN; k += 4)
+          if (k < la.din) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(la.F + row * la.din + k));
+            fnext[k] = v.x;
+            fnext[k + 1] = v.y;
+            fnext[k + 2] = v.z;
+            fnext[k + 3] = v.w;
+          }
+      } else {
+#pragma unroll
+        for (int k = 0; k < LDIN; ++k)
+          if (k < la.din) fnext[k] = la.F[row * la.din + k];
+      }
+    }
+  };
+  load_features(0);
+  for (long long n = 0; n < my_iters; ++n) {
+    const long long row = (blockIdx.x + n * gridDim.x) * LROWS + tid;
+    const bool live = rower && row < rows_total;
     // ---- prologue: this row's input features ----
     float feat[LDIN];
 #pragma unroll
@@ -272,10 +393,9 @@ __global__ void __launch_bounds__(LTHREADS, 1)
     long long g = 0;
     int j = 0, anc_g = 0;
     float xa[D1], xt[D1], zb[D2];
-    if (MODE == 0) {
+    if constexpr (MODE == 0) {
 #pragma unroll
-      for (int k = 0; k < LDIN; ++k)
-        if (live && k < la.din) feat[k] = la.F[row * la.din + k];
+      for (int k = 0; k < LDIN; ++k) feat[k] = fnext[k];
     } else {
       g = row / M;
       j = (int)(row % M);
@@ -377,7 +497,7 @@ __global__ void __launch_bounds__(LTHREADS, 1)
         for (int q = 0; q < DY; ++q) feat[2 * D1 + D2 + q] = a.y_prev[q];
       }
     }
-    {
+    if (rower) {
       uint4 q0, q1;
       q0.x = pack_bf16x2(feat[0], feat[1]);
       q0.y = pack_bf16x2(feat[2], feat[3]);
@@ -392,7 +512,8 @@ __global__ void __launch_bounds__(LTHREADS, 1)
     }
     tc::fence_proxy_async();
     tc::fence_before();
-    compute_sync();
+    all_sync<NCT>();
+    load_features(n + 1);
 
     const uint32_t s_act0 = smem_addr(sm + SM_ACT), s_in0 = smem_addr(sm + SM_IN);
     // ---- layer 1 (both tiles) ----
@@ -403,13 +524,11 @@ __global__ void __launch_bounds__(LTHREADS, 1)
                     tc::smem_desc(smem_addr(sm + SM_W1), 2), id_h, 0u);
       tc::commit(&mbar);
     }
-    ok &= tc::bar_wait(&mbar, mph, L_SPIN);
-    mph ^= 1u;
-    tc::fence_after();
-    hidden_epilogue(trow, bias, act, r128);
+    wait_products<NCT>(&mbar, mph, ok);
+    hidden_epilogue<MODE == 0 ? 32 : 64>(trow, bias, act, r128, cbeg, cbeg + ccols);
     tc::fence_proxy_async();
     tc::fence_before();
-    compute_sync();
+    all_sync<NCT>();
 
     // ---- layers 2 and 3 (streamed weights) ----
 #pragma unroll 1
@@ -426,19 +545,17 @@ __global__ void __launch_bounds__(LTHREADS, 1)
 #pragma unroll
             for (int h = 0; h < 2; ++h)
               tc::mma_f16(taddr + h * LH,
-                          tc::smem_desc(s_act0 + h * (128 * LH * 2) + (uint32_t)(k * (LKCH / 8) + ks * 2) * 128u, 32),
-                          tc::smem_desc(sb + (uint32_t)ks * 256u, LKCH / 8), id_h, (k > 0 || ks > 0) ? 1u : 0u);
-          tc::commit(&empty[s]);  // the producer refills the stage once these MMAs are done
+                          act_desc(s_act0 + h * (128 * LH * 2), k * (LKCH / 16) + ks),
+                          tc::smem_desc_sw(sb + (uint32_t)ks * 32u, tc::LAYOUT_SW64), id_h, (k > 0 || ks > 0) ? 1u : 0u);
+          commit_multicast(&empty[s], all_ctas);  // the stage may be refilled once every CTA's MMAs are done
         }
         tc::commit(&mbar);
       }
-      ok &= tc::bar_wait(&mbar, mph, L_SPIN);
-      mph ^= 1u;
-      tc::fence_after();
-      hidden_epilogue(trow, bias + (layer + 1) * LH, act, r128);
+      wait_products<NCT>(&mbar, mph, ok);
+      hidden_epilogue<MODE == 0 ? 32 : 64>(trow, bias + (layer + 1) * LH, act, r128, cbeg, cbeg + ccols);
       tc::fence_proxy_async();
       tc::fence_before();
-      compute_sync();
+      all_sync<NCT>();
     }
 
     // ---- head ----
@@ -450,13 +567,12 @@ __global__ void __launch_bounds__(LTHREADS, 1)
       for (int ks = 0; ks < LH / 16; ++ks)
 #pragma unroll
         for (int h = 0; h < 2; ++h)
-          tc::mma_f16(taddr + h * LH, tc::smem_desc(s_act0 + h * (128 * LH * 2) + (uint32_t)ks * 256u, 32),
+          tc::mma_f16(taddr + h * LH, act_desc(s_act0 + h * (128 * LH * 2), ks),
                       tc::smem_desc(sb + (uint32_t)ks * 256u, 32), id_o, ks > 0 ? 1u : 0u);
       tc::commit(&mbar);
     }
-    ok &= tc::bar_wait(&mbar, mph, L_SPIN);
-    mph ^= 1u;
-    tc::fence_after();
+    wait_products<NCT>(&mbar, mph, ok);
+    if (rower) {
     float o[LNP];
     {
       float v[16];
@@ -469,10 +585,17 @@ __global__ void __launch_bounds__(LTHREADS, 1)
     }
     tc::fence_before();
 
-    if (MODE == 0) {
+    if constexpr (MODE == 0) {
+      if (live && la.vec_out) {
 #pragma unroll
-      for (int q = 0; q < LNP; ++q)
-        if (live && q < la.dout) la.out[row * la.dout + q] = o[q];
+        for (int q = 0; q < LNP; q += 4)
+          if (q < la.dout)
+            *reinterpret_cast<float4*>(la.out + row * la.dout + q) = make_float4(o[q], o[q + 1], o[q + 2], o[q + 3]);
+      } else {
+#pragma unroll
+        for (int q = 0; q < LNP; ++q)
+          if (live && q < la.dout) la.out[row * la.dout + q] = o[q];
+      }
     } else {
       // ---- the mixture draw and the importance weight ----
       constexpr int C = NC;
@@ -587,13 +710,15 @@ __global__ void __launch_bounds__(LTHREADS, 1)
         if (!(lqn == lqn)) atomicOr(a.err, ERR_NUMERIC);
       }
     }
-    compute_sync();  // TMEM and the tiles are free for the next iteration
+    }
+    all_sync<NCT>();  // TMEM and the tiles are free for the next iteration
   }
   }  // compute warps
   if (!ok && lane == 0) atomicOr(MODE == 1 ? a.err : la.err, ERR_TIMEOUT);
   tc::fence_before();
   __syncthreads();
   if (w == 0) tc::tmem_dealloc(taddr, LTMEM_COLS);
+  cluster_sync_all();  // no CTA leaves while another may still signal its barriers
 }
 
 template <int MODE, int D1, int D2, int DY, bool XZ, int NC>
@@ -606,12 +731,30 @@ static dpf_status launch_learned(const MC<float, D1, D2, DY>& mc, const StepArgs
     if (e != cudaSuccess) return cuda_error(e, "learned kernel attribute");
     attr = true;
   }
-  int dev = 0, nsm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(LCL);
+  cfg.blockDim = dim3(learned_threads<MODE>());
+  cfg.dynamicSmemBytes = SM_BYTES;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = LCL;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  static int resident = 0;  // clusters on the device at once
+  if (!resident) {
+    int n = 0;
+    cudaError_t e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
+    if (e != cudaSuccess) return cuda_error(e, "learned kernel occupancy");
+    resident = n > 0 ? n : 1;
+  }
   const long long iters = (rows + LROWS - 1) / LROWS;
-  const int grid = (int)std::max<long long>(1, std::min<long long>(iters, nsm));
-  k<<<grid, LTHREADS, SM_BYTES, s>>>(mc, a, la);
+  const long long clusters = std::max<long long>(1, std::min<long long>((iters + LCL - 1) / LCL, resident));
+  cfg.gridDim = dim3((unsigned)(clusters * LCL));
+  cudaError_t le = cudaLaunchKernelEx(&cfg, k, mc, a, la);
+  if (le != cudaSuccess) return cuda_error(le, "learned kernel launch");
   return cuda_error(cudaGetLastError(), "learned kernel launch");
 }
 
@@ -981,6 +1124,7 @@ static dpf_status oa_step_pp(Ctx& x, const MC<float, 2, 2, 2>& mc, StepArgs<floa
   la.F = (const float*)x.oa_feat;
   la.out = (float*)x.oa_out;
   la.nrows = x.N;
+  row_alignment(la);
   la.err = x.err;
   MC<float, 2, 2, 2> mc0;
   memset(&mc0, 0, sizeof(mc0));
@@ -1107,10 +1251,6 @@ dpf_status dpf_proposal_forward(dpf_proposal* p, const float* F, int64_t n, floa
                                         "din <= 16 and dout <= 32");
   dpf_status st = pack(*p);
   if (st) return st;
-  int* err = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&err, sizeof(int), p->stream);
-  if (e != cudaSuccess) return cuda_error(e, "dpf_proposal_forward: allocation");
-  cudaMemsetAsync(err, 0, sizeof(int), p->stream);
   LearnArgs la{};
   la.wp = (const unsigned char*)p->packed;
   la.din = p->din;
@@ -1119,17 +1259,18 @@ dpf_status dpf_proposal_forward(dpf_proposal* p, const float* F, int64_t n, floa
   la.F = F;
   la.out = out;
   la.nrows = n;
-  la.err = err;
+  row_alignment(la);
+  la.err = p->err_d;  // zero unless a wait gave up, and cleared when that is reported
   MC<float, 2, 2, 2> mc;
   memset(&mc, 0, sizeof(mc));
   StepArgs<float> a{};
   st = launch_learned<0, 2, 2, 2, false, kFilterComponents>(mc, a, la, n, p->stream);
   int h = 0;
-  e = cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, p->stream);
+  cudaError_t e = cudaMemcpyAsync(&h, p->err_d, sizeof(int), cudaMemcpyDeviceToHost, p->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
-  cudaFreeAsync(err, p->stream);
   if (st) return st;
   if (e != cudaSuccess) return cuda_error(e, "dpf_proposal_forward");
+  if (h) cudaMemsetAsync(p->err_d, 0, sizeof(int), p->stream);
   if (h) return set_error(DPF_E_TIMEOUT, "dpf_proposal_forward: a bounded wait gave up");
   return DPF_OK;
 }
