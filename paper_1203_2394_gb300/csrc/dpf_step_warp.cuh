@@ -31,6 +31,17 @@ constexpr int PART_STRIDE = 36;
 template <int PPL, int D2>
 constexpr int warp_min_blocks() { return PPL * D2 >= 48 ? 2 : 4; }
 
+// Whether the propagation's normals are drawn in a rolled loop (through shared memory) rather than
+// unrolled: PPL D2 / 4 copies of Philox and Box-Muller, 110 instructions each, leave the
+// instruction cache when they and the rest of a step are long: at lg16's PPL D2 = 112 a quarter of the
+// stalls waited for instructions. Rolled, a batch of 16 such filters went from 1854 to 1647 us a
+// step, and growth_clg10 (PPL D2 = 32) from 349 to 340; below that the unrolled form keeps its lead.
+constexpr int NOISE_CHAINS = 4;
+template <typename T, int PPL, int D2>
+constexpr bool rolled_noise() { return sizeof(T) == 4 && PPL * D2 >= 32; }
+
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
 // Per-warp shared-memory carve-up (bytes from the warp's region), on the host.
 template <typename T, int D1, int D2, int DY, bool XZ>
 inline size_t warp_geometry(int M, int L, StepArgs<T>* a, bool first = false) {
@@ -617,30 +628,61 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
 #pragma unroll
         for (int r = 0; r < D2; ++r) axpy<T, PPL>(mc.Azz[r][c], zc, zr[r]);
       }
+      // the column c of noise e (a value a particle) into z_t
+      auto add_noise = [&](int c, const T (&e)[PPL]) {
+        if (mc.diag_qz) {
+          axpy<T, PPL>(mc.Lqz[c][c], e, zr[c]);
+        } else {
+          // constant bounds (not r = c ..) so that the loop unrolls before c is known
+          // and zr stays in registers
 #pragma unroll
-      for (int b = 0; b < (D2 + 3) / 4; ++b) {
-        T e4[4][PPL];
+          for (int r = 0; r < D2; ++r)
+            if (r >= c) axpy<T, PPL>(mc.Lqz[r][c], e, zr[r]);
+        }
+      };
+      if constexpr (rolled_noise<T, PPL, D2>()) {
+        // the normals in a rolled loop over their blocks, through the stage's z rows (every gather
+        // from them is done; a lane reads back only what it wrote)
+        __syncwarp();
+        constexpr int CP = PPL < NOISE_CHAINS ? PPL : NOISE_CHAINS;  // particles side by side
+#pragma unroll 1
+        for (int q = 0; q < (D2 + 3) / 4 * (PPL / CP); ++q) {
+          const int b = q / (PPL / CP), kp = k0 + q % (PPL / CP) * CP;
+          T e4[4][CP];
 #pragma unroll
-        for (int p = 0; p < PPL; ++p) {
-          T e[4];
-          normal_block_rk(rk, a.t - 1, (uint32_t)i, P_PROP, (uint32_t)(k0 + p), b, D2 - 4 * b, e);
+          for (int p = 0; p < CP; ++p) {
+            T e[4];
+            normal_block_rk(rk, a.t - 1, (uint32_t)i, P_PROP, (uint32_t)(kp + p), b, 4, e);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) e4[j][p] = e[j];
+            for (int j = 0; j < 4; ++j) e4[j][p] = e[j];
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (act && 4 * b + j < D2) vst<T, CP>(sz + (4 * b + j) * M + kp, e4[j]);
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int c = 4 * b + j;
-          if (c < D2) {
-            if (mc.diag_qz) {
-              axpy<T, PPL>(mc.Lqz[c][c], e4[j], zr[c]);
-            } else {
-              // constant bounds (not r = c ..) so that the loop unrolls before c is known
-              // and zr stays in registers
+        for (int c = 0; c < D2; ++c) {
+          T e[PPL];
 #pragma unroll
-              for (int r = 0; r < D2; ++r)
-                if (r >= c) axpy<T, PPL>(mc.Lqz[r][c], e4[j], zr[r]);
-            }
+          for (int p = 0; p < PPL; ++p) e[p] = T(0);
+          if (act) vld<T, PPL>(sz + c * M + k0, e);
+          add_noise(c, e);
+        }
+        fence_async_smem();  // these writes come before the copies that refill the stage
+      } else {
+#pragma unroll
+        for (int b = 0; b < (D2 + 3) / 4; ++b) {
+          T e4[4][PPL];
+#pragma unroll
+          for (int p = 0; p < PPL; ++p) {
+            T e[4];
+            normal_block_rk(rk, a.t - 1, (uint32_t)i, P_PROP, (uint32_t)(k0 + p), b, D2 - 4 * b, e);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) e4[j][p] = e[j];
           }
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (4 * b + j < D2) add_noise(4 * b + j, e4[j]);
         }
       }
       T ell[PPL];
@@ -954,7 +996,7 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
       }
       if (shifted) {
         // row maxima of both exponents
-#pragma unroll 2
+#pragma unroll 1
         for (int m = 0; m < L; ++m) {
           T v[PPL];
           T pa = NEG, ps = NEG;
@@ -973,7 +1015,7 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
         reduce_rows<T, true>(part + L * PART_STRIDE, L, lane, shS);
         __syncwarp();
         // A_m relative to its maximum, added lane after lane
-#pragma unroll 2
+#pragma unroll 1
         for (int m = 0; m < L; ++m) {
           const T ha = shA[m];
           T v[PPL], pa = T(0);
@@ -998,7 +1040,7 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
 #pragma unroll
         for (int p = 0; p < PPL; ++p) B[p] = T(0);
         // S_m relative to its maximum, and beta
-#pragma unroll 2
+#pragma unroll 1
         for (int m = 0; m < L; ++m) {
           const T hs = shS[m];
           T v[PPL], ps = T(0);
