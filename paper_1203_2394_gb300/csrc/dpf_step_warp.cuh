@@ -937,7 +937,7 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
       // The x transition depends on z. v = alpha's exponent, vl = v less the y terms (log2
       // units); A_m and S_m are their row sums over k. Since pi_m / S_m is proportional to
       // 1 / A_m, beta_k = sum_m w_m e(m,k) up to normalisation, with w_m known once the A rows
-      // are summed, so the pass that sums the S rows gives beta too.
+      // are summed.
       const T tiny = sizeof(T) == 4 ? T(1e-30) : T(1e-290);
       // the rows of exponents: v alone, or vl
       auto expo = [&](int m, bool with_y, T (&v)[PPL]) {
@@ -958,6 +958,8 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
       bool shifted = sizeof(T) == 4;
       if (!shifted) {
         bool bad = false;
+        // four draws side by side: a few warps an SM hide little of an FP64 exponential's chain
+#pragma unroll 4
         for (int m = 0; m < L; ++m) {
           T v[PPL];
           expo(m, false, v);
@@ -976,6 +978,7 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
           shA[m] = T(0);
         }
         __syncwarp();
+#pragma unroll 4
         for (int m = 0; m < L; ++m) {
           T v[PPL];
           expo(m, true, v);
@@ -995,68 +998,88 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
         shifted = __any_sync(FULL, bad);
       }
       if (shifted) {
-        // row maxima of both exponents
-#pragma unroll 1
-        for (int m = 0; m < L; ++m) {
-          T v[PPL];
-          T pa = NEG, ps = NEG;
+        // One pass: a row's exponents, their maxima (a reduction instruction each), the
+        // exponentials relative to them and the lane's partial sums. e receives the S row's
+        // exponentials.
+        auto row = [&](int m, T (&e)[PPL]) {
+          T v[PPL], ha = NEG, hs = NEG, pa = T(0), ps = T(0);
           expo(m, false, v);
 #pragma unroll
-          for (int p = 0; p < PPL; ++p) pa = fmax(pa, v[p]);
+          for (int p = 0; p < PPL; ++p) {
+            e[p] = v[p];
+            ha = fmax(ha, v[p]);
+          }
 #pragma unroll
-          for (int q = 0; q < DY; ++q) sub_sq<T, PPL>(cw[m * DY + q], ngk[q], v);
+          for (int q = 0; q < DY; ++q) sub_sq<T, PPL>(cw[m * DY + q], ngk[q], e);
 #pragma unroll
-          for (int p = 0; p < PPL; ++p) ps = fmax(ps, v[p]);
-          part[m * PART_STRIDE + lane] = act ? pa : NEG;
-          part[(L + m) * PART_STRIDE + lane] = act ? ps : NEG;
-        }
-        __syncwarp();
-        reduce_rows<T, true>(part, L, lane, shA);
-        reduce_rows<T, true>(part + L * PART_STRIDE, L, lane, shS);
-        __syncwarp();
-        // A_m relative to its maximum, added lane after lane
-#pragma unroll 1
-        for (int m = 0; m < L; ++m) {
-          const T ha = shA[m];
-          T v[PPL], pa = T(0);
-          expo(m, false, v);
+          for (int p = 0; p < PPL; ++p) hs = fmax(hs, e[p]);
+          ha = warp_max_redux(act ? ha : NEG);
+          hs = warp_max_redux(act ? hs : NEG);
+#pragma unroll
+          for (int p = 0; p < PPL; ++p) {
+            v[p] = exp2_t(v[p] - ha);
+            e[p] = exp2_t(e[p] - hs);
+          }
           if (act) {
 #pragma unroll
-            for (int p = 0; p < PPL; ++p) pa += exp2_t(v[p] - ha);
+            for (int p = 0; p < PPL; ++p) {
+              pa += v[p];
+              ps += e[p];
+            }
           }
           part[m * PART_STRIDE + lane] = pa;
-        }
-        __syncwarp();
-        T wmax = NEG;
-        for (int m = lane; m < L; m += 32) {
-          const T r = lane_sum_in_order<T>(part + m * PART_STRIDE);
-          rowA[m] = r;
-          coef[m] = shS[m] - shA[m] - log2_fast(r);
-          wmax = fmax(wmax, coef[m]);
-        }
-        wmax = warp_max_redux(wmax);
-        for (int m = lane; m < L; m += 32) coef[m] = exp2_t(coef[m] - wmax);
-        __syncwarp();
+          part[(L + m) * PART_STRIDE + lane] = ps;
+          if (lane == 0) {
+            shA[m] = ha;
+            shS[m] = hs;
+          }
+        };
+        // then the sums of the rows, a lane a row, and w_m relative to the largest
+        auto finish_rows = [&]() {
+          __syncwarp();
+          for (int r = lane; r < 2 * L; r += 32) {
+            const T t = lane_sum_in_order<T>(part + r * PART_STRIDE);
+            (r < L ? rowA : rowS - L)[r] = t;
+          }
+          __syncwarp();
+          T wmax = NEG;
+          for (int m = lane; m < L; m += 32) {
+            coef[m] = shS[m] - shA[m] - log2_fast(rowA[m]);
+            wmax = fmax(wmax, coef[m]);
+          }
+          wmax = warp_max_redux(wmax);
+          for (int m = lane; m < L; m += 32) coef[m] = exp2_t(coef[m] - wmax);
+          __syncwarp();
+        };
 #pragma unroll
         for (int p = 0; p < PPL; ++p) B[p] = T(0);
-        // S_m relative to its maximum, and beta
+        constexpr int KEEP = PPL <= 2 ? 8 : 0;  // draws whose exponentials fit the registers
+        if (KEEP > 0 && L <= KEEP) {
+          T e[KEEP > 0 ? KEEP : 1][PPL];
+#pragma unroll
+          for (int m = 0; m < KEEP; ++m)
+            if (m < L) row(m, e[m]);
+          finish_rows();
+#pragma unroll
+          for (int m = 0; m < KEEP; ++m)
+            if (m < L) axpy<T, PPL>(coef[m], e[m], B);
+        } else {
 #pragma unroll 1
-        for (int m = 0; m < L; ++m) {
-          const T hs = shS[m];
-          T v[PPL], ps = T(0);
-          expo(m, true, v);
-#pragma unroll
-          for (int p = 0; p < PPL; ++p) v[p] = exp2_t(v[p] - hs);
-          axpy<T, PPL>(coef[m], v, B);
-          if (act) {
-#pragma unroll
-            for (int p = 0; p < PPL; ++p) ps += v[p];
+          for (int m = 0; m < L; ++m) {
+            T e[PPL];
+            row(m, e);
           }
-          part[m * PART_STRIDE + lane] = ps;
+          finish_rows();
+#pragma unroll 1
+          for (int m = 0; m < L; ++m) {
+            T e[PPL];
+            expo(m, true, e);
+            const T hs = shS[m];
+#pragma unroll
+            for (int p = 0; p < PPL; ++p) e[p] = exp2_t(e[p] - hs);
+            axpy<T, PPL>(coef[m], e, B);
+          }
         }
-        __syncwarp();
-        for (int m = lane; m < L; m += 32) rowS[m] = lane_sum_in_order<T>(part + m * PART_STRIDE);
-        __syncwarp();
       }
     }
     T gmax = T(0);  // the largest row maximum (robust path without x-z coupling; else 0)
