@@ -32,7 +32,7 @@ typedef enum {
   DPF_E_INVALID = 1,     /* bad argument (null pointer, size out of range, bad model) */
   DPF_E_NOMEM = 2,       /* a device allocation failed; nothing leaked */
   DPF_E_CUDA = 3,        /* a CUDA runtime call failed */
-  DPF_E_TIMEOUT = 4,     /* a bounded device-side wait gave up (the scan look-back) */
+  DPF_E_TIMEOUT = 4,     /* a bounded device-side wait gave up */
   DPF_E_NUMERIC = 5,     /* all weights zero, or a NaN weight */
   DPF_E_UNSUPPORTED = 6  /* a valid request outside the compiled configurations */
 } dpf_status;
@@ -163,7 +163,8 @@ dpf_status dpf_sync(dpf_ctx* ctx);
  *  out_idx: device, n_total int32 ancestor indices, local to each segment.
  * DPF_SYS_GLOBAL accepts n_seg == 1 only. A segment whose weights are all zero,
  * or any negative/NaN/infinite weight, gives DPF_E_NUMERIC (after synchronising).
- * Allocates temporary device memory for the scan state; synchronises `stream`.
+ * Allocates temporary device memory (from a pool that keeps it for the next call);
+ * synchronises `stream`.
  */
 dpf_status dpf_resample(const void* w, int32_t dtype, int64_t n_total, int64_t n_seg, int32_t rule,
                         const uint32_t* u, int32_t* out_idx, void* stream);
@@ -174,13 +175,13 @@ dpf_status dpf_resample(const void* w, int32_t dtype, int64_t n_total, int64_t n
  * must not allocate after start-up, or an application whose framework allocator
  * already holds the whole device. The paper has no counterpart; this is a
  * property of the library, not of the method.
- * It makes no cudaMalloc, cudaFree or other allocating call: its scratch (the
- * largest weight, the quantised total and the look-back state of the scan) is
- * a fixed device array of about 40 KB, one per device, held from the first
- * call until the process exits. Consequences:
+ * It makes no cudaMalloc, cudaFree or other allocating call: its scratch (each
+ * CTA's largest weight and quantised total) is a fixed device array of about
+ * 20 KB, one per device, held from the first call until the process exits.
+ * Consequences:
  *  - n may be at most 4,194,304; larger n gives DPF_E_INVALID (use dpf_resample).
  *  - Every call on a device shares that array and leaves its contents behind;
- *    each call clears the part it uses first. Calls whose work overlaps on the
+ *    each call writes the part it uses first. Calls whose work overlaps on the
  *    GPU (different streams, or several host threads) race on it and give
  *    wrong indices: serialise them.
  *  - The first call on a device looks up the array's device address
@@ -516,13 +517,12 @@ dpf_status dpf_record_tuples_amortised(dpf_ctx* ctx, int64_t i0, int64_t n_outer
 
 /*
  * A check of the failure path of the bounded waits; the paper has no
- * counterpart. Runs (1) the global resampling's scan on 3 x 2048 unit weights
- * with tile 0 publishing nothing, so that the look-back waits of the other
- * tiles can never be satisfied, and (2) a step's outer stage (3 CTAs of one
- * cooperative launch) with CTA 0 never reaching the grid-wide barrier. In both
- * the waits give up after their bound (a few tenths of a second) and the device
- * stays usable; the call returns DPF_E_TIMEOUT when both waits ran out as they
- * should, and another status otherwise. Synchronises the stream.
+ * counterpart. Runs a step's outer stage (3 CTAs of one cooperative launch) with
+ * CTA 0 never reaching the grid-wide barrier. The waits give up after their bound
+ * (a few tenths of a second) and the device stays usable; the call returns
+ * DPF_E_TIMEOUT when they ran out as they should, and another status otherwise.
+ * (The global resampling has no waits: its CTAs take their prefixes from an
+ * earlier launch.) Synchronises the stream.
  */
 dpf_status dpf_check_bounded_wait(void* stream);
 

@@ -41,7 +41,7 @@ dpf_status err_word_status(int w, const char* what) {
 // device's default pool gives its memory back to the system at every synchronisation, so each
 // dpf_resample call, which synchronises, mapped and unmapped its block again (230 of the 285 us
 // of a call at n = 1,000,003). This pool keeps up to 32 MB, the grain in which a pool takes memory (a
-// call at the largest n, 2^31, needs 21 MB); what is above that goes back as before. The pool's own order
+// call needs 20 KB at most); what is above that goes back as before. The pool's own order
 // keeps blocks of concurrent streams and threads apart.
 static cudaMemPool_t scratch_pool() {
   static std::mutex mu;
@@ -65,26 +65,13 @@ static cudaMemPool_t scratch_pool() {
   return pools[dev];
 }
 
-dpf_status scratch_alloc(Scratch& sc, long long tiles, cudaStream_t s) {
-  const size_t head = 64;
-  const size_t bytes = head + (size_t)tiles * (4 + 8 + 8) + 16;
+dpf_status scratch_alloc(Scratch& sc, int ctas, cudaStream_t s) {
   cudaMemPool_t pool = scratch_pool();
-  cudaError_t e = pool ? cudaMallocFromPoolAsync(&sc.block, bytes, pool, s) : cudaMallocAsync(&sc.block, bytes, s);
-  if (e != cudaSuccess) {
-    sc.block = nullptr;
-    return cuda_error(e, "scratch allocation");
-  }
-  e = cudaMemsetAsync(sc.block, 0, bytes, s);
-  if (e != cudaSuccess) return cuda_error(e, "scratch memset");
-  unsigned char* b = (unsigned char*)sc.block;
-  sc.maxkey = (unsigned long long*)(b + 0);
-  sc.C = (unsigned long long*)(b + 8);
-  sc.scan.ticket = (unsigned long long*)(b + 16);
-  sc.shift = (int*)(b + 24);
-  sc.err = (int*)(b + 28);
-  sc.scan.agg = (unsigned long long*)(b + head);
-  sc.scan.incl = sc.scan.agg + tiles;
-  sc.scan.flags = (uint32_t*)(sc.scan.incl + tiles);
+  void* p = nullptr;
+  cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, scratch_bytes(ctas), pool, s)
+                       : cudaMallocAsync(&p, scratch_bytes(ctas), s);
+  if (e != cudaSuccess) return cuda_error(e, "scratch allocation");
+  scratch_layout(sc, p, ctas);
   return DPF_OK;
 }
 

@@ -20,25 +20,28 @@ dpf_status cuda_error(cudaError_t e, const char* what);
 // cudaErrorMemoryAllocation when dpf_fail_allocation_after has armed it for this call.
 cudaError_t device_malloc(void** p, size_t bytes);
 
-// Look-back state of one scan: per-tile flag words and values, and the
-// monotone ticket counter that hands out tile indices in launch order.
-struct ScanState {
-  uint32_t* flags;           // n_tiles words: (epoch << 2) | state, state 1 = aggregate, 2 = prefix
-  unsigned long long* agg;   // n_tiles
-  unsigned long long* incl;  // n_tiles
-  unsigned long long* ticket;
-};
-
 // Temporary device memory of one dpf_resample call (stream-ordered allocation).
 struct Scratch {
   void* block = nullptr;
-  unsigned long long* maxkey = nullptr;
-  unsigned long long* C = nullptr;
-  int* shift = nullptr;
   int* err = nullptr;
-  ScanState scan{};
+  unsigned long long* keys = nullptr;    // one a CTA: its largest weight's bits, ~0 for a bad weight
+  unsigned long long* totals = nullptr;  // one a CTA: its count total
 };
-dpf_status scratch_alloc(Scratch& sc, long long tiles, cudaStream_t s);
+// CTAs of the global rule's passes over n weights, each a contiguous range of 512-item chunks.
+constexpr int RS_MAX_CTAS = 8 * 152;
+inline int resample_ctas(long long n) {
+  const long long nch = (n + 511) / 512;
+  return (int)(nch < RS_MAX_CTAS ? nch : RS_MAX_CTAS);
+}
+constexpr size_t scratch_bytes(int ctas) { return 64 + (size_t)ctas * 16; }
+// The parts of a block of scratch_bytes(ctas).
+inline void scratch_layout(Scratch& sc, void* block, int ctas) {
+  sc.block = block;
+  sc.err = (int*)block;
+  sc.keys = (unsigned long long*)((unsigned char*)block + 64);
+  sc.totals = sc.keys + ctas;
+}
+dpf_status scratch_alloc(Scratch& sc, int ctas, cudaStream_t s);
 void scratch_free(Scratch& sc, cudaStream_t s);
 // Synchronise, read the device error word, free, and map it to a status.
 dpf_status scratch_finish(Scratch& sc, cudaStream_t s, const char* what);
@@ -49,7 +52,8 @@ dpf_status err_word_status(int w, const char* what);
 dpf_status check_outer_barrier(cudaStream_t s);
 
 // Launch the global systematic-resampling kernels on caller-provided scratch
-// (laid out as by scratch_alloc and zeroed); no allocation, no synchronisation.
+// (laid out for resample_ctas(n) CTAs; nothing in it need be cleared); no allocation, no
+// synchronisation. *sc.err holds the call's error bits afterwards.
 void launch_global_on(const void* w, int32_t dtype, long long n, const uint32_t* u, int32_t* out,
                       Scratch& sc, cudaStream_t s);
 
@@ -87,10 +91,6 @@ struct BatchLaunch {
 };
 
 // Per-variant launchers, one set per compiled (precision, d1, d2, dy).
-// Tiles of the decoupled look-back scan of the global resampling.
-constexpr int SCAN_NT = 256;   // threads per scan tile
-constexpr int SCAN_IPT = 8;    // items per thread
-constexpr int SCAN_TILE = SCAN_NT * SCAN_IPT;
 // the outer stage of a step (dpf_outer.cuh): threads a CTA, items a thread in one
 // chunk, items a chunk, the bound on its grid (rows of partial sums, count totals),
 // and the sums a filter: W, W^2 and the d <= 64 weighted means

@@ -17,8 +17,7 @@
 namespace dpf {
 
 constexpr long long kNoAllocMaxN = 1ll << 22;  // at most 4,194,304 weights per call
-constexpr long long kNoAllocTiles = (kNoAllocMaxN + 2047) / 2048;
-constexpr size_t kNoAllocBytes = 64 + (size_t)kNoAllocTiles * (8 + 8 + 4) + 16;  // 41,040 bytes
+constexpr size_t kNoAllocBytes = scratch_bytes(RS_MAX_CTAS);  // 19,520 bytes
 
 // The scratch itself (every device that loads the library holds one copy
 // until the process exits). Host code must not pass this name to a kernel:
@@ -67,21 +66,8 @@ extern "C" dpf_status dpf_resample_noalloc(const void* w, int32_t dtype, int64_t
   unsigned char* b = (unsigned char*)scratch_address(dev, &e);
   if (!b) return cuda_error(e, "dpf_resample_noalloc: cudaGetSymbolAddress");
   cudaStream_t s = (cudaStream_t)stream;
-  const long long tiles = (n + 2047) / 2048;
-  const size_t used = 64 + (size_t)tiles * (8 + 8 + 4);
-  // the scratch keeps the previous call's contents: clear the part this call uses
-  e = cudaMemsetAsync(b, 0, used, s);
-  if (e != cudaSuccess) return cuda_error(e, "dpf_resample_noalloc: clearing the scratch");
   Scratch sc;
-  sc.block = b;
-  sc.maxkey = (unsigned long long*)(b + 0);
-  sc.C = (unsigned long long*)(b + 8);
-  sc.scan.ticket = (unsigned long long*)(b + 16);
-  sc.shift = (int*)(b + 24);
-  sc.err = (int*)(b + 28);
-  sc.scan.agg = (unsigned long long*)(b + 64);
-  sc.scan.incl = sc.scan.agg + tiles;
-  sc.scan.flags = (uint32_t*)(sc.scan.incl + tiles);
+  scratch_layout(sc, b, resample_ctas(n));  // (the passes overwrite all of it that they read)
   launch_global_on(w, dtype, n, u, out_idx, sc, s);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_error(e, "dpf_resample_noalloc: launch");

@@ -51,6 +51,16 @@ struct FusedOuterArgs {
 };
 
 // ---- A: the partial sums and the count total of CTA `bid` of the `nb` CTAs of one filter ----
+// What only the bootstrap particle filter's outer stage does (PF; its sets are a hundred times
+// larger and its step has the weighted sums already). The other filters' stage is a few microseconds
+// of latency, most of it cold instruction fetches, so none of it is compiled into theirs.
+// Whether a CTA owns at least two long chunks of the scatter.
+template <typename T>
+__device__ __forceinline__ bool long_ranges(const FusedOuterArgs<T>& a, int nb) {
+  const long long nch = (a.o.N + OF_CHUNK - 1) / OF_CHUNK;
+  return a.w_out && nch >= (long long)nb * 2 * SCATTER_IPT_LONG / OF_IPT;
+}
+
 // Whether the sums that came with the step serve (OuterArgs::npre): with the largest weight at
 // least e^-20 of the reference its square is 4e-18, so single precision holds W'^2 and every
 // weight of consequence beside it.
@@ -59,7 +69,7 @@ __device__ __forceinline__ bool sums_given(const OuterArgs<T>& o, T lwmax) {
   return o.npre > 0 && lwmax >= o.lref - T(20) && lwmax <= o.lref + T(20);
 }
 
-template <typename T, int D1, int D2>
+template <typename T, int D1, int D2, bool PF>
 __device__ __forceinline__ void outer_sums(const FusedOuterArgs<T>& a, int bid, int nb, T lwmax) {
   constexpr int NV = 2 + D1 + D2, NW = OF_NT / 32;
   __shared__ T sv[NV][NW];
@@ -71,42 +81,51 @@ __device__ __forceinline__ void outer_sums(const FusedOuterArgs<T>& a, int bid, 
   const long long nch = (N + OF_CHUNK - 1) / OF_CHUNK;
   const long long i0 = nch * bid / nb * OF_CHUNK, i1 = nch * (bid + 1) / nb * OF_CHUNK;
   const long long iend = i1 < N ? i1 : N;
-  T v[NV];
-#pragma unroll
-  for (int q = 0; q < NV; ++q) v[q] = T(0);
+  const bool given = PF && sums_given(o, lwmax), keep = PF && long_ranges(a, nb);  // uniform over the grid
   unsigned long long cc = 0;
-  const bool given = sums_given(o, lwmax);  // uniform over the grid
   if (given) {
-    for (long long i = i0 + tid; i < iend; i += OF_NT)
-      cc += (unsigned long long)floor(exp_t<T>(o.lw[i] - lwmax) * sS);
-  } else {
     for (long long i = i0 + tid; i < iend; i += OF_NT) {
       const T W = exp_t<T>(o.lw[i] - lwmax);
+      if (keep) a.w_out[i] = W;
+      cc += (unsigned long long)floor(W * sS);
+    }
+  } else {
+    T v[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] = T(0);
+    for (long long i = i0 + tid; i < iend; i += OF_NT) {
+      // every load of the item first (d of them in flight, not one product's at a time)
+      T m[D1 + D2];
+#pragma unroll
+      for (int c = 0; c < D1; ++c) m[c] = PF ? o.xm[c * o.xc + i * o.xi] : o.xm[(long long)c * N + i];
+#pragma unroll
+      for (int c = 0; c < D2; ++c) m[D1 + c] = o.zm[(long long)c * N + i];
+      const T W = exp_t<T>(o.lw[i] - lwmax);
+      if (keep) a.w_out[i] = W;
       cc += (unsigned long long)floor(W * sS);  // exact: a power-of-two scaling, then a floor
       v[0] += W;
       v[1] += W * W;
 #pragma unroll
-      for (int c = 0; c < D1; ++c) v[2 + c] += W * o.xm[c * o.xc + i * o.xi];
-#pragma unroll
-      for (int c = 0; c < D2; ++c) v[2 + D1 + c] += W * o.zm[(long long)c * N + i];
+      for (int c = 0; c < D1 + D2; ++c) v[2 + c] += W * m[c];
     }
 #pragma unroll
     for (int q = 0; q < NV; ++q) v[q] = warp_sum(v[q]);
+    if (lane == 0) {
+#pragma unroll
+      for (int q = 0; q < NV; ++q) sv[q][w] = v[q];
+    }
   }
   cc = warp_sum(cc);
-  if (lane == 0) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) sv[q][w] = v[q];
-    su[w] = cc;
-  }
+  if (lane == 0) su[w] = cc;
   __syncthreads();
-  if (tid == 0) {  // one thread publishes the CTA's row (so that one fence covers it)
-    for (int q = 0; q < (given ? 0 : NV); ++q) {
-      T s = T(0);
+  // the CTA's row, a thread a sum (the caller's barrier and its one thread's fence cover them all)
+  if (!given && tid < NV) {
+    T s = T(0);
 #pragma unroll
-      for (int r = 0; r < NW; ++r) s += sv[q][r];
-      o.partials[(long long)bid * NV + q] = (double)s;
-    }
+    for (int r = 0; r < NW; ++r) s += sv[tid][r];
+    o.partials[(long long)bid * NV + tid] = (double)s;
+  }
+  if (tid == OF_NT - 1) {
     unsigned long long s = 0;
 #pragma unroll
     for (int r = 0; r < NW; ++r) s += su[r];
@@ -114,111 +133,51 @@ __device__ __forceinline__ void outer_sums(const FusedOuterArgs<T>& a, int bid, 
   }
 }
 
-// ---- B: the exclusive prefix of CTA `bid`'s count total and the total C, once every
-// CTA's total is in place (block-wide: every thread receives both) ----
-__device__ __forceinline__ void count_prefix(const unsigned long long* ctot, int bid, int nb,
-                                             unsigned long long& pre, unsigned long long& C) {
-  constexpr int NW = OF_NT / 32;
-  __shared__ unsigned long long su[2][NW];
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  unsigned long long p = 0, t = 0;
-  for (int b = tid; b < nb; b += OF_NT) {
-    const unsigned long long c = __ldcg(ctot + b);
-    t += c;
-    if (b < bid) p += c;
-  }
-  p = warp_sum(p);
-  t = warp_sum(t);
-  __syncthreads();
-  if (lane == 0) {
-    su[0][w] = p;
-    su[1][w] = t;
-  }
-  __syncthreads();
-  pre = 0;
-  C = 0;
-#pragma unroll
-  for (int r = 0; r < NW; ++r) {
-    pre += su[0][r];
-    C += su[1][r];
-  }
-}
-
-// ---- C: the chunks' cumulative counts, the points below them, the ancestors (C > 0) ----
-template <typename T>
+// ---- C: the chunks' cumulative counts, the points below them, the ancestors (C > 0). A CTA of a
+// large particle set (at least two long chunks each) reads back the weights the sums left in w_out
+// and takes four times the items between barriers; else the weights are formed again from the
+// log-weights, which the sums have just brought into the L1 cache ----
+template <typename T, bool PF>
 __device__ __forceinline__ void outer_scatter(const FusedOuterArgs<T>& a, int bid, int nb, T lwmax,
                                               unsigned long long pre, unsigned long long C) {
-  constexpr int NW = OF_NT / 32;
-  __shared__ unsigned long long su[NW];
-  __shared__ int ks[OF_CHUNK + 1];
+  __shared__ unsigned long long su[OF_NT / 32];
+  __shared__ int ks[OF_NT * (PF ? SCATTER_IPT_LONG : OF_IPT) + 1];
   const OuterArgs<T>& o = a.o;
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const long long N = o.N;
   const T sS = pow2_t<T>(a.shift);
   const long long nch = (N + OF_CHUNK - 1) / OF_CHUNK;
-  const long long ch0 = nch * bid / nb, ch1 = nch * (bid + 1) / nb;
+  const long long i0 = nch * bid / nb * OF_CHUNK, i1 = nch * (bid + 1) / nb * OF_CHUNK;
+  const long long iend = i1 < N ? i1 : N;
   const uint32_t u = rand_word(a.key, a.t, 0, P_OUTER, 0);
-  unsigned long long run = pre;
-  for (long long ch = ch0; ch < ch1; ++ch) {
-    const long long base = ch * OF_CHUNK;
-    unsigned long long c[OF_IPT], ts = 0;
-#pragma unroll
-    for (int q = 0; q < OF_IPT; ++q) {
-      const long long i = base + tid * OF_IPT + q;
-      unsigned long long ci = 0;
-      if (i < N) {
-        const T W = exp_t<T>(o.lw[i] - lwmax);
-        if (a.w_out) a.w_out[i] = W;
-        ci = (unsigned long long)floor(W * sS);
-      }
-      c[q] = ci;
-      ts += ci;
+  auto quant = [&](T W) { return (unsigned long long)floor(W * sS); };
+  if constexpr (PF) {
+    if (long_ranges(a, nb)) {
+      __shared__ PointScale s_ps;
+      if (threadIdx.x == 0) s_ps = point_scale(N, C);
+      __syncthreads();
+      auto load = [&](long long i, T (&W)[SCATTER_IPT_LONG]) {
+        load_weights<T, SCATTER_IPT_LONG>(a.w_out, i, iend, true, W);
+      };
+      scatter_range<T, SCATTER_IPT_LONG, true>(i0, iend, N, u, pre, C, s_ps, a.anc, ks, su, load, quant);
+      return;
     }
-    // exclusive block scan of the per-thread sums
-    unsigned long long incl = ts;
-#pragma unroll
-    for (int s = 1; s < 32; s <<= 1) {
-      const unsigned long long n = __shfl_up_sync(FULL, incl, s);
-      if (lane >= s) incl += n;
-    }
-    if (lane == 31) su[w] = incl;
-    __syncthreads();
-    unsigned long long wpre = 0, agg = 0;
-#pragma unroll
-    for (int r = 0; r < NW; ++r) {
-      if (r < w) wpre += su[r];
-      agg += su[r];
-    }
-    unsigned long long cum = run + wpre + incl - ts;
-    if (tid == 0) ks[0] = points_below_est(run, N, u, C);
-#pragma unroll
-    for (int q = 0; q < OF_IPT; ++q) {
-      cum += c[q];
-      ks[tid * OF_IPT + q + 1] = points_below_est(cum, N, u, C);
-    }
-    __syncthreads();
-    // output k lies in item j's range ks[j] <= k < ks[j + 1] (an empty range is never
-    // hit, so j is never an item past N, whose count is zero)
-    const int khi = ks[OF_CHUNK];
-    for (int k = ks[0] + tid; k < khi; k += OF_NT) {
-      int lo = 0, hi = OF_CHUNK;
-      while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (ks[mid] <= k)
-          lo = mid;
-        else
-          hi = mid;
-      }
-      a.anc[k] = (int32_t)(base + lo);
-    }
-    run += agg;
-    __syncthreads();  // ks and su are reused by the next chunk
   }
+  auto load = [&](long long i, T (&W)[OF_IPT]) {
+#pragma unroll
+    for (int q = 0; q < OF_IPT; ++q) {
+      W[q] = T(0);
+      if (i + q < iend) {
+        W[q] = exp_t<T>(o.lw[i + q] - lwmax);
+        if (a.w_out) a.w_out[i + q] = W[q];
+      }
+    }
+  };
+  scatter_range<T, OF_IPT, false>(i0, iend, N, u, pre, C, PointScale{0ull, -1}, a.anc, ks, su, load, quant);
 }
 
 // ---- D: the statistics from the `nb` CTAs' partial sums, by one CTA once they are
 // all in place ----
-template <typename T>
+template <typename T, bool PF>
 __device__ __forceinline__ void outer_stats(const FusedOuterArgs<T>& a, int nb, T lwmax,
                                             unsigned long long C) {
   constexpr int NW = OF_NT / 32;
@@ -226,10 +185,12 @@ __device__ __forceinline__ void outer_stats(const FusedOuterArgs<T>& a, int nb, 
   const OuterArgs<T>& o = a.o;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int D = o.d1 + o.d2, NV = 2 + D;
-  const bool given = sums_given(o, lwmax);
+  const bool given = PF && sums_given(o, lwmax);
   const int rows = given ? o.npre : nb;
+  // a warp a sum; four of its rows in flight
   for (int q = w; q < NV; q += NW) {
     double s = 0.0;
+#pragma unroll 4
     for (int b = lane; b < rows; b += 32) s += __ldcg(o.partials + (long long)b * NV + q);
     s = warp_sum(s);
     if (lane == 0) sd[q] = s;
@@ -274,17 +235,17 @@ __device__ __forceinline__ void outer_done(const FusedOuterArgs<T>& a, int nb) {
 }
 
 // One filter's outer stage in one cooperative launch (every CTA resident at once).
-template <typename T, int D1, int D2>
+template <typename T, int D1, int D2, bool PF>
 __global__ void __launch_bounds__(OF_NT) fused_outer_kernel(const __grid_constant__ FusedOuterArgs<T> a) {
   __shared__ int s_ok;
   const int tid = threadIdx.x, bid = blockIdx.x, nb = gridDim.x, nw = a.nwork;
   T lwmax;
   order_decode(*a.o.lwmax_key, lwmax);
-  if (bid < nw) outer_sums<T, D1, D2>(a, bid, nw, lwmax);
+  if (bid < nw) outer_sums<T, D1, D2, PF>(a, bid, nw, lwmax);
   __syncthreads();
   // grid-wide barrier: every CTA is resident, and the wait is bounded all the same
   if (tid == 0) {
-    __threadfence();  // the CTA's partial row and count total, written by this thread
+    __threadfence();  // the CTA's partial row and count total, written before the barrier above
     cuda::atomic_ref<unsigned int, cuda::thread_scope_device> arr(*a.arrive);
     if (bid != a.withhold) arr.fetch_add(1u, cuda::memory_order_release);
     bool ok = arr.load(cuda::memory_order_acquire) >= (unsigned)nb;
@@ -300,8 +261,8 @@ __global__ void __launch_bounds__(OF_NT) fused_outer_kernel(const __grid_constan
   __syncthreads();
   unsigned long long pre, C;
   count_prefix(a.ctot, bid < nw ? bid : nw, nw, pre, C);
-  if (bid == (nb > nw ? nw : nw - 1)) outer_stats<T>(a, nw, lwmax, C);
-  if (bid < nw && s_ok && C > 0) outer_scatter<T>(a, bid, nw, lwmax, pre, C);  // else the ancestors stay
+  if (bid == (nb > nw ? nw : nw - 1)) outer_stats<T, PF>(a, nw, lwmax, C);
+  if (bid < nw && s_ok && C > 0) outer_scatter<T, PF>(a, bid, nw, lwmax, pre, C);  // else the ancestors stay
   outer_done<T>(a, nb);
 }
 
@@ -318,7 +279,7 @@ __global__ void __launch_bounds__(OF_NT)
   const FusedOuterArgs<T>& a = args[f];
   T lwmax;
   order_decode(*a.o.lwmax_key, lwmax);
-  outer_sums<T, D1, D2>(a, (int)blockIdx.x - cstart[f], cstart[f + 1] - cstart[f], lwmax);
+  outer_sums<T, D1, D2, false>(a, (int)blockIdx.x - cstart[f], cstart[f + 1] - cstart[f], lwmax);
 }
 
 template <typename T>
@@ -334,19 +295,19 @@ __global__ void __launch_bounds__(OF_NT)
   order_decode(*a.o.lwmax_key, lwmax);
   unsigned long long pre, C;
   count_prefix(a.ctot, bid, nb, pre, C);
-  if (C > 0) outer_scatter<T>(a, bid, nb, lwmax, pre, C);
-  if (bid == nb - 1) outer_stats<T>(a, nb, lwmax, C);
+  if (C > 0) outer_scatter<T, false>(a, bid, nb, lwmax, pre, C);
+  if (bid == nb - 1) outer_stats<T, false>(a, nb, lwmax, C);
   outer_done<T>(a, nb);
 }
 
 // CTAs resident on the device at once for the single-filter launch.
-template <typename T, int D1, int D2>
+template <typename T, int D1, int D2, bool PF = false>
 int fused_outer_cap() {
   static const int cap = [] {
     int dev = 0, sms = 0, occ = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fused_outer_kernel<T, D1, D2>, OF_NT, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fused_outer_kernel<T, D1, D2, PF>, OF_NT, 0);
     const int c = occ * sms;
     return c < 2 ? 2 : c;
   }();
@@ -356,16 +317,16 @@ int fused_outer_cap() {
 // CTAs that own items in a filter's outer stage over N items: one a chunk, at most
 // OF_MAX_CTAS and one fewer than the resident capacity (the same in the single and
 // batched forms, so that their partitions agree).
-template <typename T, int D1, int D2>
+template <typename T, int D1, int D2, bool PF = false>
 int fused_outer_grid(long long N) {
-  const long long cap = fused_outer_cap<T, D1, D2>() - 1;
+  const long long cap = fused_outer_cap<T, D1, D2, PF>() - 1;
   const long long lim = cap < OF_MAX_CTAS ? cap : OF_MAX_CTAS;
   const long long nch = (N + OF_CHUNK - 1) / OF_CHUNK;
   return (int)(nch < lim ? nch : lim);
 }
 
 // The single-filter launch: a.nwork CTAs with items and one for the statistics.
-template <typename T, int D1, int D2>
+template <typename T, int D1, int D2, bool PF = false>
 cudaError_t fused_outer_launch(const FusedOuterArgs<T>& a, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)a.nwork + 1u);
@@ -377,7 +338,7 @@ cudaError_t fused_outer_launch(const FusedOuterArgs<T>& a, cudaStream_t st) {
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, fused_outer_kernel<T, D1, D2>, a);
+  return cudaLaunchKernelEx(&cfg, fused_outer_kernel<T, D1, D2, PF>, a);
 }
 
 }  // namespace dpf

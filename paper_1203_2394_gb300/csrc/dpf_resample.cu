@@ -10,56 +10,138 @@
 
 namespace dpf {
 
-constexpr int WQ = 8;  // weights a thread loads at once
+// The global rule in three passes over the same partition (CTA b of nb owns a contiguous range of
+// 512-item chunks): the largest weight, the counts' totals, and the scatter, whose prefix comes from
+// the totals before it. The launch boundaries stand in for grid barriers; no CTA waits for another.
+// (A single scan pass with decoupled look-back took 25 us at n = 1,000,003, of a call of 84,
+// waiting along its chain of tiles; the call takes 78 now.)
+constexpr int RS_Q = 8;  // weights a thread loads at once
+constexpr unsigned long long RS_BAD = ~0ull;
 
-// Largest weight as an order-preserving 64-bit key (weights are >= 0, so the
-// IEEE bit pattern orders like the value); flags negative, NaN and inf.
+struct RsRange {
+  long long i0, iend;
+};
+__device__ __forceinline__ RsRange rs_range(long long n, int bid, int nb) {
+  const long long nch = (n + 511) / 512;
+  const long long i1 = nch * (bid + 1) / nb * 512;
+  return RsRange{nch * bid / nb * 512, i1 < n ? i1 : n};
+}
+
+// keys[b]: the bits of CTA b's largest weight (weights are >= 0, so the IEEE bit pattern orders like
+// the value), RS_BAD where a weight is negative, NaN or infinite.
 template <typename T>
-__global__ void __launch_bounds__(256) wmax_kernel(const T* w, long long n, unsigned long long* maxkey, int* err) {
+__global__ void __launch_bounds__(OF_NT) resample_max_kernel(const T* w, long long n, unsigned long long* keys) {
+  __shared__ unsigned long long su[OF_NT / 32];
+  const RsRange r = rs_range(n, blockIdx.x, gridDim.x);
   const bool vec = ((uintptr_t)w & 15) == 0;
   T best = T(0);
   bool bad = false;
-  for (long long i = (blockIdx.x * 256ll + threadIdx.x) * WQ; i < n; i += (long long)gridDim.x * 256 * WQ) {
-    T W[WQ];
-    load_weights<T, WQ>(w, i, n, vec, W);
+  for (long long i = r.i0 + threadIdx.x * RS_Q; i < r.iend; i += OF_NT * RS_Q) {
+    T W[RS_Q];
+    load_weights<T, RS_Q>(w, i, r.iend, vec, W);
 #pragma unroll
-    for (int q = 0; q < WQ; ++q) {
+    for (int q = 0; q < RS_Q; ++q) {
       bad |= !(W[q] >= T(0)) || isinf(W[q]);
       best = fmax(best, W[q]);
     }
   }
   best = warp_max(best);
-  if (__any_sync(FULL, bad) && (threadIdx.x & 31) == 0) atomicOr(err, ERR_NUMERIC);
-  if ((threadIdx.x & 31) == 0 && best > T(0))
-    atomicMax(maxkey, sizeof(T) == 8 ? (unsigned long long)__double_as_longlong((double)best)
-                                     : (unsigned long long)__float_as_uint((float)best));
+  bad = __any_sync(FULL, bad);
+  if ((threadIdx.x & 31) == 0)
+    su[threadIdx.x >> 5] = bad ? RS_BAD
+                               : sizeof(T) == 8 ? (unsigned long long)__double_as_longlong((double)best)
+                                                : (unsigned long long)__float_as_uint((float)best);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long k = 0;
+#pragma unroll
+    for (int q = 0; q < OF_NT / 32; ++q) k = su[q] > k ? su[q] : k;
+    keys[blockIdx.x] = k;
+  }
 }
 
-// C = sum floor(W_i 2^(S - e)) with e from the largest weight; also publishes S - e.
+// The shift S - e of the largest of the nb keys, with S = 62 - ceil(log2 n); false where no weight
+// is positive or one is bad. Block-wide.
 template <typename T>
-__global__ void __launch_bounds__(256) sumc_kernel(const T* w, long long n, int S, const unsigned long long* maxkey,
-                                                   unsigned long long* C, int* shift_out, int* err) {
-  const unsigned long long k = *maxkey;
-  if (k == 0) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(err, ERR_NUMERIC);
-    return;
+__device__ __forceinline__ bool rs_shift(const unsigned long long* keys, int nb, long long n, int& shift) {
+  __shared__ unsigned long long su[OF_NT / 32];
+  unsigned long long k = 0;
+  for (int b = threadIdx.x; b < nb; b += OF_NT) {
+    const unsigned long long v = keys[b];
+    k = v > k ? v : k;
   }
-  const int e = sizeof(T) == 8 ? ilogb(__longlong_as_double((long long)k))
-                               : ilogbf(__uint_as_float((uint32_t)k));
-  if (e > 2000) return;  // an infinite weight (wmax_kernel has flagged it): C stays 0
-  const int shift = S - e;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *shift_out = shift;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long v = __shfl_xor_sync(FULL, k, o);
+    k = v > k ? v : k;
+  }
+  if ((threadIdx.x & 31) == 0) su[threadIdx.x >> 5] = k;
+  __syncthreads();
+  k = su[0];
+#pragma unroll
+  for (int q = 1; q < OF_NT / 32; ++q) k = su[q] > k ? su[q] : k;
+  if (k == 0 || k == RS_BAD) return false;
+  const int e = sizeof(T) == 8 ? ilogb(__longlong_as_double((long long)k)) : ilogbf(__uint_as_float((uint32_t)k));
+  shift = 62 - ceil_log2_i(n) - e;
+  return true;
+}
+
+// totals[b] = sum of floor(W_i 2^(S - e)) over CTA b's weights.
+template <typename T>
+__global__ void __launch_bounds__(OF_NT)
+    resample_sum_kernel(const T* w, long long n, const unsigned long long* keys, unsigned long long* totals) {
+  __shared__ unsigned long long su[OF_NT / 32];
+  int shift = 0;
+  const bool ok = rs_shift<T>(keys, gridDim.x, n, shift);
+  const RsRange r = rs_range(n, blockIdx.x, gridDim.x);
   const bool vec = ((uintptr_t)w & 15) == 0;
   unsigned long long s = 0;
-  for (long long i = (blockIdx.x * 256ll + threadIdx.x) * WQ; i < n; i += (long long)gridDim.x * 256 * WQ) {
-    T W[WQ];
-    load_weights<T, WQ>(w, i, n, vec, W);
+  for (long long i = ok ? r.i0 + threadIdx.x * RS_Q : r.iend; i < r.iend; i += OF_NT * RS_Q) {
+    T W[RS_Q];
+    load_weights<T, RS_Q>(w, i, r.iend, vec, W);
 #pragma unroll
-    for (int q = 0; q < WQ; ++q) s += quantize_u64(W[q], shift);
+    for (int q = 0; q < RS_Q; ++q) s += quantize_u64(W[q], shift);
   }
+  s = warp_sum(s);
+  if ((threadIdx.x & 31) == 0) su[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s = 0;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
-  if ((threadIdx.x & 31) == 0 && s) atomicAdd(C, s);
+    for (int q = 0; q < OF_NT / 32; ++q) s += su[q];
+    totals[blockIdx.x] = s;
+  }
+}
+
+// The ancestors; also the call's error word.
+template <typename T>
+__global__ void __launch_bounds__(OF_NT)
+    resample_scatter_kernel(const T* w, long long n, const uint32_t* up, const unsigned long long* keys,
+                            const unsigned long long* totals, int32_t* out, int* err) {
+  __shared__ unsigned long long su[OF_NT / 32];
+  __shared__ int ks[OF_NT * SCATTER_IPT_LONG + 1];
+  __shared__ PointScale s_ps;
+  int shift = 0;
+  const bool ok = rs_shift<T>(keys, gridDim.x, n, shift);
+  unsigned long long pre, C;
+  count_prefix(totals, blockIdx.x, gridDim.x, pre, C);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *err = ok && C > 0 ? 0 : ERR_NUMERIC;
+  if (!ok || C == 0) return;
+  const RsRange r = rs_range(n, blockIdx.x, gridDim.x);
+  const bool vec = ((uintptr_t)w & 15) == 0;
+  const bool scaled = n >= (1ll << 17);  // a division a CTA, repaid by a few hundred items
+  if (threadIdx.x == 0) s_ps = scaled ? point_scale(n, C) : PointScale{0ull, -1};
+  __syncthreads();
+  auto quant = [&](T W) { return quantize_u64(W, shift); };
+  if (r.iend - r.i0 > OF_CHUNK) {
+    auto load = [&](long long i, T (&W)[SCATTER_IPT_LONG]) {
+      load_weights<T, SCATTER_IPT_LONG>(w, i, r.iend, vec, W);
+    };
+    scatter_range<T, SCATTER_IPT_LONG, true>(r.i0, r.iend, n, *up, pre, C, s_ps, out, ks, su, load, quant);
+  } else {
+    auto load = [&](long long i, T (&W)[OF_IPT]) { load_weights<T, OF_IPT>(w, i, r.iend, false, W); };
+    scatter_range<T, OF_IPT, false>(r.i0, r.iend, n, *up, pre, C, s_ps, out, ks, su, load, quant);
+  }
 }
 
 // Local rule: one block per segment of n <= NT weights.
@@ -113,28 +195,14 @@ static dpf_status launch_local(const T* w, int n, long long nseg, const uint32_t
 
 template <typename T>
 static void launch_global(const T* w, long long n, const uint32_t* u, int32_t* out, Scratch& sc,
-                          cudaStream_t s, long long withhold = -1) {
-  const int S = 62 - ceil_log2_i(n);
-  const int grid = (int)std::min<long long>((n + 256 * WQ - 1) / (256 * WQ), 8 * 152);
-  wmax_kernel<T><<<grid, 256, 0, s>>>(w, n, sc.maxkey, sc.err);
-  sumc_kernel<T><<<grid, 256, 0, s>>>(w, n, S, sc.maxkey, sc.C, sc.shift, sc.err);
-  GlobalArgs<T> a{};
-  a.w = w;
-  a.n = n;
-  a.shift_dev = sc.shift;
-  a.C = sc.C;
-  a.u_ptr = u;
-  a.out = out;
-  a.st = sc.scan;
-  a.ticket_base = 0;
-  a.epoch = 1;
-  a.err = sc.err;
-  a.withhold = withhold;
-  const long long tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-  global_scan_scatter<T><<<(unsigned)tiles, SCAN_NT, 0, s>>>(a);
+                          cudaStream_t s) {
+  const int nb = resample_ctas(n);
+  resample_max_kernel<T><<<nb, OF_NT, 0, s>>>(w, n, sc.keys);
+  resample_sum_kernel<T><<<nb, OF_NT, 0, s>>>(w, n, sc.keys, sc.totals);
+  resample_scatter_kernel<T><<<nb, OF_NT, 0, s>>>(w, n, u, sc.keys, sc.totals, out, sc.err);
 }
 
-// Launch the global-rule pipeline on scratch the caller has laid out (and zeroed).
+// Launch the global-rule passes on scratch the caller has laid out.
 void launch_global_on(const void* w, int32_t dtype, long long n, const uint32_t* u, int32_t* out,
                       Scratch& sc, cudaStream_t s) {
   if (dtype == DPF_F32)
@@ -173,37 +241,10 @@ extern "C" dpf_status dpf_box_muller(const uint32_t* words, int64_t n_pairs, int
   return cuda_error(cudaGetLastError(), "dpf_box_muller");
 }
 
-__global__ void fill_ones_kernel(float* w, long long n) {
-  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (e < n) w[e] = 1.f;
-}
-
 extern "C" dpf_status dpf_check_bounded_wait(void* stream) {
   clear_error();
-  cudaStream_t s = (cudaStream_t)stream;
-  const long long n = 3 * SCAN_TILE;
-  float* w = nullptr;
-  int32_t* out = nullptr;
-  uint32_t* u = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&w, sizeof(float) * n, s);
-  if (e == cudaSuccess) e = cudaMallocAsync((void**)&out, sizeof(int32_t) * n, s);
-  if (e == cudaSuccess) e = cudaMallocAsync((void**)&u, sizeof(uint32_t), s);
-  if (e != cudaSuccess) return cuda_error(e, "dpf_check_bounded_wait: allocation");
-  fill_ones_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(w, n);
-  cudaMemsetAsync(u, 0, sizeof(uint32_t), s);
-  Scratch sc;
-  dpf_status st = scratch_alloc(sc, 3, s);
-  if (!st) {
-    launch_global<float>(w, n, u, out, sc, s, 0);  // tile 0 withholds its prefix
-    st = scratch_finish(sc, s, "dpf_check_bounded_wait");
-  }
-  cudaFreeAsync(w, s);
-  cudaFreeAsync(out, s);
-  cudaFreeAsync(u, s);
-  if (st != DPF_E_TIMEOUT)
-    return st ? st : set_error(DPF_E_CUDA, "dpf_check_bounded_wait: the scan's wait did not run out");
-  // the same for the grid barrier of a step's outer stage (CTA 0 never arrives)
-  st = check_outer_barrier(s);
+  // the grid barrier of a step's outer stage, which CTA 0 never reaches
+  dpf_status st = check_outer_barrier((cudaStream_t)stream);
   if (st != DPF_E_TIMEOUT)
     return st ? st : set_error(DPF_E_CUDA, "dpf_check_bounded_wait: the outer stage's barrier wait did not run out");
   return st;
@@ -223,14 +264,10 @@ extern "C" dpf_status dpf_resample(const void* w, int32_t dtype, int64_t n_total
   const long long seglen = n_total / n_seg;
   if (rule == DPF_SYS_GLOBAL) {
     if (n_seg != 1) return set_error(DPF_E_INVALID, "dpf_resample: global rule needs n_seg == 1");
-    const long long tiles = (n_total + SCAN_TILE - 1) / SCAN_TILE;
     Scratch sc;
-    dpf_status st = scratch_alloc(sc, tiles, s);
+    dpf_status st = scratch_alloc(sc, resample_ctas(n_total), s);
     if (st) return st;
-    if (dtype == DPF_F32)
-      launch_global<float>((const float*)w, n_total, u, out_idx, sc, s);
-    else
-      launch_global<double>((const double*)w, n_total, u, out_idx, sc, s);
+    launch_global_on(w, dtype, n_total, u, out_idx, sc, s);
     return scratch_finish(sc, s, "dpf_resample");
   }
   if (rule != DPF_SYS_LOCAL) return set_error(DPF_E_INVALID, "dpf_resample: unknown rule");
@@ -238,6 +275,7 @@ extern "C" dpf_status dpf_resample(const void* w, int32_t dtype, int64_t n_total
   Scratch sc;
   dpf_status st = scratch_alloc(sc, 0, s);
   if (st) return st;
+  cudaMemsetAsync(sc.err, 0, sizeof(int), s);
   st = dtype == DPF_F32
            ? launch_local<float>((const float*)w, (int)seglen, n_seg, u, out_idx, sc.err, s)
            : launch_local<double>((const double*)w, (int)seglen, n_seg, u, out_idx, sc.err, s);

@@ -1,7 +1,6 @@
-// Global systematic resampling on the GPU: a reduction for the quantised total
-// C, then one pass that scans the quantised counts with a decoupled look-back
-// (Merrill & Garland, "Single-pass Parallel Prefix Scan with Decoupled
-// Look-back", 2016) and scatters each tile's share of the ancestor indices.
+// Global systematic resampling on the GPU: the exact integer rule's building blocks, shared by
+// dpf_resample and by the outer stage of a step: the quantised counts, the number of systematic
+// points below a cumulative count, the CTAs' prefixes, and the scatter of one CTA's ancestors.
 #pragma once
 
 #include <cuda/atomic>
@@ -12,7 +11,7 @@
 
 namespace dpf {
 
-constexpr int SPIN_LIMIT = 1 << 22;  // bounded look-back wait (~0.3 s with the back-off)
+constexpr int SPIN_LIMIT = 1 << 22;  // bounded wait at the outer stage's grid barrier (~0.3 s with the back-off)
 
 typedef unsigned __int128 u128;
 
@@ -48,25 +47,39 @@ __device__ __forceinline__ int points_below_est(unsigned long long c, long long 
   return (int)k;
 }
 
-// Inputs of the scan-and-scatter pass: the weights W_i, with e = floor(log2 max W)
-// given through the shift S - e.
-template <typename T>
-struct GlobalArgs {
-  const T* w;              // n weights
-  long long n;
-  int shift;               // S - e
-  const int* shift_dev;    // if non-null, read S - e from here instead
-  const unsigned long long* C;  // device scalar: the quantised total
-  const uint32_t* u_ptr;   // device scalar uniform word, or null
-  Key key;                 // else u = rand_word(key, t, 0, P_OUTER, 0)
-  uint32_t t;
-  int32_t* out;
-  ScanState st;
-  unsigned long long ticket_base;
-  uint32_t epoch;
-  int* err;
-  long long withhold;  // a tile that publishes nothing (a check of the bounded waits); -1: none
+// The same count by one 64-bit product for almost every c. With P = c n / C (so K(c) =
+// ceil(P - u 2^-32)) and F = floor(n 2^(64+f) / C), m = floor(c F 2^-64) satisfies
+// P 2^f in [m, m + 1.5) (c < 2^63), and U = floor(u 2^(f-32)) satisfies u 2^(f-32) in [U, U + 1);
+// so (P - u 2^-32) 2^f lies in (d - 1, d + 1.5), d = m - U, and its ceiling in units of 2^f is
+// certain unless that interval meets a multiple of 2^f: 2.5 in 2^f of the values, which take
+// the exact comparisons. Both scales are computed once a CTA.
+struct PointScale {
+  unsigned long long F;
+  int f;  // < 0: no scale (C / n below 2^9)
 };
+__device__ __forceinline__ PointScale point_scale(long long n, unsigned long long C) {
+  PointScale p{0ull, -1};
+  const unsigned long long q = C / (unsigned long long)n;
+  const int f = q ? 62 - __clzll((long long)q) : -1;  // n 2^f < C
+  if (f < 8) return p;
+  p.f = f < 32 ? f : 32;
+  p.F = (unsigned long long)(((u128)(unsigned long long)n << (64 + p.f)) / C);
+  return p;
+}
+__device__ __forceinline__ int points_below(unsigned long long c, long long n, uint32_t u, unsigned long long C,
+                                            const PointScale& p) {
+  if (c == 0) return 0;
+  if (p.f > 0) {
+    const long long d = (long long)__umul64hi(c, p.F) - (long long)((unsigned long long)u >> (32 - p.f));
+    if (d >= 1) {
+      const long long r = (d - 1) & ((1ll << p.f) - 1), k = ((d - 1) >> p.f) + 1;
+      if (r + 3 <= (1ll << p.f)) return (int)(k < n ? k : n);
+    } else if (d <= -2) {
+      return 0;
+    }
+  }
+  return points_below_est(c, n, u, C);
+}
 
 template <typename T>
 __device__ __forceinline__ T exp_t(T v);
@@ -86,14 +99,14 @@ __device__ __forceinline__ unsigned long long quantize_u64(T W, int shift) {
 }
 
 // Q consecutive weights from w[i], zeros past n: 16-byte loads where `vec` (w on 16 bytes, i a
-// multiple of Q).
+// multiple of Q). Plain loads: the weights may have been written earlier in the same kernel.
 template <typename T, int Q>
-__device__ __forceinline__ void load_weights(const T* __restrict__ w, long long i, long long n, bool vec, T (&v)[Q]) {
+__device__ __forceinline__ void load_weights(const T* w, long long i, long long n, bool vec, T (&v)[Q]) {
   if (vec && i + Q <= n) {
     constexpr int V = 16 / (int)sizeof(T);
 #pragma unroll
     for (int q = 0; q < Q / V; ++q) {
-      const uint4 b = __ldg(reinterpret_cast<const uint4*>(w + i) + q);
+      const uint4 b = reinterpret_cast<const uint4*>(w + i)[q];
       memcpy(&v[q * V], &b, 16);
     }
   } else {
@@ -102,147 +115,109 @@ __device__ __forceinline__ void load_weights(const T* __restrict__ w, long long 
   }
 }
 
-// One tile of the `ntiles` tiles of one resampling, the tile taken by ticket.
-template <typename T>
-__device__ __forceinline__ void global_scan_scatter_body(const GlobalArgs<T>& a, long long ntiles) {
-  __shared__ int ks[SCAN_TILE + 1];  // systematic points below each item's cumulative count
-  __shared__ unsigned long long wsum[SCAN_NT / 32];
-  __shared__ unsigned long long s_prefix;
-  __shared__ long long s_tile;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-
-  if (tid == 0) {
-    const unsigned long long tk = atomicAdd(a.st.ticket, 1ull) - a.ticket_base;
-    s_tile = tk < (unsigned long long)ntiles ? (long long)tk : -1;
-    if (s_tile < 0) atomicOr(a.err, ERR_BOUNDS);
+// The exclusive prefix of CTA `bid`'s count total and the total C of the `nb` CTAs of OF_NT
+// threads, once every CTA's total is in place (block-wide: every thread receives both).
+__device__ __forceinline__ void count_prefix(const unsigned long long* ctot, int bid, int nb,
+                                             unsigned long long& pre, unsigned long long& C) {
+  constexpr int NW = OF_NT / 32;
+  __shared__ unsigned long long su[2][NW];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  unsigned long long p = 0, t = 0;
+  for (int b = tid; b < nb; b += OF_NT) {
+    const unsigned long long c = __ldcg(ctot + b);
+    t += c;
+    if (b < bid) p += c;
+  }
+  p = warp_sum(p);
+  t = warp_sum(t);
+  __syncthreads();
+  if (lane == 0) {
+    su[0][w] = p;
+    su[1][w] = t;
   }
   __syncthreads();
-  const long long tile = s_tile;
-  if (tile < 0) return;
-  const long long base = tile * SCAN_TILE;
-  const unsigned long long C = *a.C;
-  if (C == 0) return;  // no positive finite weight (flagged): in every tile, so none waits for another
-  const int shift = a.shift_dev ? *a.shift_dev : a.shift;
-  const uint32_t u = a.u_ptr ? *a.u_ptr : rand_word(a.key, a.t, 0, P_OUTER, 0);
-
-  // quantise this thread's items (blocked arrangement) and sum them
-  unsigned long long c[SCAN_IPT];
-  unsigned long long tsum = 0;
-  {
-    T W[SCAN_IPT];
-    load_weights<T, SCAN_IPT>(a.w, base + (long long)tid * SCAN_IPT, a.n, ((uintptr_t)a.w & 15) == 0, W);
+  pre = 0;
+  C = 0;
 #pragma unroll
-    for (int q = 0; q < SCAN_IPT; ++q) {
-      c[q] = quantize_u64(W[q], shift);
-      tsum += c[q];
-    }
-  }
-  // block exclusive scan of the per-thread sums
-  unsigned long long v = tsum;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long nb = __shfl_up_sync(FULL, v, o);
-    if (lane >= o) v += nb;
-  }
-  if (lane == 31) wsum[wid] = v;
-  __syncthreads();
-  unsigned long long wpre = 0, agg = 0;
-#pragma unroll
-  for (int q = 0; q < SCAN_NT / 32; ++q) {
-    if (q < wid) wpre += wsum[q];
-    agg += wsum[q];
-  }
-  const unsigned long long texcl = v - tsum + wpre;
-
-  // decoupled look-back for the tile's exclusive prefix: warp 0 publishes the
-  // tile's aggregate, then reads its predecessors' flags 32 at a time until it
-  // meets an inclusive prefix (every wait is bounded)
-  if (wid == 0) {
-    const uint32_t ep = a.epoch & 0x3FFFFFFFu;
-    unsigned long long prefix = 0;
-    if (tile == a.withhold) {
-      // publishes nothing: its successors' waits must run out and report
-    } else if (tile == 0) {
-      if (lane == 0) {
-        a.st.incl[0] = agg;
-        cuda::atomic_ref<uint32_t, cuda::thread_scope_device>(a.st.flags[0])
-            .store((ep << 2) | 2u, cuda::memory_order_release);
-      }
-    } else {
-      if (lane == 0) {
-        a.st.agg[tile] = agg;
-        cuda::atomic_ref<uint32_t, cuda::thread_scope_device>(a.st.flags[tile])
-            .store((ep << 2) | 1u, cuda::memory_order_release);
-      }
-      long long hi = tile - 1;
-      while (true) {
-        const long long j = hi - lane;
-        uint32_t fv = 0;
-        bool ready = true;
-        if (j >= 0) {
-          cuda::atomic_ref<uint32_t, cuda::thread_scope_device> f(a.st.flags[j]);
-          fv = f.load(cuda::memory_order_acquire);
-          ready = (fv >> 2) == ep && (fv & 3u) != 0u;
-          int spins = 0;
-          while (!ready && spins < SPIN_LIMIT) {
-            __nanosleep(64);
-            fv = f.load(cuda::memory_order_acquire);
-            ready = (fv >> 2) == ep && (fv & 3u) != 0u;
-            ++spins;
-          }
-        }
-        if (!__all_sync(FULL, ready)) {
-          if (lane == 0) atomicOr(a.err, ERR_TIMEOUT);
-          break;
-        }
-        const unsigned inc = __ballot_sync(FULL, j >= 0 && (fv & 3u) == 2u);
-        const int first = inc ? __ffs(inc) - 1 : 32;
-        unsigned long long val = 0;
-        if (j >= 0 && lane <= first) val = lane == first ? a.st.incl[j] : a.st.agg[j];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) val += __shfl_xor_sync(FULL, val, o);
-        prefix += val;
-        if (inc || hi < 32) break;
-        hi -= 32;
-      }
-      if (lane == 0) {
-        a.st.incl[tile] = prefix + agg;
-        cuda::atomic_ref<uint32_t, cuda::thread_scope_device>(a.st.flags[tile])
-            .store((ep << 2) | 2u, cuda::memory_order_release);
-      }
-    }
-    if (lane == 0) s_prefix = prefix;
-  }
-  __syncthreads();
-  // scatter: output k takes the item j of this tile with ks[j] <= k < ks[j + 1]. The exact 128-bit
-  // arithmetic is done once an item (the count of points below its cumulative count) and the
-  // search compares 32-bit counts; a search on cumulative counts took eleven 128-bit products
-  // an output (36 us of a call at n = 1,000,003)
-  unsigned long long run = s_prefix + texcl;
-  if (tid == 0) ks[0] = points_below_est(run, a.n, u, C);
-#pragma unroll
-  for (int q = 0; q < SCAN_IPT; ++q) {
-    run += c[q];
-    ks[tid * SCAN_IPT + q + 1] = points_below_est(run, a.n, u, C);
-  }
-  __syncthreads();
-  const int khi = ks[SCAN_TILE];
-  for (int k = ks[0] + tid; k < khi; k += SCAN_NT) {
-    int lo = 0, hi = SCAN_TILE;
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (ks[mid] <= k)
-        lo = mid;
-      else
-        hi = mid;
-    }
-    a.out[k] = (int32_t)(base + lo);
+  for (int r = 0; r < NW; ++r) {
+    pre += su[0][r];
+    C += su[1][r];
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(SCAN_NT) global_scan_scatter(GlobalArgs<T> a) {
-  global_scan_scatter_body<T>(a, gridDim.x);
+// The outputs of one CTA (OF_NT threads): items i0 .. iend - 1 of n, the CTAs before it holding `pre`
+// of the total count C > 0. Chunk by chunk (IPT consecutive items a thread): the items' counts
+// (load(i, W) gives a thread's weights, zeros past iend; quant the count of one), their scan, the
+// number of systematic points below each cumulative count, and then output k takes the item j with
+// ks[j] <= k < ks[j + 1]. The exact arithmetic is done once an item and the search compares 32-bit
+// counts. ks: OF_NT IPT + 1 ints, su: OF_NT / 32 words of shared memory.
+constexpr int SCATTER_IPT_LONG = 8;  // items a thread where a CTA owns many
+
+// SCALED: by the 64-bit product (points_below); else by the estimate alone, kept to one copy of its
+// 128-bit comparisons, which a kernel that runs once through its code has to fetch.
+template <typename T, int IPT, bool SCALED, class Load, class Quant>
+__device__ __forceinline__ void scatter_range(long long i0, long long iend, long long n, uint32_t u,
+                                              unsigned long long pre, unsigned long long C, const PointScale ps,
+                                              int32_t* out, int* ks, unsigned long long* su, Load load, Quant quant) {
+  constexpr int NW = OF_NT / 32, CHUNK = OF_NT * IPT;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  unsigned long long run = pre;
+  for (long long base = i0; base < iend; base += CHUNK) {
+    unsigned long long c[IPT], ts = 0;
+    T W[IPT];
+    load(base + tid * IPT, W);
+#pragma unroll
+    for (int q = 0; q < IPT; ++q) {
+      c[q] = quant(W[q]);
+      ts += c[q];
+    }
+    // exclusive block scan of the per-thread sums
+    unsigned long long incl = ts;
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+      const unsigned long long m = __shfl_up_sync(FULL, incl, s);
+      if (lane >= s) incl += m;
+    }
+    if (lane == 31) su[w] = incl;
+    __syncthreads();
+    unsigned long long wpre = 0, agg = 0;
+#pragma unroll
+    for (int r = 0; r < NW; ++r) {
+      if (r < w) wpre += su[r];
+      agg += su[r];
+    }
+    unsigned long long cum = run + wpre + incl - ts;
+    if constexpr (SCALED) {
+      if (tid == 0) ks[0] = points_below(run, n, u, C, ps);
+#pragma unroll
+      for (int q = 0; q < IPT; ++q) {
+        cum += c[q];
+        ks[tid * IPT + q + 1] = points_below(cum, n, u, C, ps);
+      }
+    } else {
+      static_assert(IPT == 2, "the short form");
+      const unsigned long long c0 = cum + c[0], c1 = c0 + c[1];
+#pragma unroll 1
+      for (int q = tid == 0 ? -1 : 0; q < 2; ++q)
+        ks[tid * 2 + q + 1] = points_below_est(q < 0 ? run : q == 0 ? c0 : c1, n, u, C);
+    }
+    __syncthreads();
+    // (an empty range is never hit, so j is never an item past the range, whose count is zero)
+    const int khi = ks[CHUNK];
+    for (int k = ks[0] + tid; k < khi; k += OF_NT) {
+      int lo = 0, hi = CHUNK;
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (ks[mid] <= k)
+          lo = mid;
+        else
+          hi = mid;
+      }
+      out[k] = (int32_t)(base + lo);
+    }
+    run += agg;
+    __syncthreads();  // ks and su are reused by the next chunk
+  }
 }
 
 }  // namespace dpf

@@ -62,10 +62,16 @@ void fill_outer_args(Ctx& x, double* mean_out, double* logz_out, unsigned int* a
     a.host_stats = x.host_out ? x.hstats_dev : nullptr;
   }
 
-template <typename T, int D1, int D2>
+template <typename T, int D1, int D2, bool PFSTAGE = false>
 dpf_status outer_stage(Ctx& x, double* mean_out, double* logz_out, cudaStream_t st) {
     FusedOuterArgs<T> a;
     fill_outer_args<T>(x, mean_out, logz_out, x.done + 1, &a);
+    if constexpr (PFSTAGE) {
+      if (x.pf && x.pf_rows) {
+        a.nwork = fused_outer_grid<T, D1, D2, true>(x.N);
+        return cuda_error(fused_outer_launch<T, D1, D2, true>(a, st), "outer stage launch");
+      }
+    }
     a.nwork = fused_outer_grid<T, D1, D2>(x.N);
     return cuda_error(fused_outer_launch<T, D1, D2>(a, st), "outer stage launch");
   }
@@ -361,7 +367,7 @@ struct VariantImpl {
   static int outer_ctas(long long N) { return fused_outer_grid<T, D1, D2>(N); }
 
   static dpf_status outer(Ctx& x, double* mean_out, double* logz_out, cudaStream_t st) {
-    return outer_stage<T, D1, D2>(x, mean_out, logz_out, st);
+    return outer_stage<T, D1, D2, (D2 <= 32)>(x, mean_out, logz_out, st);
   }
 
   // The outer sums of F filters of this variant in one launch (device arguments,

@@ -606,7 +606,7 @@ class Proposal:
 
 
 def check_bounded_wait(stream=None):
-    """Run the scan whose look-back can never finish (see ``dpf_check_bounded_wait``);
+    """Run an outer stage whose grid barrier can never be passed (see ``dpf_check_bounded_wait``);
     raises DpfError with status DPF_E_TIMEOUT when the waits give up as designed."""
     import torch
     s = stream if stream is not None else torch.cuda.current_stream().cuda_stream
