@@ -273,33 +273,6 @@ __global__ void __launch_bounds__(1024)
   }
 }
 
-// Sums over the warp of N values a lane, returned to every lane as out[0..N-1]. Halving: a
-// shuffle step exchanges half of the values still held for the other half of its partner's,
-// so a step costs half of the one before it (N = 8: 4 + 2 + 1 + 1 + 1 shuffles and one each to
-// hand out a total, not 40).
-template <int N, typename T>
-__device__ __forceinline__ T warp_sum_vec(const T (&v)[N], int lane) {
-  // lane l returns the total of value l mod NP (NP: N rounded up to a power of two)
-  constexpr int NP = N <= 1 ? 1 : N <= 2 ? 2 : N <= 4 ? 4 : N <= 8 ? 8 : N <= 16 ? 16 : 32;
-  static_assert(N <= 32, "one total a lane");
-  T w[NP];
-#pragma unroll
-  for (int q = 0; q < NP; ++q) w[q] = q < N ? v[q < N ? q : 0] : T(0);
-#pragma unroll
-  for (int h = NP / 2; h > 0; h /= 2) {
-    const bool up = (lane & h) != 0;
-#pragma unroll
-    for (int q = 0; q < h; ++q) {
-      const T give = up ? w[q] : w[q + h];
-      const T keep = up ? w[q + h] : w[q];
-      w[q] = keep + __shfl_xor_sync(FULL, give, h);
-    }
-  }
-#pragma unroll
-  for (int o = NP; o < 32; o <<= 1) w[0] += __shfl_xor_sync(FULL, w[0], o);
-  return w[0];
-}
-
 // The same step with one warp a group (M <= 256, rows of whole 16-byte units): each lane owns
 // PPL consecutive inner particles in registers, every reduction and scan is a warp shuffle, the
 // local resampling takes the offspring ranges (no search), and the ancestor's rows of the next
