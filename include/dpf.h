@@ -321,7 +321,8 @@ dpf_status dpf_set_debug(dpf_ctx* ctx, int32_t enable);
 /* Choose the tensor-core propagation z_new = A_zz z (3xTF32 on tcgen05, the
  * default) or the CUDA-core one, for variants that have both (FP32, d2 a
  * multiple of 8 with constants too large for a launch parameter, M = 128 or
- * 256; elsewhere the flag has no effect). Takes effect at the next step. */
+ * 256, L a multiple of 4; elsewhere the flag has no effect). Takes effect at
+ * the next step. */
 dpf_status dpf_set_tensor_cores(dpf_ctx* ctx, int32_t enable);
 
 /*

@@ -331,7 +331,9 @@ static void tg_launch(cudaStream_t s, bool overlap, int* err, const TgProb& a, c
   // memory that no more become resident (they would wait inside the allocation)
   const size_t floor_smem = g.ncols >= 64 ? 29 * 1024 : 0;
   const size_t smem = std::max((size_t)(128 + npad) * g.kc * (PREC == 0 ? 2 : 8), floor_smem);
-  cudaFuncSetAttribute(tgemm_kernel<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (the attribute belongs to the kernel: the largest any launch asks for, not this one's)
+  constexpr int most = (128 + 64) * tg_chunk<PREC>() * (PREC == 0 ? 2 : 8);
+  cudaFuncSetAttribute(tgemm_kernel<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   launch_after(s, overlap, (unsigned)(n0 + n1), TG_NT, smem, tgemm_kernel<PREC>, g);
 }
 

@@ -1140,7 +1140,7 @@ struct PaperVariant {
     const size_t wb = 4 * (size_t)o.total;
     if (x.grid_step == 0) {  // as many CTAs as fit on the device at once
       int nb = 0, dev = 0, nsm = 0;
-      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(wb * WARPS_PER_CTA));
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, WARP_MAX_SMEM);
       if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, WARPS_PER_CTA * 32, wb * WARPS_PER_CTA);
       if (e == cudaSuccess) e = cudaGetDevice(&dev);

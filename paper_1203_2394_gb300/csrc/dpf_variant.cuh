@@ -11,6 +11,10 @@
 
 namespace dpf {
 
+// The dynamic shared memory a kernel of many sizes is allowed, whatever the filter that sets it: the
+// attribute belongs to the kernel, so one filter's smaller need must not cut another's.
+constexpr int WARP_MAX_SMEM = 200 * 1024;
+
 constexpr int FEW_GROUPS = 16 * 152;  // one-warp CTAs: 16 fit on an SM at 128 registers a thread
 
 inline int threads_for(int M) { return ((M + 31) / 32) * 32; }
@@ -153,7 +157,7 @@ struct VariantImpl {
     auto k = step_kernel<T, D1, D2, DY, XZ, PPT, MAXNT, BULK>;
     static bool attr_done = false;
     if (!attr_done) {
-      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, WARP_MAX_SMEM);
       if (e != cudaSuccess) return cuda_error(e, "cudaFuncSetAttribute");
       attr_done = true;
     }
@@ -177,7 +181,7 @@ struct VariantImpl {
     auto k = step_warp_kernel<T, D1, D2, DY, XZ, PPL, MF>;
     static bool attr_done = false;
     if (!attr_done) {
-      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, WARP_MAX_SMEM);
       if (e != cudaSuccess) return cuda_error(e, "cudaFuncSetAttribute");
       attr_done = true;
     }
@@ -319,7 +323,7 @@ struct VariantImpl {
     auto k = step_warp_batch_kernel<T, D1, D2, DY, XZ, PPL, SHARED, MF>;
     static bool attr_done = false;
     if (!attr_done) {
-      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, WARP_MAX_SMEM);
       if (e != cudaSuccess) return cuda_error(e, "cudaFuncSetAttribute");
       attr_done = true;
     }
@@ -428,7 +432,7 @@ struct VariantImpl {
     const int nw = x.N <= FEW_GROUPS ? 1 : WARPS_PER_CTA;
     if (x.grid_step == 0 || x.grid_kernel != (const void*)k) {  // as many CTAs as fit on the device at once
       int nb = 0, dev = 0, nsm = 0;
-      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(wb * WARPS_PER_CTA));
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, WARP_MAX_SMEM);
       if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, WARPS_PER_CTA * 32, wb * WARPS_PER_CTA);
       if (e == cudaSuccess) e = cudaGetDevice(&dev);
@@ -484,7 +488,7 @@ struct VariantImpl {
     a.gauss = x.std_gauss ? 1 : 0;
     a.dbg_b = x.debug ? x.dbg_b : nullptr;
     a.dbg_j = x.debug ? x.dbg_j : nullptr;
-    if (!a.gauss && warp_path(x.M, 16) && std_warp_smem<T, D1, D2>(x.M, x.xp) * WARPS_PER_CTA <= 200 * 1024) {
+    if (!a.gauss && warp_path(x.M, 16) && std_warp_smem<T, D1, D2>(x.M, x.xp) * WARPS_PER_CTA <= WARP_MAX_SMEM) {
       if constexpr (XZM == 1) return launch_std<true>(x, a);
       else return use_xz(x) ? launch_std<true>(x, a) : launch_std<false>(x, a);
     }

@@ -49,8 +49,11 @@ struct WideVariantImpl {
     return cuda_error(cudaGetLastError(), "init kernel launch");
   }
 
+  // The tensor-core step stages a group's rows by bulk copies, which take whole 16-byte units: a row
+  // of L look-ahead weights is one when L is a multiple of 4, and other L take the CUDA-core form
+  // (whose loads are plain; any other size would fault).
   static dpf_status launch(Ctx& x, StepArgs<T>& a, cudaStream_t s) {
-    return x.tensor_cores && tc_shape(x.M) ? wide_launch<T, D1, D2, DY, true>(x, a, s)
+    return x.tensor_cores && tc_shape(x.M) && x.L % 4 == 0 ? wide_launch<T, D1, D2, DY, true>(x, a, s)
                                            : wide_launch<T, D1, D2, DY, false>(x, a, s);
   }
 
