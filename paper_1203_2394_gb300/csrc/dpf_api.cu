@@ -68,8 +68,11 @@ static cudaMemPool_t scratch_pool() {
 dpf_status scratch_alloc(Scratch& sc, int ctas, cudaStream_t s) {
   cudaMemPool_t pool = scratch_pool();
   void* p = nullptr;
-  cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, scratch_bytes(ctas), pool, s)
-                       : cudaMallocAsync(&p, scratch_bytes(ctas), s);
+  cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, scratch_bytes(ctas), pool, s) : cudaErrorMemoryAllocation;
+  if (e != cudaSuccess) {  // (on a full device the default pool may still hold free memory)
+    if (pool) cudaGetLastError();
+    e = cudaMallocAsync(&p, scratch_bytes(ctas), s);
+  }
   if (e != cudaSuccess) return cuda_error(e, "scratch allocation");
   scratch_layout(sc, p, ctas);
   return DPF_OK;
