@@ -27,11 +27,14 @@ struct Scratch {
   unsigned long long* keys = nullptr;    // one a CTA: its largest weight's bits, ~0 for a bad weight
   unsigned long long* totals = nullptr;  // one a CTA: its count total
 };
-// CTAs of the global rule's passes over n weights, each a contiguous range of 512-item chunks.
+// CTAs of the global rule's passes over n weights, each a contiguous range of 512-item chunks:
+// four an SM as long as each has at most one 2048-item chunk of the scatter (which is then nearly
+// full, and its prefix has half as many totals to read), up to eight an SM for larger sets.
 constexpr int RS_MAX_CTAS = 8 * 152;
 inline int resample_ctas(long long n) {
-  const long long nch = (n + 511) / 512;
-  return (int)(nch < RS_MAX_CTAS ? nch : RS_MAX_CTAS);
+  const long long nch = (n + 511) / 512, full = (n + 2047) / 2048;
+  const long long want = full < RS_MAX_CTAS / 2 ? RS_MAX_CTAS / 2 : full < RS_MAX_CTAS ? full : RS_MAX_CTAS;
+  return (int)(nch < want ? nch : want);
 }
 constexpr size_t scratch_bytes(int ctas) { return 64 + (size_t)ctas * 16; }
 // The parts of a block of scratch_bytes(ctas).

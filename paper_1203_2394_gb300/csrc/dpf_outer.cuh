@@ -141,7 +141,7 @@ template <typename T, bool PF>
 __device__ __forceinline__ void outer_scatter(const FusedOuterArgs<T>& a, int bid, int nb, T lwmax,
                                               unsigned long long pre, unsigned long long C) {
   __shared__ unsigned long long su[OF_NT / 32];
-  __shared__ int ks[OF_NT * (PF ? SCATTER_IPT_LONG : OF_IPT) + 1];
+  __shared__ __align__(16) int slots[OF_NT * (PF ? SCATTER_IPT_LONG : OF_IPT)];
   const OuterArgs<T>& o = a.o;
   const long long N = o.N;
   const T sS = pow2_t<T>(a.shift);
@@ -158,7 +158,7 @@ __device__ __forceinline__ void outer_scatter(const FusedOuterArgs<T>& a, int bi
       auto load = [&](long long i, T (&W)[SCATTER_IPT_LONG]) {
         load_weights<T, SCATTER_IPT_LONG>(a.w_out, i, iend, true, W);
       };
-      scatter_range<T, SCATTER_IPT_LONG, true>(i0, iend, N, u, pre, C, s_ps, a.anc, ks, su, load, quant);
+      scatter_range<T, SCATTER_IPT_LONG, true>(i0, iend, N, u, pre, C, s_ps, a.anc, slots, su, load, quant);
       return;
     }
   }
@@ -172,7 +172,7 @@ __device__ __forceinline__ void outer_scatter(const FusedOuterArgs<T>& a, int bi
       }
     }
   };
-  scatter_range<T, OF_IPT, false>(i0, iend, N, u, pre, C, PointScale{0ull, -1}, a.anc, ks, su, load, quant);
+  scatter_range<T, OF_IPT, false>(i0, iend, N, u, pre, C, PointScale{0ull, -1}, a.anc, slots, su, load, quant);
 }
 
 // ---- D: the statistics from the `nb` CTAs' partial sums, by one CTA once they are

@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(OF_NT)
     resample_scatter_kernel(const T* w, long long n, const uint32_t* up, const unsigned long long* keys,
                             const unsigned long long* totals, int32_t* out, int* err) {
   __shared__ unsigned long long su[OF_NT / 32];
-  __shared__ int ks[OF_NT * SCATTER_IPT_LONG + 1];
+  __shared__ __align__(16) int slots[OF_NT * SCATTER_IPT_LONG];
   __shared__ PointScale s_ps;
   int shift = 0;
   const bool ok = rs_shift<T>(keys, gridDim.x, n, shift);
@@ -137,10 +137,10 @@ __global__ void __launch_bounds__(OF_NT)
     auto load = [&](long long i, T (&W)[SCATTER_IPT_LONG]) {
       load_weights<T, SCATTER_IPT_LONG>(w, i, r.iend, vec, W);
     };
-    scatter_range<T, SCATTER_IPT_LONG, true>(r.i0, r.iend, n, *up, pre, C, s_ps, out, ks, su, load, quant);
+    scatter_range<T, SCATTER_IPT_LONG, true>(r.i0, r.iend, n, *up, pre, C, s_ps, out, slots, su, load, quant);
   } else {
     auto load = [&](long long i, T (&W)[OF_IPT]) { load_weights<T, OF_IPT>(w, i, r.iend, false, W); };
-    scatter_range<T, OF_IPT, false>(r.i0, r.iend, n, *up, pre, C, s_ps, out, ks, su, load, quant);
+    scatter_range<T, OF_IPT, false>(r.i0, r.iend, n, *up, pre, C, s_ps, out, slots, su, load, quant);
   }
 }
 

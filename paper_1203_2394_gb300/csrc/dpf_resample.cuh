@@ -5,6 +5,7 @@
 
 #include <cuda/atomic>
 #include <cstring>
+#include <type_traits>
 
 #include "dpf_common.cuh"
 #include "dpf_internal.h"
@@ -149,8 +150,12 @@ __device__ __forceinline__ void count_prefix(const unsigned long long* ctot, int
 // of the total count C > 0. Chunk by chunk (IPT consecutive items a thread): the items' counts
 // (load(i, W) gives a thread's weights, zeros past iend; quant the count of one), their scan, the
 // number of systematic points below each cumulative count, and then output k takes the item j with
-// ks[j] <= k < ks[j + 1]. The exact arithmetic is done once an item and the search compares 32-bit
-// counts. ks: OF_NT IPT + 1 ints, su: OF_NT / 32 words of shared memory.
+// K[j] <= k < K[j + 1]. That last step is a warp's own: its 32 IPT items own a contiguous range of
+// outputs, taken in windows of 32 IPT; every item with outputs marks its first one, a maximum scan
+// over the window (eight slots a lane, then shuffles) carries the marks forward, and the window
+// leaves in whole lines. What bounds it is shared memory and latency: a binary search among the
+// block's counts read 11 words an output, one after another, where this moves about one and a half,
+// and it has no block barrier. slots: OF_NT IPT ints on 16 bytes, su: OF_NT / 32 words of shared memory.
 constexpr int SCATTER_IPT_LONG = 8;  // items a thread where a CTA owns many
 
 // SCALED: by the 64-bit product (points_below); else by the estimate alone, kept to one copy of its
@@ -158,9 +163,13 @@ constexpr int SCATTER_IPT_LONG = 8;  // items a thread where a CTA owns many
 template <typename T, int IPT, bool SCALED, class Load, class Quant>
 __device__ __forceinline__ void scatter_range(long long i0, long long iend, long long n, uint32_t u,
                                               unsigned long long pre, unsigned long long C, const PointScale ps,
-                                              int32_t* out, int* ks, unsigned long long* su, Load load, Quant quant) {
-  constexpr int NW = OF_NT / 32, CHUNK = OF_NT * IPT;
+                                              int32_t* out, int* slots, unsigned long long* su, Load load, Quant quant) {
+  constexpr int NW = OF_NT / 32, CHUNK = OF_NT * IPT, WIN = 32 * IPT;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  int* const slot = slots + w * WIN;
+  typedef typename std::conditional<IPT % 4 == 0, int4, int2>::type Vec;
+  constexpr int VI = (int)sizeof(Vec) / 4;
+  static_assert(IPT % VI == 0, "whole vectors a lane");
   unsigned long long run = pre;
   for (long long base = i0; base < iend; base += CHUNK) {
     unsigned long long c[IPT], ts = 0;
@@ -187,36 +196,81 @@ __device__ __forceinline__ void scatter_range(long long i0, long long iend, long
       agg += su[r];
     }
     unsigned long long cum = run + wpre + incl - ts;
+    int K[IPT + 1];  // points below each of the thread's items, and below the one after them
+    K[0] = 0;
     if constexpr (SCALED) {
-      if (tid == 0) ks[0] = points_below(run, n, u, C, ps);
+      if (lane == 0) K[0] = points_below(cum, n, u, C, ps);
 #pragma unroll
       for (int q = 0; q < IPT; ++q) {
         cum += c[q];
-        ks[tid * IPT + q + 1] = points_below(cum, n, u, C, ps);
+        K[q + 1] = points_below(cum, n, u, C, ps);
       }
     } else {
       static_assert(IPT == 2, "the short form");
       const unsigned long long c0 = cum + c[0], c1 = c0 + c[1];
 #pragma unroll 1
-      for (int q = tid == 0 ? -1 : 0; q < 2; ++q)
-        ks[tid * 2 + q + 1] = points_below_est(q < 0 ? run : q == 0 ? c0 : c1, n, u, C);
-    }
-    __syncthreads();
-    // (an empty range is never hit, so j is never an item past the range, whose count is zero)
-    const int khi = ks[CHUNK];
-    for (int k = ks[0] + tid; k < khi; k += OF_NT) {
-      int lo = 0, hi = CHUNK;
-      while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (ks[mid] <= k)
-          lo = mid;
-        else
-          hi = mid;
+      for (int q = lane == 0 ? -1 : 0; q < 2; ++q) {
+        const int v = points_below_est(q < 0 ? cum : q == 0 ? c0 : c1, n, u, C);
+        if (q < 0) K[0] = v;
+        else if (q == 0) K[1] = v;
+        else K[2] = v;
       }
-      out[k] = (int32_t)(base + lo);
+      __syncwarp();
+    }
+    {
+      const int before = __shfl_up_sync(FULL, K[IPT], 1);
+      if (lane > 0) K[0] = before;
+    }
+    const int kbeg = __shfl_sync(FULL, K[0], 0), kend = __shfl_sync(FULL, K[IPT], 31);
+    int carry = -1;  // the item whose outputs reach into the window (the first window starts with a mark)
+    for (int k0 = kbeg, left = kend - kbeg; left > 0; left -= WIN, k0 = (int)((unsigned)k0 + WIN)) {
+      int v[IPT];
+#pragma unroll
+      for (int q = 0; q < IPT; ++q) v[q] = -1;
+#pragma unroll
+      for (int q = 0; q < IPT; q += VI) {
+        Vec x;
+        memcpy(&x, v + q, sizeof(Vec));
+        *reinterpret_cast<Vec*>(slot + lane * IPT + q) = x;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < IPT; ++q)
+        if (K[q + 1] > K[q] && (unsigned)(K[q] - k0) < (unsigned)WIN) slot[K[q] - k0] = lane * IPT + q;
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < IPT; q += VI) {
+        const Vec x = *reinterpret_cast<const Vec*>(slot + lane * IPT + q);
+        memcpy(v + q, &x, sizeof(Vec));
+      }
+#pragma unroll
+      for (int q = 1; q < IPT; ++q) v[q] = max(v[q], v[q - 1]);
+      int m = max(v[IPT - 1], carry);
+#pragma unroll
+      for (int s = 1; s < 32; s <<= 1) {
+        const int o = __shfl_up_sync(FULL, m, s);
+        if (lane >= s) m = max(m, o);
+      }
+      const int o = __shfl_up_sync(FULL, m, 1), first = lane > 0 ? o : carry;
+      carry = __shfl_sync(FULL, m, 31);
+#pragma unroll
+      for (int q = 0; q < IPT; ++q) v[q] = max(v[q], first);
+#pragma unroll
+      for (int q = 0; q < IPT; q += VI) {
+        Vec x;
+        memcpy(&x, v + q, sizeof(Vec));
+        *reinterpret_cast<Vec*>(slot + lane * IPT + q) = x;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < IPT; ++q) {
+        const int e = lane + 32 * q;
+        if (e < left) out[k0 + e] = (int32_t)(base + w * WIN) + slot[e];
+      }
+      __syncwarp();  // the slots are written again by the next window
     }
     run += agg;
-    __syncthreads();  // ks and su are reused by the next chunk
+    __syncthreads();  // su is reused by the next chunk
   }
 }
 
