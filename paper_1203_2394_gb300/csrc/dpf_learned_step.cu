@@ -770,21 +770,25 @@ static uint32_t scale_for(int n) {
 // + sum log s + log p(y_t | x_t, z).
 
 // Selection, local resampling and the group features; one warp per outer particle,
-// PP = M / 32 consecutive inner particles a lane.
+// PP = M / 32 consecutive inner particles a lane. Bound by the latency of its chain (ancestor, rows,
+// scans, gather): a lane's rows move as one vector, one Philox evaluation serves the selection (lane
+// 0) and the resampling, and the ancestors come from the sources' ranges (no search).
 template <int D1, int D2, int DY, bool XZ, int PP>
 __global__ void __launch_bounds__(128)
     oa_prepare_kernel(const __grid_constant__ MC<float, D1, D2, DY> mc, const __grid_constant__ StepArgs<float> a,
                       int32_t* __restrict__ bidx_out, float* __restrict__ feat, int din) {
   constexpr int M = 32 * PP;
-  __shared__ uint32_t cum_s[4][M];
+  __shared__ __align__(16) int slot_s[4][M];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long g = blockIdx.x * 4LL + w;
   if (g >= a.N) return;  // whole warps only
-  uint32_t* cum = cum_s[w];
   const float NEG = -INFINITY;
   const long long NM = a.N * (long long)M;
   const int anc_g = a.anc[g];
   const int L = a.L;
+  const int k0 = lane * PP;
+  const uint32_t word = philox(ctr(a.t - 1, (uint32_t)g, lane == 0 ? P_SEL : P_INNER, 0u, 0u), a.key).x;
+  const uint32_t uin = __shfl_sync(FULL, word, 1);
   int msel;
   {
     const float l0 = lane < L ? a.lwh_old[(long long)anc_g * L + lane] : NEG;
@@ -803,7 +807,7 @@ __global__ void __launch_bounds__(128)
     }
     const uint32_t tot0 = __shfl_sync(FULL, s0, 31), tot1 = __shfl_sync(FULL, s1, 31);
     const uint64_t Cs = (uint64_t)tot0 + tot1;
-    const uint32_t usel = philox(ctr(a.t - 1, (uint32_t)g, P_SEL, 0u, 0u), a.key).x;
+    const uint32_t usel = __shfl_sync(FULL, word, 0);
     const uint64_t rhs = (uint64_t)usel * Cs;
     const unsigned b0 = __ballot_sync(FULL, ((uint64_t)s0 << 32) > rhs);
     const unsigned b1 = __ballot_sync(FULL, ((uint64_t)(s1 + tot0) << 32) > rhs);
@@ -835,24 +839,26 @@ __global__ void __launch_bounds__(128)
   }
   float al[PP];
   float amax = NEG;
+  vld<float, PP>(a.lq_old + (long long)anc_g * M + k0, al);
+  if (XZ) {
+    float zc[D2][PP];
 #pragma unroll
-  for (int p = 0; p < PP; ++p) {
-    const int k = lane * PP + p;
-    float v0 = a.lq_old[(long long)anc_g * M + k];
-    if (XZ) {
+    for (int c = 0; c < D2; ++c) vld<float, PP>(a.z_old + c * NM + (long long)anc_g * M + k0, zc[c]);
+#pragma unroll
+    for (int p = 0; p < PP; ++p) {
       float q = 0.f;
 #pragma unroll
       for (int r = 0; r < D1; ++r) {
         float v = wres[r];
 #pragma unroll
-        for (int c = 0; c < D2; ++c) v -= mc.WAxz[r][c] * a.z_old[c * NM + (long long)anc_g * M + k];
+        for (int c = 0; c < D2; ++c) v -= mc.WAxz[r][c] * zc[c][p];
         q += v * v;
       }
-      v0 -= 0.5f * q;
+      al[p] -= 0.5f * q;
     }
-    al[p] = v0;
-    amax = fmaxf(amax, v0);
   }
+#pragma unroll
+  for (int p = 0; p < PP; ++p) amax = fmaxf(amax, al[p]);
   amax = warp_max(amax);
   uint32_t loc[PP];
   uint32_t run = 0;
@@ -868,21 +874,20 @@ __global__ void __launch_bounds__(128)
     if (lane >= o) inc += n;
   }
 #pragma unroll
-  for (int p = 0; p < PP; ++p) cum[lane * PP + p] = loc[p] + inc - run;
-  __syncwarp();
-  const uint32_t C = cum[M - 1];
+  for (int p = 0; p < PP; ++p) loc[p] += inc - run;
+  const uint32_t C = __shfl_sync(FULL, inc, 31);
   if (C == 0 && lane == 0) atomicOr(a.err, ERR_NUMERIC);
-  const uint32_t uin = philox(ctr(a.t - 1, (uint32_t)g, P_INNER, 0u, 0u), a.key).x;
+  int bidx[PP];
+  sys_local_offspring<PP>(loc, C, M, uin >> 16, k0, true, lane, slot_s[w], bidx);
+  vst<int, PP>(bidx_out + g * M + k0, bidx);
+  if (a.dbg_b) vst<int, PP>(a.dbg_b + g * M + k0, bidx);
   float mu[PP][D2];
   float msum[D2];
 #pragma unroll
   for (int d = 0; d < D2; ++d) msum[d] = 0.f;
 #pragma unroll
   for (int p = 0; p < PP; ++p) {
-    const int k = lane * PP + p;
-    const int b = sys_local_pick(cum, M, C, M, k, uin);
-    bidx_out[g * M + k] = b;
-    if (a.dbg_b) a.dbg_b[g * M + k] = b;
+    const int b = bidx[p];
     float zb[D2];
 #pragma unroll
     for (int c = 0; c < D2; ++c) zb[c] = a.z_old[c * NM + (long long)anc_g * M + b];
@@ -956,10 +961,11 @@ __global__ void __launch_bounds__(128)
   h_x(mc, xt, hx);
   float z[PP][D2], lr[PP];
   float lmax = NEG;
+  int bs[PP];
+  vld<int, PP>(bidx + g * M + lane * PP, bs);
 #pragma unroll
   for (int p = 0; p < PP; ++p) {
-    const int k = lane * PP + p;
-    const int b = bidx[g * M + k];
+    const int k = lane * PP + p, b = bs[p];
     float zb[D2], mu[D2];
 #pragma unroll
     for (int c = 0; c < D2; ++c) zb[c] = a.z_old[c * NM + (long long)anc_g * M + b];
@@ -1019,14 +1025,18 @@ __global__ void __launch_bounds__(128)
   for (int p = 0; p < PP; ++p) se += expf(lr[p] - lmax);
   const float lse = lmax + logf(warp_sum(se));
 #pragma unroll
-  for (int p = 0; p < PP; ++p) {
-    const int k = lane * PP + p;
+  for (int d = 0; d < D2; ++d) {
+    float zd[PP];
 #pragma unroll
-    for (int d = 0; d < D2; ++d) a.z_new[d * NM + g * M + k] = z[p][d];
-    const float lq = lr[p] - lse;
-    a.lq_new[g * M + k] = lq;
-    if (!(lq == lq)) atomicOr(a.err, ERR_NUMERIC);
+    for (int p = 0; p < PP; ++p) zd[p] = z[p][d];
+    vst<float, PP>(a.z_new + d * NM + g * M + lane * PP, zd);
   }
+#pragma unroll
+  for (int p = 0; p < PP; ++p) {
+    lr[p] -= lse;
+    if (!(lr[p] == lr[p])) atomicOr(a.err, ERR_NUMERIC);
+  }
+  vst<float, PP>(a.lq_new + g * M + lane * PP, lr);
 }
 
 // Training rows of the amortised proposal from the last inner update: one warp per
@@ -1141,24 +1151,36 @@ static dpf_status oa_step_pp(Ctx& x, const MC<float, 2, 2, 2>& mc, StepArgs<floa
 // The per-group fallback: the inner effective sample size of each group's learned
 // update, ESS = (sum_j W_j)^2 / sum_j W_j^2 with W = exp(lq), against thr = fb_frac M.
 // Groups below it (or with no finite weight) are flagged and listed (in no particular
-// order) for the plain inner update; one warp a group.
+// order) for the plain inner update. A warp takes FB_GROUPS groups, their rows in flight together:
+// with a group a warp the kernel was as many launches of CTAs as reads.
+constexpr int FB_GROUPS = 4;
 __global__ void fallback_lists_kernel(const float* __restrict__ lq, long long N, int M, float thr,
                                       int32_t* flag, int32_t* list, int32_t* count) {
-  const long long i = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const long long i0 = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * FB_GROUPS;
   const int lane = threadIdx.x & 31;
-  if (i >= N) return;  // whole warps
-  float s1 = 0.f, s2 = 0.f;
+  if (i0 >= N) return;  // whole warps
+  float s1[FB_GROUPS], s2[FB_GROUPS];
+#pragma unroll
+  for (int r = 0; r < FB_GROUPS; ++r) s1[r] = s2[r] = 0.f;
   for (int k = lane; k < M; k += 32) {
-    const float w = expf(lq[i * M + k]);
-    s1 += w;
-    s2 += w * w;
+    float v[FB_GROUPS];
+#pragma unroll
+    for (int r = 0; r < FB_GROUPS; ++r) v[r] = i0 + r < N ? lq[(i0 + r) * M + k] : 0.f;
+#pragma unroll
+    for (int r = 0; r < FB_GROUPS; ++r) {
+      const float w = expf(v[r]);
+      s1[r] += w;
+      s2[r] += w * w;
+    }
   }
-  s1 = warp_sum(s1);
-  s2 = warp_sum(s2);
-  if (lane == 0) {
-    const bool fb = !(s1 * s1 >= thr * s2);
-    flag[i] = fb ? 1 : 0;
-    if (fb) list[atomicAdd(count, 1)] = (int32_t)i;
+#pragma unroll
+  for (int r = 0; r < FB_GROUPS; ++r) {
+    const float t1 = warp_sum(s1[r]), t2 = warp_sum(s2[r]);
+    if (lane == 0 && i0 + r < N) {
+      const bool fb = !(t1 * t1 >= thr * t2);
+      flag[i0 + r] = fb ? 1 : 0;
+      if (fb) list[atomicAdd(count, 1)] = (int32_t)(i0 + r);
+    }
   }
 }
 
@@ -1168,7 +1190,7 @@ dpf_status learned_fallback_lists(Ctx& x) {
     return cuda_error(cudaMemsetAsync(x.fb_flag, 0, sizeof(int32_t) * x.N, x.stream), "fallback flags");
   cudaError_t e = cudaMemsetAsync(x.fb_count, 0, sizeof(int32_t), x.stream);
   if (e != cudaSuccess) return cuda_error(e, "fallback counts");
-  const unsigned blocks = (unsigned)((x.N + 3) / 4);
+  const unsigned blocks = (unsigned)((x.N + 4 * FB_GROUPS - 1) / (4 * FB_GROUPS));
   fallback_lists_kernel<<<blocks, 128, 0, x.stream>>>((const float*)x.lq[(t + 1) % 2], x.N, x.M,
                                                       (float)(x.fb_frac * x.M), x.fb_flag, x.fb_list,
                                                       x.fb_count);
