@@ -48,15 +48,11 @@ constexpr size_t PK_BYTES = PK_B + sizeof(float) * (3 * LH + LNP);
 // 256..511). The first 256 compute threads hold one row each; the hidden layers' epilogues are
 // shared by LSPLIT threads a row (each a range of columns). One more warp feeds the weight ring.
 //
-// The weights reach the ring by multicast: the LCL CTAs of a cluster walk the same chunks in step,
-// each copies 1 / LCL of a chunk from L2 into all of their rings, and a stage is refilled when
-// the MMAs of every CTA of the cluster have read it. Alone, each of 152 SMs fetched the same 128 KB a
-// layer, and a 16 KB copy took 6,000 cycles whatever the ring's depth: the streamed layers ran
-// at 3.6 times their MMA time (together with the polls, see wait_products). With both gone the
-// layers run at the pace of their MMAs: 1,000,003 rows 929 us, now 372 (298 and 744 TFLOP/s).
-// Clusters of 4 left some SMs out (140 of 152 busy) and were no faster.
+// Every CTA copies the weights it streams (256 KB for 256 rows) into its own ring by plain bulk
+// copies: 1.0 GB from L2 for 1,000,003 rows, 2.8 TB/s at the 370 us they take (928 us with eight
+// warps polling, see wait_products, and unswizzled tiles). Copies shared by a cluster of two took 371 us:
+// what the L2 delivers is not what bounds the layers.
 constexpr int LROWS = 256;
-constexpr int LCL = 2;  // CTAs of a cluster
 template <int MODE>
 constexpr int learned_split() { return MODE == 0 ? 2 : 1; }  // the filter's pass needs 136 registers a thread
 template <int MODE>
@@ -93,32 +89,6 @@ __device__ __forceinline__ void wait_products(uint64_t* mbar, uint32_t& phase, b
   tc::fence_before();
   all_sync<NT>();
   tc::fence_after();
-}
-
-// ---- cluster pieces: rank, barrier, multicast copy and commit (the same shared-memory offsets in
-// every CTA of the mask) ----
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void bulk_load_multicast(void* dst, const void* src, uint32_t bytes, uint64_t* b,
-                                                    uint16_t mask) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1], %2, [%3], %4;" ::
-          "r"(smem_addr(dst)),
-      "l"(src), "r"(bytes), "r"(smem_addr(b)), "h"(mask)
-      : "memory");
-}
-__device__ __forceinline__ void commit_multicast(uint64_t* bar, uint16_t mask) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-          smem_addr(bar)),
-      "h"(mask)
-      : "memory");
 }
 
 // Pack one FP32 matrix (rows x cols, row-major) into BF16 K-major chunks of kch
@@ -291,19 +261,14 @@ __global__ void __launch_bounds__(learned_threads<MODE>(), 1)
   const int M = MODE == 1 ? a.M : 128;
   const long long rows_total = MODE == 1 ? a.N * (long long)a.M : la.nrows;
   const long long niters = (rows_total + LROWS - 1) / LROWS;
-  // every CTA of a cluster runs as many iterations as its first one (some on no live row), so that
-  // they walk the weights' chunks together
-  const uint32_t rank = cluster_rank();
-  const long long first = (long long)blockIdx.x - rank;
-  const long long my_iters = niters > first ? (niters - 1 - first) / gridDim.x + 1 : 0;
-  constexpr uint16_t all_ctas = (uint16_t)((1u << LCL) - 1u);
+  const long long my_iters = niters > blockIdx.x ? (niters - 1 - blockIdx.x) / gridDim.x + 1 : 0;
   const long long total_chunks = my_iters * 2 * LNCH;
 
   // ---- set-up: barriers, TMEM, resident weights and biases ----
   if (tid == 0) {
     for (int s = 0; s < LSTAGES; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], LCL);
+      mbar_init(&empty[s], 1);
     }
     mbar_init(&mbar, 1);
     mbar_fence_init();
@@ -320,7 +285,6 @@ __global__ void __launch_bounds__(learned_threads<MODE>(), 1)
   tc::fence_proxy_async();
   tc::fence_before();
   __syncthreads();
-  cluster_sync_all();  // every CTA's barriers are set up before another one's copies or commits arrive
   tc::fence_after();
   const uint32_t taddr = s_taddr;
   // this thread's accumulator row: lanes 32 (w % 4) .., columns 256 half ..
@@ -330,6 +294,7 @@ __global__ void __launch_bounds__(learned_threads<MODE>(), 1)
   if (w == NCT / 32) {
     // ---- producer warp: refill each ring stage as soon as its MMAs are done ----
     if (lane == 0) {
+      long long issued = 0;
       for (long long c = 0; c < total_chunks; ++c) {
         const int s = (int)(c % LSTAGES);
         if (c >= LSTAGES && !tc::bar_wait(&empty[s], (uint32_t)(((c / LSTAGES) - 1) & 1), L_SPIN)) {
@@ -339,14 +304,15 @@ __global__ void __launch_bounds__(learned_threads<MODE>(), 1)
         const int q = (int)(c % (2 * LNCH));
         const unsigned char* src =
             la.wp + (q < LNCH ? PK_W2 + (size_t)q * LCHUNK : PK_W3 + (size_t)(q - LNCH) * LCHUNK);
-        // this CTA's part of the chunk, into the same stage of every CTA of the cluster
-        constexpr uint32_t part = LCHUNK / LCL;
         mbar_arrive_tx(&full[s], LCHUNK);
-        bulk_load_multicast(sm + SM_RING + s * LCHUNK + rank * part, src + rank * part, part, &full[s], all_ctas);
+        bulk_load(sm + SM_RING + s * LCHUNK, src, LCHUNK, &full[s]);
+        issued = c + 1;
       }
-      // wait until the last chunks' MMAs have released their stages, so that no
-      // copy is in flight when the kernel ends
-      for (long long c = std::max<long long>(0, total_chunks - LSTAGES); c < total_chunks && ok; ++c)
+      // wait until the last chunks' copies have landed and their MMAs have released their stages, so
+      // that neither is in flight when the kernel ends (the copies also when a wait has given up)
+      for (long long c = std::max<long long>(0, issued - LSTAGES); c < issued; ++c)
+        if (!tc::bar_wait(&full[c % LSTAGES], (uint32_t)((c / LSTAGES) & 1), L_SPIN)) ok = false;
+      for (long long c = std::max<long long>(0, issued - LSTAGES); c < issued && ok; ++c)
         if (!tc::bar_wait(&empty[c % LSTAGES], (uint32_t)((c / LSTAGES) & 1), L_SPIN)) ok = false;
     }
   } else {
@@ -547,7 +513,7 @@ __global__ void __launch_bounds__(learned_threads<MODE>(), 1)
               tc::mma_f16(taddr + h * LH,
                           act_desc(s_act0 + h * (128 * LH * 2), k * (LKCH / 16) + ks),
                           tc::smem_desc_sw(sb + (uint32_t)ks * 32u, tc::LAYOUT_SW64), id_h, (k > 0 || ks > 0) ? 1u : 0u);
-          commit_multicast(&empty[s], all_ctas);  // the stage may be refilled once every CTA's MMAs are done
+          tc::commit(&empty[s]);  // the producer refills the stage once these MMAs are done
         }
         tc::commit(&mbar);
       }
@@ -718,7 +684,6 @@ __global__ void __launch_bounds__(learned_threads<MODE>(), 1)
   tc::fence_before();
   __syncthreads();
   if (w == 0) tc::tmem_dealloc(taddr, LTMEM_COLS);
-  cluster_sync_all();  // no CTA leaves while another may still signal its barriers
 }
 
 template <int MODE, int D1, int D2, int DY, bool XZ, int NC>
@@ -731,30 +696,13 @@ static dpf_status launch_learned(const MC<float, D1, D2, DY>& mc, const StepArgs
     if (e != cudaSuccess) return cuda_error(e, "learned kernel attribute");
     attr = true;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(LCL);
-  cfg.blockDim = dim3(learned_threads<MODE>());
-  cfg.dynamicSmemBytes = SM_BYTES;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = LCL;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  static int resident = 0;  // clusters on the device at once
-  if (!resident) {
-    int n = 0;
-    cudaError_t e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
-    if (e != cudaSuccess) return cuda_error(e, "learned kernel occupancy");
-    resident = n > 0 ? n : 1;
-  }
+  int dev = 0, nsm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return cuda_error(e, "learned kernel launch shape");
   const long long iters = (rows + LROWS - 1) / LROWS;
-  const long long clusters = std::max<long long>(1, std::min<long long>((iters + LCL - 1) / LCL, resident));
-  cfg.gridDim = dim3((unsigned)(clusters * LCL));
-  cudaError_t le = cudaLaunchKernelEx(&cfg, k, mc, a, la);
-  if (le != cudaSuccess) return cuda_error(le, "learned kernel launch");
+  const unsigned grid = (unsigned)std::max<long long>(1, std::min<long long>(iters, nsm));
+  k<<<grid, learned_threads<MODE>(), SM_BYTES, s>>>(mc, a, la);
   return cuda_error(cudaGetLastError(), "learned kernel launch");
 }
 
