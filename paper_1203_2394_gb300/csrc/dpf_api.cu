@@ -65,6 +65,28 @@ static cudaMemPool_t scratch_pool() {
   return pools[dev];
 }
 
+static std::mutex g_bank_mutex;  // held through a use: copies, launches and records keep one order
+
+ConstantBankUse::ConstantBankUse(cudaStream_t s) : s_(s) {
+  static cudaEvent_t last[64] = {};  // a device's last use (under the mutex)
+  g_bank_mutex.lock();
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  err_ = cudaStreamIsCapturing(s, &cs);
+  if (err_ != cudaSuccess || cs != cudaStreamCaptureStatusNone) return;
+  int dev = 0;
+  err_ = cudaGetDevice(&dev);
+  if (err_ == cudaSuccess && dev >= 64) err_ = cudaErrorInvalidDevice;
+  if (err_ == cudaSuccess && !last[dev]) err_ = cudaEventCreateWithFlags(&last[dev], cudaEventDisableTiming);
+  if (err_ != cudaSuccess) return;
+  ev_ = last[dev];
+  err_ = cudaStreamWaitEvent(s, ev_, 0);  // (an event that was never recorded holds nothing up)
+}
+
+ConstantBankUse::~ConstantBankUse() {
+  if (ev_) cudaEventRecord(ev_, s_);
+  g_bank_mutex.unlock();
+}
+
 dpf_status scratch_alloc(Scratch& sc, int ctas, cudaStream_t s) {
   cudaMemPool_t pool = scratch_pool();
   void* p = nullptr;

@@ -521,7 +521,11 @@ dpf_status dpf_batch_run(dpf_batch* b, const void* ys_dev, int64_t T, double* me
     }
     cudaGraphExec_t exec = nullptr;
     e = cudaGraphInstantiate(&exec, graph, 0);
-    if (e == cudaSuccess) e = cudaGraphLaunch(exec, cap);
+    if (e == cudaSuccess) {
+      ConstantBankUse use(cap);  // (the captured launches may hold copies into a constant bank)
+      e = use.error();
+      if (e == cudaSuccess) e = cudaGraphLaunch(exec, cap);
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(cap);
     if (exec) cudaGraphExecDestroy(exec);
     cudaGraphDestroy(graph);

@@ -93,6 +93,25 @@ struct BatchLaunch {
   int grid;
 };
 
+// The constant banks of the wide kernels hold one model at a time, copied in before the launches
+// that read it. A copy and its launches are enqueued inside one ConstantBankUse: it makes their
+// stream wait for the launches of the last use on the device, whatever stream they went to, so that
+// no copy replaces constants that a kernel still reads. (Inside a capture it does nothing; the
+// library's own graphs are launched inside a use.)
+class ConstantBankUse {
+ public:
+  explicit ConstantBankUse(cudaStream_t s);
+  ~ConstantBankUse();
+  ConstantBankUse(const ConstantBankUse&) = delete;
+  ConstantBankUse& operator=(const ConstantBankUse&) = delete;
+  cudaError_t error() const { return err_; }
+
+ private:
+  cudaStream_t s_;
+  cudaEvent_t ev_ = nullptr;  // null inside a capture
+  cudaError_t err_ = cudaSuccess;
+};
+
 // Per-variant launchers, one set per compiled (precision, d1, d2, dy).
 // the outer stage of a step (dpf_outer.cuh): threads a CTA, items a thread in one
 // chunk, items a chunk, the bound on its grid (rows of partial sums, count totals),

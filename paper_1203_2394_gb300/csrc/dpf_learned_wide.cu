@@ -42,7 +42,7 @@ constexpr int OW_DOUT = 2 * OW_D2;                      // raw log s, c
 typedef MC<float, OW_D1, OW_D2, OW_DY> OwConst;
 
 // 52 KB of this module's 64 KB constant bank; copied from the context's device copy
-// before the stages of every step, in stream order.
+// before the stages of every step, inside a ConstantBankUse (no other filter's copy overtakes them).
 __constant__ OwConst c_ow;
 
 // The ancestor's inner set z_{t-1}^(src, .) into sz[c * M + j] (M threads).
@@ -655,6 +655,8 @@ dpf_status oa_wide_step(Ctx& x, dpf_proposal& p) {
   StepArgs<float> a{};
   VariantImpl<float, OW_D1, OW_D2, OW_DY, 0>::fill_args(x, a);
   a.xp = x.xp;
+  ConstantBankUse use(x.stream);
+  if (use.error() != cudaSuccess) return cuda_error(use.error(), "amortised wide step: model constants");
   cudaError_t e = cudaMemcpyToSymbolAsync(c_ow, x.d_mconst, sizeof(OwConst), 0, cudaMemcpyDeviceToDevice, x.stream);
   if (e != cudaSuccess) return cuda_error(e, "amortised wide step: model constants");
   unsigned grid = 0, grid_u = 0;
@@ -708,6 +710,8 @@ dpf_status oa_wide_record(Ctx& x, long long i0, long long n_outer, float* G, flo
   r.G = G;
   r.Z = Z;
   r.w = w;
+  ConstantBankUse use(x.stream);
+  if (use.error() != cudaSuccess) return cuda_error(use.error(), "amortised wide record: model constants");
   cudaError_t e = cudaMemcpyToSymbolAsync(c_ow, x.d_mconst, sizeof(OwConst), 0, cudaMemcpyDeviceToDevice, x.stream);
   if (e != cudaSuccess) return cuda_error(e, "amortised wide record: model constants");
   const size_t sm = sizeof(float) * ((size_t)OW_D2 * x.M + OW_AT_FLOATS);

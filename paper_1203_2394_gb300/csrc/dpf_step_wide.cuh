@@ -66,6 +66,7 @@ __device__ __forceinline__ void wide_pair_body(const MC<float, D1, D2, DY>& mc, 
   __shared__ uint32_t s_taddr, s_uin;
   __shared__ int s_ok;
   __shared__ float s_x[D1], s_mux[D1], s_ps, s_mx;
+  __shared__ float s_model[6];  // growth (0 or 1), its a and b; h_x's quadratic part (0 or 1) and factor; log norm of R
   const int M = a.M, L = a.L;
   const long long N = a.N, NM = N * (long long)M;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5, hw = M >> 5;
@@ -117,6 +118,14 @@ __device__ __forceinline__ void wide_pair_body(const MC<float, D1, D2, DY>& mc, 
     mbar_fence_init();
   }
   const int NT = blockDim.x;
+  if (tid == 0) {
+    s_model[0] = mc.growth ? 1.f : 0.f;
+    s_model[1] = mc.ga;
+    s_model[2] = mc.gb;
+    s_model[3] = mc.quad ? 1.f : 0.f;
+    s_model[4] = mc.qc;
+    s_model[5] = mc.lognorm_y;
+  }
   for (int e = tid; e < D2 * (D2 + DY); e += NT) {
     const int r = e / (D2 + DY), c = e % (D2 + DY);
     zmat[e] = c < D2 ? mc.Azz[r][c] : mc.K[r][c - D2];
@@ -177,7 +186,7 @@ __device__ __forceinline__ void wide_pair_body(const MC<float, D1, D2, DY>& mc, 
   // h_x(x) = qc x.^2 + H_x x, as h_x in dpf_step.cuh
   auto obs_x = [&](const float (&xv)[D1], float (&out)[DY]) {
 #pragma unroll
-    for (int q = 0; q < DY; ++q) out[q] = mc.quad ? mc.qc * xv[q < D1 ? q : 0] * xv[q < D1 ? q : 0] : 0.f;
+    for (int q = 0; q < DY; ++q) out[q] = s_model[3] != 0.f ? s_model[4] * xv[q < D1 ? q : 0] * xv[q < D1 ? q : 0] : 0.f;
 #pragma unroll
     for (int c = 0; c < D1; ++c) axpy_row<DY>(xv[c], s_HxT + c * DY, out);
   };
@@ -274,7 +283,7 @@ __device__ __forceinline__ void wide_pair_body(const MC<float, D1, D2, DY>& mc, 
       if (w == hw && lane < D1) {  // mean of x_t without the z part, as mu_x in dpf_step.cuh
         float v = 0.f;
         const float xl = s_x[lane];
-        if (mc.growth) v = mc.ga * xl + mc.gb * xl / (1.f + xl * xl) + a.gcos_cur;
+        if (s_model[0] != 0.f) v = s_model[1] * xl + s_model[2] * xl / (1.f + xl * xl) + a.gcos_cur;
 #pragma unroll
         for (int c = 0; c < D1; ++c) v += s_Axx[lane * D1 + c] * s_x[c];
         s_mux[lane] = v;
@@ -534,8 +543,8 @@ __device__ __forceinline__ void wide_pair_body(const MC<float, D1, D2, DY>& mc, 
       const float LN2 = (float)LN2_D;
       const float lA = log2_t(lsum);
       float lw0 = NEG, lw1 = NEG;
-      if (lane < L) lw0 = mc.lognorm_y + LN2 * ((log2_t(rowS[lane]) + shS[lane]) - lA);
-      if (lane + 32 < L) lw1 = mc.lognorm_y + LN2 * ((log2_t(rowS[lane + 32]) + shS[lane + 32]) - lA);
+      if (lane < L) lw0 = s_model[5] + LN2 * ((log2_t(rowS[lane]) + shS[lane]) - lA);
+      if (lane + 32 < L) lw1 = s_model[5] + LN2 * ((log2_t(rowS[lane + 32]) + shS[lane + 32]) - lA);
       if (lane < L) a.lwh_new[i * L + lane] = lw0;
       if (lane + 32 < L) a.lwh_new[i * L + lane + 32] = lw1;
       const float mx = warp_max(fmaxf(lw0, lw1));
