@@ -6,7 +6,9 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -313,8 +315,8 @@ extern "C" {
 
 const char* dpf_last_error(void) { return g_err.c_str(); }
 
-dpf_status dpf_create(const dpf_model_desc* model, int32_t d1, int32_t d2, int64_t N, int32_t M,
-                      int32_t L, uint64_t seed, void* stream, dpf_ctx** out) {
+static dpf_status create_ctx(const dpf_model_desc* model, int32_t d1, int32_t d2, int64_t N, int32_t M,
+                             int32_t L, uint64_t seed, void* stream, bool pf, dpf_ctx** out) {
   clear_error();
   if (!model || !out) return set_error(DPF_E_INVALID, "dpf_create: null argument");
   *out = nullptr;
@@ -407,8 +409,9 @@ dpf_status dpf_create(const dpf_model_desc* model, int32_t d1, int32_t d2, int64
     ok &= !dalloc(*x, x->lwh[q], s * N * L);
     ok &= !dalloc(*x, x->xbb[q], s * N * L * d1);
   }
-  ok = ok && !dalloc(*x, x->lw, s * N) && !dalloc(*x, x->xm, s * N * d1) &&
-       !dalloc(*x, x->zm, s * N * d2) && !dalloc(*x, x->wout, s * N) &&
+  if (!(pf && x->var->pf_own_means))
+    ok = ok && !dalloc(*x, x->xm, s * N * d1) && !dalloc(*x, x->zm, s * N * d2);
+  ok = ok && !dalloc(*x, x->lw, s * N) && !dalloc(*x, x->wout, s * N) &&
        !dalloc(*x, x->yb, s * 2 * x->dy) && !dalloc(*x, x->anc, 4 * N) && !dalloc(*x, x->sel, 4 * N) &&
        !dalloc(*x, x->stats, ssz) && !dalloc(*x, x->lwmax_t, 8) && !dalloc(*x, x->lwmax_key, 8) &&
        !dalloc(*x, x->Csum, 8) && !dalloc(*x, x->done, 8) && !dalloc(*x, x->err, 8) &&
@@ -451,10 +454,14 @@ dpf_status dpf_create(const dpf_model_desc* model, int32_t d1, int32_t d2, int64
   return DPF_OK;
 }
 
+dpf_status dpf_create(const dpf_model_desc* model, int32_t d1, int32_t d2, int64_t N, int32_t M,
+                      int32_t L, uint64_t seed, void* stream, dpf_ctx** out) {
+  return create_ctx(model, d1, d2, N, M, L, seed, stream, false, out);
+}
+
 dpf_status dpf_create_pf(const dpf_model_desc* model, int32_t d1, int32_t d2, int64_t N, uint64_t seed,
                          void* stream, dpf_ctx** out) {
-  clear_error();
-  dpf_status st = dpf_create(model, d1, d2, N, 1, 1, seed, stream, out);
+  dpf_status st = create_ctx(model, d1, d2, N, 1, 1, seed, stream, true, out);
   if (st) return st;
   if (!(*out)->var->pf_step) {
     dpf_destroy(*out);
@@ -782,6 +789,25 @@ dpf_status dpf_set_state(dpf_ctx* x, const void* src, size_t bytes) {
   return cuda_error(e, "dpf_set_state");
 }
 
+// The N padded rows at src (device) to dst (host) coordinate by coordinate, [d1][N]: whole rows
+// cross in blocks and are transposed here. (A strided copy of one 4-byte element a row instead
+// moves each element by itself.)
+static dpf_status read_rows_by_coordinate(dpf_ctx& x, const void* src, char* dst) {
+  const size_t s = x.prec == DPF_F64 ? 8 : 4, row = s * x.xp;
+  const long long N = x.N, most = std::min<long long>(N, (8 << 20) / (long long)row);
+  std::unique_ptr<char[]> buf(new (std::nothrow) char[row * most]);
+  if (!buf) return set_error(DPF_E_NOMEM, "dpf_read: host memory");
+  for (long long i0 = 0; i0 < N; i0 += most) {
+    const long long n = std::min(most, N - i0);
+    cudaError_t e = cudaMemcpyAsync(buf.get(), (const char*)src + row * i0, row * n, cudaMemcpyDeviceToHost, x.stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(x.stream);
+    if (e != cudaSuccess) return cuda_error(e, "dpf_read");
+    for (int c = 0; c < x.d1; ++c)
+      for (long long i = 0; i < n; ++i) memcpy(dst + s * (N * c + i0 + i), buf.get() + row * i + s * c, s);
+  }
+  return DPF_OK;
+}
+
 dpf_status dpf_read(dpf_ctx* x, const char* which, void* dst, size_t bytes) {
   clear_error();
   if (!x || !which || !dst) return set_error(DPF_E_INVALID, "dpf_read: null argument");
@@ -791,6 +817,7 @@ dpf_status dpf_read(dpf_ctx* x, const char* which, void* dst, size_t bytes) {
   const int cur = (int)(t % 2);                   // look-ahead products of step t
   // newest materialised state (the particle filter's particles of step t)
   const int mat = (x->pf || x->std_dpf) ? cur : (t >= 2 ? (int)((t - 1) % 2) : 0);
+  const bool own_means = x->pf && x->var->pf_own_means;
   const void* src = nullptr;
   size_t need = 0;
   std::string w(which);
@@ -800,18 +827,13 @@ dpf_status dpf_read(dpf_ctx* x, const char* which, void* dst, size_t bytes) {
   else if (w == "anc") { src = x->anc; need = 4 * N; }
   else if (w == "sel") { src = x->sel; need = 4 * N; }
   else if (w == "wout") { src = x->wout; need = s * N; }
-  else if (w == "xm" && x->pf && x->pf_rows) {  // a particle's part is the particle: rows of x, by coordinate
+  else if (w == "xm" && own_means) {  // a particle's part is the particle: rows of x, by coordinate
     if (bytes != s * N * x->d1)
       return set_error(DPF_E_INVALID, "dpf_read: 'xm' needs " + std::to_string(s * N * x->d1) + " bytes");
-    cudaError_t e = cudaSuccess;
-    for (int c = 0; c < x->d1 && e == cudaSuccess; ++c)
-      e = cudaMemcpy2DAsync((char*)dst + s * N * c, s, (const char*)x->x[cur] + s * c, s * x->xp, s, N,
-                            cudaMemcpyDeviceToHost, x->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(x->stream);
-    return cuda_error(e, "dpf_read");
+    return read_rows_by_coordinate(*x, x->x[cur], (char*)dst);
   }
   else if (w == "xm") { src = x->xm; need = s * N * x->d1; }
-  else if (w == "zm") { src = x->pf && x->pf_rows ? x->z[cur] : x->zm; need = s * N * x->d2; }
+  else if (w == "zm") { src = own_means ? x->z[cur] : x->zm; need = s * N * x->d2; }
   else if (w == "x") {  // rows are padded to xp elements on the device; returned packed
     if (bytes != s * N * x->d1)
       return set_error(DPF_E_INVALID, "dpf_read: 'x' needs " + std::to_string(s * N * x->d1) + " bytes");

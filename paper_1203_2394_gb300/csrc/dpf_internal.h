@@ -129,6 +129,7 @@ struct Variant {
   dpf_status (*step)(Ctx&, int profile_slot);
   dpf_status (*outer)(Ctx&, double* mean_out, double* logz_out, cudaStream_t s);
   dpf_status (*pf_step)(Ctx&) = nullptr;  // the bootstrap particle filter's step (null: none)
+  bool pf_own_means = false;  // ... whose particles serve as their own means: it has no xm, zm
   dpf_status (*std_step)(Ctx&) = nullptr;  // the DPF without look-ahead (null: none)
   // the outer stage in two launches, for many filters at once: the per-filter
   // arguments, the filter's CTA count, the sums (one variant), then the

@@ -507,6 +507,7 @@ struct VariantImpl {
   static Variant make(int prec) {
     Variant v;
     v.pf_step = &pf_step;
+    v.pf_own_means = true;
     v.std_step = &std_step;
     v.xpad = &xpad;
     v.prec = prec;
