@@ -596,18 +596,34 @@ dpf_status proposal_requantize(dpf_proposal& p) {
   return cuda_error(cudaGetLastError(), "proposal quantize");
 }
 
-// Ensure the per-minibatch workspace holds nb rows.
-static dpf_status workspace(dpf_proposal& p, int nb) {
-  if (nb <= p.ws_rows) return DPF_OK;
-  const size_t H = p.hidden;
-  auto take = [&](float** q, size_t n) { return palloc(p, (void**)q, sizeof(float) * n); };
-  if (take(&p.Fb, (size_t)nb * p.din) || take(&p.Zb, (size_t)nb * p.zw) || take(&p.wb, nb) ||
-      take(&p.h1, nb * H) || take(&p.h2, nb * H) || take(&p.h3, nb * H) || take(&p.ob, (size_t)nb * p.dout) ||
-      take(&p.dA, nb * H) || take(&p.dB, nb * H) || take(&p.dO, (size_t)nb * p.dout) ||
-      palloc(p, (void**)&p.perm_d, sizeof(int64_t) * nb))
-    return DPF_E_NOMEM;
-  p.ws_rows = nb;
+// The buffers bufs[q] of nb x widths[q] floats, where they hold `rows` rows now: kept if that is
+// enough, else given back and allocated anew (the sizes need not be held twice).
+template <size_t NB>
+static dpf_status hold_rows(dpf_proposal& p, int nb, int& rows, float** const (&bufs)[NB], const int (&widths)[NB]) {
+  if (nb <= rows) return DPF_OK;
+  cudaError_t e = cudaStreamSynchronize(p.stream);
+  if (e != cudaSuccess) return cuda_error(e, "proposal workspace");
+  rows = 0;
+  for (float** b : bufs) {
+    p.allocs.erase(std::remove(p.allocs.begin(), p.allocs.end(), (void*)*b), p.allocs.end());
+    cudaFree(*b);
+    *b = nullptr;
+  }
+  for (size_t q = 0; q < NB; ++q) {
+    dpf_status st = palloc(p, (void**)bufs[q], sizeof(float) * (size_t)nb * widths[q]);
+    if (st) return st;
+  }
+  rows = nb;
   return DPF_OK;
+}
+
+// Ensure the per-minibatch workspace holds nb rows; gather: training's gathered rows too.
+static dpf_status workspace(dpf_proposal& p, int nb, bool gather) {
+  const int H = p.hidden;
+  dpf_status st = hold_rows(p, nb, p.ws_rows, {&p.h1, &p.h2, &p.h3, &p.ob, &p.dA, &p.dB, &p.dO},
+                            {H, H, H, p.dout, H, H, p.dout});
+  if (!st && gather) st = hold_rows(p, nb, p.gather_rows, {&p.Fb, &p.Zb, &p.wb}, {p.din, p.zw, 1});
+  return st;
 }
 
 // Forward and backward over nb rows (features F, targets Z, weights w): loss into *loss_dev
@@ -890,7 +906,7 @@ dpf_status dpf_proposal_loss_grad(dpf_proposal* p, const float* F, const float* 
   clear_error();
   if (!p || !F || !Z || !w || n < 1 || n > (1 << 24))
     return set_error(DPF_E_INVALID, "dpf_proposal_loss_grad: bad arguments");
-  dpf_status st = workspace(*p, (int)n);
+  dpf_status st = workspace(*p, (int)n, false);
   if (st) return st;
   cudaStream_t s = p->stream;
   // the caller's rows are read where they lie (the products round them as they stage them)
@@ -922,7 +938,7 @@ dpf_status dpf_proposal_train(dpf_proposal* p, const float* F, const float* Z, c
   if (!p || !F || !Z || !w || n < 1 || batch < 1 || batch > (1 << 16) || epochs < 1 || !(lr > 0.f))
     return set_error(DPF_E_INVALID, "dpf_proposal_train: bad arguments");
   const int nb_max = (int)std::min<int64_t>(batch, n);
-  dpf_status st = workspace(*p, nb_max);
+  dpf_status st = workspace(*p, nb_max, true);
   if (st) return st;
   cudaStream_t s = p->stream;
   const int rd = p->bf16 ? 1 : 0;

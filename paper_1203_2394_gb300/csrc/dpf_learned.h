@@ -51,11 +51,11 @@ struct dpf_proposal {
   double* wsum_d = nullptr;
   int* err_d = nullptr;    // device error word of the training products (bounded waits)
   int adam_t = 0;
-  // minibatch workspace
-  int ws_rows = 0;
-  float *Fb = nullptr, *Zb = nullptr, *wb = nullptr, *h1 = nullptr, *h2 = nullptr, *h3 = nullptr;
-  float *ob = nullptr, *dA = nullptr, *dB = nullptr, *dO = nullptr;
-  int64_t* perm_d = nullptr;
+  // minibatch workspace: the layers' values and gradients of ws_rows rows, and for training (which
+  // gathers its minibatches) gather_rows rows of features, targets and weights
+  int ws_rows = 0, gather_rows = 0;
+  float *h1 = nullptr, *h2 = nullptr, *h3 = nullptr, *ob = nullptr, *dA = nullptr, *dB = nullptr, *dO = nullptr;
+  float *Fb = nullptr, *Zb = nullptr, *wb = nullptr;
   // weights packed for the tensor-core forward pass (rebuilt when stale)
   bool packed_valid = false;
   void* packed = nullptr;
