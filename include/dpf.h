@@ -431,6 +431,10 @@ dpf_status dpf_proposal_set_bf16(dpf_proposal* p, int32_t enable);
  * sum_b w_b (-log q(Z_b | F_b)) / sum_b w_b. F (n x din), Z (n x d2), w (n):
  * device float arrays; loss: host (may be NULL); grad_dev: device, num_params
  * floats in the parameter order, or NULL. Synchronises.
+ * Below 1024 rows the gradient repeats bit for bit from call to call (and so does
+ * training in minibatches below that); from 1024 rows on the bias gradients do, and
+ * the weight gradients may differ in their last bits. The loss is summed in double
+ * precision in no fixed order.
  */
 dpf_status dpf_proposal_loss_grad(dpf_proposal* p, const float* F, const float* Z, const float* w, int64_t n,
                                   double* loss, float* grad_dev);

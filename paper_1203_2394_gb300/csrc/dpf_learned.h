@@ -50,6 +50,9 @@ struct dpf_proposal {
   double* loss_d = nullptr;
   double* wsum_d = nullptr;
   int* err_d = nullptr;    // device error word of the training products (bounded waits)
+  // the weight gradients' slices of a minibatch before they are added in their order (grad_tail_kernel)
+  float* bias_part = nullptr;   // [slice][layer][kMaxHidden]
+  float* grad_part = nullptr;   // [slice][nparams, rounded up to 4], below TG_REPEAT_ROWS rows
   int adam_t = 0;
   // minibatch workspace: the layers' values and gradients of ws_rows rows, and for training (which
   // gathers its minibatches) gather_rows rows of features, targets and weights
