@@ -1148,7 +1148,7 @@ struct PaperVariant {
       if (e != cudaSuccess) return cuda_error(e, "paper-model step occupancy");
       x.grid_step = (nb > 0 ? nb : 1) * nsm;
     }
-    const int nw = x.N <= FEW_GROUPS ? 1 : WARPS_PER_CTA;
+    const int nw = x.N <= few_groups(4) ? 1 : WARPS_PER_CTA;
     const long long want = (x.N + nw - 1) / nw;
     const unsigned grid = (unsigned)(nw == 1 ? want : std::min<long long>(want, x.grid_step));
     k<<<grid, 32 * nw, wb * nw, x.stream>>>(a, o);

@@ -15,7 +15,12 @@ namespace dpf {
 // attribute belongs to the kernel, so one filter's smaller need must not cut another's.
 constexpr int WARP_MAX_SMEM = 200 * 1024;
 
-constexpr int FEW_GROUPS = 16 * 152;  // one-warp CTAs: 16 fit on an SM at 128 registers a thread
+// Most groups that run as one-warp CTAs: as many warps of a kernel compiled for `min_blocks` CTAs an
+// SM (by its registers) as the device holds at once. Above that a one-warp CTA has no next group
+// to prefetch and its start is not hidden. (Compiled for two, growth_clg10 at M = 256: N = 1300, 1800 and
+// 2400 take 45.8, 48.6 and 50.9 us a step in one-warp CTAs, 44.4, 46.7 and 49.0 in full ones;
+// lg16 at d1 = 2, M = 128: 55.3, 56.3 and 60.3 against 51.3, 53.3 and 56.2.)
+constexpr int few_groups(int min_blocks) { return min_blocks * WARPS_PER_CTA * 152; }
 
 inline int threads_for(int M) { return ((M + 31) / 32) * 32; }
 
@@ -189,9 +194,8 @@ struct VariantImpl {
     // Few groups: a CTA of one warp each, so that they spread over every SM. (Four to a CTA left
     // the 256 groups of a small filter on 64 of the 152 SMs, four warps sharing each one's FP64
     // pipe. lg4 in FP64 at N = 256, M = 32, L = 8: 90.8 us a step, 74.5 with the spread and the
-    // two-pass look-ahead.) Above FEW_GROUPS four-warp CTAs fill every
-    // SM anyway.
-    if (x.N <= FEW_GROUPS) {
+    // two-pass look-ahead.) Above that four-warp CTAs fill every SM anyway.
+    if (x.N <= few_groups(warp_min_blocks<PPL, D2>())) {
       k<<<(unsigned)x.N, 32, sm / WARPS_PER_CTA, stream ? stream : x.stream>>>(cst(x), a);
       return cuda_error(cudaGetLastError(), "step kernel launch");
     }
@@ -429,7 +433,7 @@ struct VariantImpl {
   static dpf_status launch_std_warp(Ctx& x, const StdArgs<T>& a) {
     auto k = std_warp_kernel<T, D1, D2, DY, XZ, PPL>;
     const size_t wb = std_warp_smem<T, D1, D2>(x.M, x.xp);
-    const int nw = x.N <= FEW_GROUPS ? 1 : WARPS_PER_CTA;
+    const int nw = x.N <= few_groups(warp_min_blocks<PPL, D2>()) ? 1 : WARPS_PER_CTA;
     if (x.grid_step == 0 || x.grid_kernel != (const void*)k) {  // as many CTAs as fit on the device at once
       int nb = 0, dev = 0, nsm = 0;
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, WARP_MAX_SMEM);
