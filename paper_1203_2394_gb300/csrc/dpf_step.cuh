@@ -476,15 +476,9 @@ __device__ __forceinline__ void step_body(const MC<T, D1, D2, DY>& mc, const Ste
     }
   }
   if constexpr (TC && D2 > 32) {
-    // per coordinate r: (L_r^-1 H_z)[., r] then (H_z A_zz)[., r]; then the rows of A_zx
-    // and the diagonal of L_qz
-    T* pj = (T*)(smem_raw + a.off_proj);
-    for (int e = tid; e < D2 * 2 * DY; e += NT) {
-      const int r = e / (2 * DY), q = e % (2 * DY);
-      pj[e] = q < DY ? mc.LrHz[q][r] : mc.HzAzz[q - DY][r];
-    }
-    for (int e = tid; e < D2 * D1; e += NT) pj[D2 * 2 * DY + e] = mc.Azx[e / D1][e % D1];
-    for (int r = tid; r < D2; r += NT) pj[D2 * (2 * DY + D1) + r] = mc.Lqz[r][r];
+    // the rows of A_zx (their place in the two-thread form's block of matrices)
+    T* azx = (T*)(smem_raw + a.off_proj) + D2 * 2 * DY;
+    for (int e = tid; e < D2 * D1; e += NT) azx[e] = mc.Azx[e / D1][e % D1];
   }
   uint32_t taddr = 0, tc_phase = 0;
   constexpr uint32_t TC_COLS = TC ? (NP * 2 <= 32 ? 32 : NP * 2 <= 64 ? 64 : NP * 2 <= 128 ? 128 : 256) : 32;
@@ -579,10 +573,6 @@ __device__ __forceinline__ void step_body(const MC<T, D1, D2, DY>& mc, const Ste
     }
     T* sz = (T*)(st + a.off_sz);
     T* zsrc = sz;          // wide z: where the look-ahead's z sits for the z-mean
-    bool zstored = false;  // z_t already written (the rolled tensor-core epilogue)
-    T gz[DY];              // ... and its H_z A_zz z_t
-#pragma unroll
-    for (int q = 0; q < DY; ++q) gz[q] = T(0);
     T* slq = (T*)(st + a.off_slq);
     T* sx = (T*)(st + a.off_sx);
     T* slwh = (T*)(st + a.off_slwh);
@@ -808,10 +798,8 @@ __device__ __forceinline__ void step_body(const MC<T, D1, D2, DY>& mc, const Ste
         float zb2[D2];
 #pragma unroll
         for (int c = 0; c < D2; ++c) zb2[c] = (float)sz[c * M + b];
-        // A_zx x_a, the same for the whole group, and the diagonal of L_qz (part is free
-        // until the z-mean)
+        // A_zx x_a, the same for the whole group (part is free until the z-mean)
         T* s_azx = part;
-        const T* s_lqd = (const T*)(smem_raw + a.off_proj) + D2 * (2 * DY + D1);
         if (tid < D2) {
           const T* azr = (const T*)(smem_raw + a.off_proj) + D2 * 2 * DY + tid * D1;
           T v = T(0);
@@ -858,74 +846,8 @@ __device__ __forceinline__ void step_body(const MC<T, D1, D2, DY>& mc, const Ste
         const uint32_t ta = taddr + ((uint32_t)(32 * ((tid >> 5) & 3)) << 16) + (uint32_t)((j >> 7) * NP);
         if constexpr (D2 > 32) zsrc = (T*)(smem_raw + a.off_zlo);  // the low parts are consumed
         T qf = T(0);
-        if (mc.diag_qz) {
-          // diagonal Q_z: four coordinates at a time (a TMEM load, one Philox block of noise);
-          // z_t goes to the state and to shared memory, and the whitened y residual and the
-          // look-ahead's H_z A_zz z_t accumulate on the way (a rolled loop: small code)
-          const bool ok = tc::bar_wait(&tcbar, tc_phase, TC_SPIN);
-          tc_phase ^= 1u;
-          if (!ok && tid == 0) atomicOr(a.err, ERR_TIMEOUT);
-          tc::fence_after();
-          // the MMAs have read the stage: the next group's rows may come in
-          if (PF && tid < 32 && g + gridDim.x < G)
-            stage_group<T, D1, D2, true, true>(a, stage0, &bars[0], source_of(g + gridDim.x));
-          pf_issued = PF;
-          const T* pj = (const T*)(smem_raw + a.off_proj);
-          T* zn = a.z_new + i * M + j;
-          T rl[DY];
-#pragma unroll
-          for (int q = 0; q < DY; ++q) rl[q] = yh[q];
-#pragma unroll 2
-          for (int cb = 0; cb < D2 / 8; ++cb) {  // eight coordinates: one TMEM load, two noise blocks
-            float a8[8];
-            tc::ld8(ta + (uint32_t)(8 * cb), a8);
-            T e[8];
-            {
-              T e0[4], e1[4];
-              normal_block_rk(rk, a.t - 1, (uint32_t)i, P_PROP, (uint32_t)j, 2 * cb, 4, e0);
-              normal_block_rk(rk, a.t - 1, (uint32_t)i, P_PROP, (uint32_t)j, 2 * cb + 1, 4, e1);
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                e[u] = e0[u];
-                e[4 + u] = e1[u];
-              }
-            }
-            const float4* az4 = reinterpret_cast<const float4*>(s_azx + 8 * cb);
-            const float4* lq4 = reinterpret_cast<const float4*>(s_lqd + 8 * cb);
-            const float4 za = az4[0], zb = az4[1], la = lq4[0], lb = lq4[1];
-            const T azv[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w};
-            const T lqv[8] = {la.x, la.y, la.z, la.w, lb.x, lb.y, lb.z, lb.w};
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-              const int r = 8 * cb + u;
-              const T v = ((ok ? (T)a8[u] : T(0)) + azv[u]) + lqv[u] * e[u];
-              zsrc[r * M + j] = v;
-              zn[(long long)r * NM] = v;
-              const float4* pr = reinterpret_cast<const float4*>(pj + r * 2 * DY);
-#pragma unroll
-              for (int h = 0; h < DY / 4; ++h) {
-                const float4 l4 = pr[h];
-                rl[4 * h + 0] -= l4.x * v;
-                rl[4 * h + 1] -= l4.y * v;
-                rl[4 * h + 2] -= l4.z * v;
-                rl[4 * h + 3] -= l4.w * v;
-              }
-#pragma unroll
-              for (int h = 0; h < DY / 4; ++h) {
-                const float4 g4 = pr[DY / 4 + h];
-                gz[4 * h + 0] += g4.x * v;
-                gz[4 * h + 1] += g4.y * v;
-                gz[4 * h + 2] += g4.z * v;
-                gz[4 * h + 3] += g4.w * v;
-              }
-            }
-          }
-          tc::fence_before();
-#pragma unroll
-          for (int q = 0; q < DY; ++q) qf += rl[q] * rl[q];
-          zstored = true;
-        } else {
-        // a general L_qz: every coordinate's noise at once, drawn while the MMAs run
+        // every coordinate's noise at once (a general L_qz; a diagonal one takes dpf_step_wide.cuh), drawn
+        // while the MMAs run
         T eps[D2];
         normals_rk<D2>(rk, a.t - 1, (uint32_t)i, P_PROP, (uint32_t)j, eps);
         const bool ok = tc::bar_wait(&tcbar, tc_phase, TC_SPIN);
@@ -960,7 +882,6 @@ __device__ __forceinline__ void step_body(const MC<T, D1, D2, DY>& mc, const Ste
           for (int c = 0; c < D2; ++c) v -= mc.LrHz[q][c] * zr[0][c];
           qf += v * v;
         }
-        }
         ell[0] = T(-0.5) * qf;
         lmax = ell[0];
       }
@@ -976,13 +897,11 @@ __device__ __forceinline__ void step_body(const MC<T, D1, D2, DY>& mc, const Ste
       for (int p = 0; p < PPT; ++p) {
         if (tid + p * NT < M) {
           lqr[p] = ell[p] - lmax - llsum;
-          if (!zstored) {
 #pragma unroll
-            for (int c = 0; c < D2; ++c) zn[c * NM + p * NT] = zr[p][c];
-            if constexpr (D2 > 32) {  // z_t for the z-mean (every gather from the stage is done)
+          for (int c = 0; c < D2; ++c) zn[c * NM + p * NT] = zr[p][c];
+          if constexpr (D2 > 32) {  // z_t for the z-mean (every gather from the stage is done)
 #pragma unroll
-              for (int c = 0; c < D2; ++c) zsrc[c * M + tid + p * NT] = zr[p][c];
-            }
+            for (int c = 0; c < D2; ++c) zsrc[c * M + tid + p * NT] = zr[p][c];
           }
           a.lq_new[i * M + tid + p * NT] = lqr[p];
         }
@@ -1012,12 +931,8 @@ __device__ __forceinline__ void step_body(const MC<T, D1, D2, DY>& mc, const Ste
           T v = e;
 #pragma unroll
           for (int c = 0; c < D1; ++c) v += mc.HzAzx[q][c] * x[c];
-          if (zstored) {
-            v += gz[q];
-          } else {
 #pragma unroll
-            for (int c = 0; c < D2; ++c) v += mc.HzAzz[q][c] * zr[p][c];
-          }
+          for (int c = 0; c < D2; ++c) v += mc.HzAzz[q][c] * zr[p][c];
           g_[q] = v;
         }
 #pragma unroll

@@ -40,8 +40,6 @@ constexpr int NOISE_CHAINS = 4;
 template <typename T, int PPL, int D2>
 constexpr bool rolled_noise() { return sizeof(T) == 4 && PPL * D2 >= 32; }
 
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
 // Per-warp shared-memory carve-up (bytes from the warp's region), on the host.
 template <typename T, int D1, int D2, int DY, bool XZ>
 inline size_t warp_geometry(int M, int L, StepArgs<T>* a, bool first = false) {
@@ -668,7 +666,7 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
           if (act) vld<T, PPL>(sz + c * M + k0, e);
           add_noise(c, e);
         }
-        fence_async_smem();  // these writes come before the copies that refill the stage
+        tc::fence_proxy_async();  // these writes come before the copies that refill the stage
       } else {
 #pragma unroll
         for (int b = 0; b < (D2 + 3) / 4; ++b) {
