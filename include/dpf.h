@@ -522,7 +522,8 @@ dpf_status dpf_record_tuples_amortised(dpf_ctx* ctx, int64_t i0, int64_t n_outer
 
 /*
  * A check of the failure path of the bounded waits; the paper has no
- * counterpart. Runs a step's outer stage (3 CTAs of one cooperative launch) with
+ * counterpart. Runs (1) a warp of a step waiting for staged rows that no copy
+ * brings and (2) a step's outer stage (3 CTAs of one cooperative launch) with
  * CTA 0 never reaching the grid-wide barrier. The waits give up after their bound
  * (a few tenths of a second) and the device stays usable; the call returns
  * DPF_E_TIMEOUT when they ran out as they should, and another status otherwise.

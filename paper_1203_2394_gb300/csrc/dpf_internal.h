@@ -53,6 +53,7 @@ dpf_status err_word_status(int w, const char* what);
 // The outer stage with one CTA that never reaches the grid barrier: the waits run
 // out and the status is DPF_E_TIMEOUT (dpf_check_bounded_wait).
 dpf_status check_outer_barrier(cudaStream_t s);
+dpf_status check_stage_wait(cudaStream_t s);
 
 // Launch the global systematic-resampling kernels on caller-provided scratch
 // (laid out for resample_ctas(n) CTAs; nothing in it need be cleared); no allocation, no

@@ -590,15 +590,7 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32, 4)
     if (i + W < N) src_next = a.first ? i + W : (long long)a.anc[i + W];
   }
   for (; i < N; i += W, phase ^= 1u) {
-    {  // wait for this group's rows (bounded)
-      int spins = 0;
-      while (!mbar_test(bar, phase)) {
-        if (++spins > MBAR_SPIN_LIMIT) {
-          if (lane == 0) atomicOr(a.err, ERR_TIMEOUT);
-          break;
-        }
-      }
-    }
+    if (!warp_rows_in(bar, phase, a.err, lane)) break;
     float x[D1], zk[D2][PPL], lqk[PPL];
 #pragma unroll
     for (int p = 0; p < PPL; ++p) {

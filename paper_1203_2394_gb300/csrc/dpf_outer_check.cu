@@ -1,11 +1,12 @@
-// A check of the outer stage's bounded barrier wait (part of
-// dpf_check_bounded_wait): no GPU fault, only a wait that runs out.
+// Checks of bounded waits (parts of dpf_check_bounded_wait): the outer stage's barrier and a step's
+// wait for staged rows. No GPU fault, only waits that run out.
 #include <cuda_runtime.h>
 
 #include <cmath>
 
 #include "dpf_internal.h"
 #include "dpf_outer.cuh"
+#include "dpf_step_warp.cuh"
 
 namespace dpf {
 
@@ -62,6 +63,38 @@ dpf_status check_outer_barrier(cudaStream_t s) {
   cudaFreeAsync(b, s);
   if (e != cudaSuccess) return cuda_error(e, "dpf_check_bounded_wait: outer stage");
   return err_word_status(w, "dpf_check_bounded_wait: outer stage");
+}
+
+// One warp waits for rows that no copy brings: out[0] is its error word, out[1] the lanes that were
+// told to go on.
+__global__ void unfed_stage_kernel(int* out) {
+  __shared__ __align__(8) uint64_t bar;
+  const int lane = threadIdx.x;
+  if (lane == 0) {
+    mbar_init(&bar, 1);
+    mbar_fence_init();
+  }
+  __syncwarp();
+  const unsigned on = __ballot_sync(FULL, warp_rows_in(&bar, 0u, out, lane));
+  if (lane == 0) out[1] = (int)on;
+}
+
+dpf_status check_stage_wait(cudaStream_t s) {
+  int* out = nullptr;
+  int h[2] = {0, 0};
+  cudaError_t e = cudaMallocAsync((void**)&out, sizeof(h), s);
+  if (e != cudaSuccess) return cuda_error(e, "dpf_check_bounded_wait: allocation");
+  e = cudaMemsetAsync(out, 0, sizeof(h), s);
+  if (e == cudaSuccess) {
+    unfed_stage_kernel<<<1, 32, 0, s>>>(out);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(h, out, sizeof(h), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  cudaFreeAsync(out, s);
+  if (e != cudaSuccess) return cuda_error(e, "dpf_check_bounded_wait: staged rows");
+  if (h[1]) return set_error(DPF_E_CUDA, "dpf_check_bounded_wait: lanes went on without their rows");
+  return err_word_status(h[0], "dpf_check_bounded_wait: staged rows");
 }
 
 }  // namespace dpf

@@ -243,8 +243,12 @@ extern "C" dpf_status dpf_box_muller(const uint32_t* words, int64_t n_pairs, int
 
 extern "C" dpf_status dpf_check_bounded_wait(void* stream) {
   clear_error();
+  // a step's wait for staged rows that no copy brings
+  dpf_status st = check_stage_wait((cudaStream_t)stream);
+  if (st != DPF_E_TIMEOUT)
+    return st ? st : set_error(DPF_E_CUDA, "dpf_check_bounded_wait: the wait for staged rows did not run out");
   // the grid barrier of a step's outer stage, which CTA 0 never reaches
-  dpf_status st = check_outer_barrier((cudaStream_t)stream);
+  st = check_outer_barrier((cudaStream_t)stream);
   if (st != DPF_E_TIMEOUT)
     return st ? st : set_error(DPF_E_CUDA, "dpf_check_bounded_wait: the outer stage's barrier wait did not run out");
   return st;

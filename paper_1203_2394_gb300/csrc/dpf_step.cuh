@@ -315,7 +315,10 @@ __device__ __forceinline__ double exp2_t(double x) { return exp2(x); }
 __device__ __forceinline__ float log2_t(float x) { return log2f(x); }
 __device__ __forceinline__ double log2_t(double x) { return log2(x); }
 
-constexpr int MBAR_SPIN_LIMIT = 1 << 16;  // bounded wait on a stage's barrier
+// Bounded wait on a stage's barrier. After it has given up a kernel reports it, waits once more (as
+// long) for the copies it has in flight, which must not land when its shared memory is another
+// CTA's, and leaves.
+constexpr int MBAR_SPIN_LIMIT = 1 << 16;
 constexpr double LOG2E_D = 1.4426950408889634;
 constexpr double LN2_D = 0.6931471805599453;
 constexpr double SQ_D = 0.84932180028801907;  // sqrt(log2(e) / 2): -x^2/2 in log2 units is -(SQ x)^2
@@ -530,7 +533,11 @@ __device__ __forceinline__ void step_body(const MC<T, D1, D2, DY>& mc, const Ste
       src_next = a.first ? i1 : (long long)a.anc[i1];
     }
   }
-  for (int k = 0; g < G; g += gridDim.x, ++k) {
+  bool gave_up = false;  // a wait of this thread's ran out: the CTA leaves at the group's last barrier
+  bool pf_issued = false;  // the next group's stage copy is under way
+  bool mma_out = false;    // the MMAs were not seen to finish
+  int k = 0;
+  for (; g < G; g += gridDim.x, ++k) {
     const long long i = group_at(a, g);
     const int sidx = k & 1;
     unsigned char* st = stage0 + (BULK ? sidx * a.stage_bytes : 0);
@@ -544,29 +551,22 @@ __device__ __forceinline__ void step_body(const MC<T, D1, D2, DY>& mc, const Ste
           src_next = a.first ? i2 : (long long)a.anc[i2];
         }
       }
-      int spins = 0;
-      while (!mbar_test(&bars[sidx], (uint32_t)((k >> 1) & 1))) {
-        if (++spins > MBAR_SPIN_LIMIT) {
-          if (tid == 0) atomicOr(a.err, ERR_TIMEOUT);
-          break;
-        }
-      }
+      gave_up = !tc::bar_wait(&bars[sidx], (uint32_t)((k >> 1) & 1), MBAR_SPIN_LIMIT);
     } else if (PF) {
-      int spins = 0;
-      while (!mbar_test(&bars[0], (uint32_t)(k & 1))) {
-        if (++spins > MBAR_SPIN_LIMIT) {
-          if (tid == 0) atomicOr(a.err, ERR_TIMEOUT);
-          break;
-        }
-      }
+      gave_up = !tc::bar_wait(&bars[0], (uint32_t)(k & 1), MBAR_SPIN_LIMIT);
     } else if (!(a.gskip && a.gskip[i])) {
       const long long src = a.first ? i : (long long)a.anc[i];
       stage_group<T, D1, D2, BULK>(a, st, nullptr, src);
       __syncthreads();
     }
-    bool pf_issued = false;  // the next group's stage copy is under way
+    pf_issued = false;
     if (a.gskip && a.gskip[i]) {  // every thread has left the stage wait before it is re-armed
-      __syncthreads();
+      if (BULK || PF) {
+        gave_up = __syncthreads_or(gave_up);
+        if (gave_up) break;
+      } else {
+        __syncthreads();
+      }
       if (PF && tid < 32 && g + gridDim.x < G)
         stage_group<T, D1, D2, true, true>(a, stage0, &bars[0], source_of(g + gridDim.x));
       continue;
@@ -852,11 +852,13 @@ __device__ __forceinline__ void step_body(const MC<T, D1, D2, DY>& mc, const Ste
         normals_rk<D2>(rk, a.t - 1, (uint32_t)i, P_PROP, (uint32_t)j, eps);
         const bool ok = tc::bar_wait(&tcbar, tc_phase, TC_SPIN);
         tc_phase ^= 1u;
-        if (!ok && tid == 0) atomicOr(a.err, ERR_TIMEOUT);
+        mma_out = !ok;
+        gave_up |= !ok;
         tc::fence_after();
-        if (PF && tid < 32 && g + gridDim.x < G)
+        if (PF && tid < 32 && g + gridDim.x < G && !__any_sync(FULL, gave_up)) {
           stage_group<T, D1, D2, true, true>(a, stage0, &bars[0], source_of(g + gridDim.x));
-        pf_issued = PF;
+          pf_issued = true;
+        }
         {
           float azz[(D2 + 15) / 16 * 16];
           if constexpr (NP == 64) {  // the whole padded row in one load
@@ -1234,7 +1236,13 @@ __device__ __forceinline__ void step_body(const MC<T, D1, D2, DY>& mc, const Ste
           }
         }
       }
-      __syncthreads();  // the stage and the work buffers are free for the next group
+      // the stage and the work buffers are free for the next group
+      if (BULK || PF) {
+        gave_up = __syncthreads_or(gave_up);
+        if (gave_up) break;
+      } else {
+        __syncthreads();
+      }
       if (PF && !pf_issued && tid < 32 && g + gridDim.x < G)
         stage_group<T, D1, D2, true, true>(a, stage0, &bars[0], source_of(g + gridDim.x));
     } else {
@@ -1279,9 +1287,27 @@ __device__ __forceinline__ void step_body(const MC<T, D1, D2, DY>& mc, const Ste
         for (int q = 0; q < DY; ++q) v += mc.K[r][q] * sb[D2 + q];
         a.zm[(long long)r * N + i] = v;
       }
-      __syncthreads();  // the stage and the work buffers are free for the next group
+      // the stage and the work buffers are free for the next group
+      if (BULK || PF) {
+        gave_up = __syncthreads_or(gave_up);
+        if (gave_up) break;
+      } else {
+        __syncthreads();
+      }
       if (PF && !pf_issued && tid < 32 && g + gridDim.x < G)
         stage_group<T, D1, D2, true, true>(a, stage0, &bars[0], source_of(g + gridDim.x));
+    }
+  }
+  if ((BULK || PF) && gave_up && tid == 0) {  // (the whole CTA left the loop in group k)
+    atomicOr(a.err, ERR_TIMEOUT);
+    if (PF) {
+      tc::bar_wait(&bars[0], (uint32_t)((k + (pf_issued ? 1 : 0)) & 1), MBAR_SPIN_LIMIT);
+    } else {
+      tc::bar_wait(&bars[k & 1], (uint32_t)((k >> 1) & 1), MBAR_SPIN_LIMIT);
+      if (g + gridDim.x < G) tc::bar_wait(&bars[(k + 1) & 1], (uint32_t)(((k + 1) >> 1) & 1), MBAR_SPIN_LIMIT);
+    }
+    if constexpr (TC) {
+      if (mma_out) tc::bar_wait(&tcbar, tc_phase ^ 1u, MBAR_SPIN_LIMIT);
     }
   }
   if constexpr (TC) {

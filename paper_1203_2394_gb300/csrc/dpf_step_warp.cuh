@@ -335,6 +335,21 @@ __device__ __forceinline__ T lane_sum_in_order(const T* part) {
   return r;
 }
 
+// The phase of a warp whose wait gave up: it steps no group of a later filter of the launch either.
+constexpr uint32_t WARP_DEAD = 2;
+
+// A warp's bounded wait for its group's rows. False, in every lane, when it gave up: the timeout is
+// reported and the copies have had a second wait; the warp must leave its stage.
+__device__ __forceinline__ bool warp_rows_in(uint64_t* bar, uint32_t phase, int* err, int lane) {
+  if (__all_sync(FULL, tc::bar_wait(bar, phase, MBAR_SPIN_LIMIT))) return true;
+  if (lane == 0) {
+    atomicOr(err, ERR_TIMEOUT);
+    tc::bar_wait(bar, phase, MBAR_SPIN_LIMIT);
+  }
+  __syncwarp();
+  return false;
+}
+
 // Issue the bulk copies of one group's source rows into a warp's stage (lane 0).
 template <typename T, int D1, int D2>
 __device__ __forceinline__ void warp_stage(const StepArgs<T>& a, unsigned char* st, uint64_t* bar,
@@ -371,6 +386,10 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
                                          unsigned char* ws, uint64_t* bar, uint32_t& phase) {
   static_assert(MF == 0 || MF == 32 * PPL, "MF is 0 or 32 PPL");
   const int lane = threadIdx.x & 31;
+  if (phase == WARP_DEAD) {
+    if (lane == 0) atomicOr(a.err, ERR_TIMEOUT);
+    return;
+  }
   const int M = MF ? MF : a.M, L = a.L;
   const long long N = a.N;
   const long long NM = N * (long long)M;
@@ -424,14 +443,9 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
   __syncwarp();
   for (; g < gend; g += W, phase ^= 1u) {
     const long long i = group_at(a, g);
-    {  // wait for this group's rows (bounded)
-      int spins = 0;
-      while (!mbar_test(bar, phase)) {
-        if (++spins > MBAR_SPIN_LIMIT) {
-          if (lane == 0) atomicOr(a.err, ERR_TIMEOUT);
-          break;
-        }
-      }
+    if (!warp_rows_in(bar, phase, a.err, lane)) {
+      phase = WARP_DEAD;
+      return;
     }
     if (a.gskip && a.gskip[i]) {  // a group left untouched: pass its stage on
       __syncwarp();

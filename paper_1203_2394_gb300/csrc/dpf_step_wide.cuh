@@ -199,16 +199,14 @@ __device__ __forceinline__ void wide_pair_body(const MC<float, D1, D2, DY>& mc, 
   if (g < G && w == 0) stage_group<float, D1, D2, true, true>(a, stage0, &bars[0], source_of(g));
   for (int k = 0; g < G; g += gridDim.x, ++k) {
     const long long i = group_at(a, g);
-    if (tid == 0) {  // one thread polls; the barrier releases the rest
-      int spins = 0;
-      while (!mbar_test(&bars[0], (uint32_t)(k & 1))) {
-        if (++spins > MBAR_SPIN_LIMIT) {
-          atomicOr(a.err, ERR_TIMEOUT);
-          break;
-        }
+    // one thread polls; the barrier releases the rest
+    if (!__syncthreads_and(tid || tc::bar_wait(&bars[0], (uint32_t)(k & 1), MBAR_SPIN_LIMIT))) {
+      if (tid == 0) {
+        atomicOr(a.err, ERR_TIMEOUT);
+        tc::bar_wait(&bars[0], (uint32_t)(k & 1), MBAR_SPIN_LIMIT);
       }
+      break;
     }
-    __syncthreads();
     if (a.gskip && a.gskip[i]) {
       __syncthreads();
       if (w == 0 && g + gridDim.x < G)
@@ -382,17 +380,21 @@ __device__ __forceinline__ void wide_pair_body(const MC<float, D1, D2, DY>& mc, 
       }
     }
     if (tid == 0) {
-      const bool ok = tc::bar_wait(&tcbar, tc_phase, TC_SPIN);
-      if (!ok) atomicOr(a.err, ERR_TIMEOUT);
-      s_ok = ok;
+      s_ok = tc::bar_wait(&tcbar, tc_phase, TC_SPIN);
     }
     tc_phase ^= 1u;
     __syncwarp();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
+    if (!s_ok) {  // (no copy is in flight here; the MMAs get a second wait)
+      if (tid == 0) {
+        atomicOr(a.err, ERR_TIMEOUT);
+        tc::bar_wait(&tcbar, tc_phase ^ 1u, MBAR_SPIN_LIMIT);
+      }
+      break;
+    }
     {
-      const bool ok = s_ok != 0;
       float az[HC];
       tc::ld16(ta, *reinterpret_cast<float(*)[16]>(az));
       tc::ld8(ta + 16, *reinterpret_cast<float(*)[8]>(az + 16));
@@ -411,7 +413,7 @@ __device__ __forceinline__ void wide_pair_body(const MC<float, D1, D2, DY>& mc, 
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int r = HC * h + c + u;
-          const float v = ((ok ? az[c + u] : 0.f) + azv[u]) + lqv[u] * eps[c + u];
+          const float v = (az[c + u] + azv[u]) + lqv[u] * eps[c + u];
           zsrc[r * M + j] = v;
         }
       }
