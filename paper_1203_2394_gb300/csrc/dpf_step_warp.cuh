@@ -335,7 +335,8 @@ __device__ __forceinline__ T lane_sum_in_order(const T* part) {
   return r;
 }
 
-// The phase of a warp whose wait gave up: it steps no group of a later filter of the launch either.
+// From here on the phase is that of a warp whose wait gave up: it steps no group of a later filter of
+// the launch either.
 constexpr uint32_t WARP_DEAD = 2;
 
 // A warp's bounded wait for its group's rows. False, in every lane, when it gave up: the timeout is
@@ -386,10 +387,6 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
                                          unsigned char* ws, uint64_t* bar, uint32_t& phase) {
   static_assert(MF == 0 || MF == 32 * PPL, "MF is 0 or 32 PPL");
   const int lane = threadIdx.x & 31;
-  if (phase == WARP_DEAD) {
-    if (lane == 0) atomicOr(a.err, ERR_TIMEOUT);
-    return;
-  }
   const int M = MF ? MF : a.M, L = a.L;
   const long long N = a.N;
   const long long NM = N * (long long)M;
@@ -428,6 +425,10 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
 
   long long g = gfirst;
   long long src_next = -1;  // the same in every lane
+  if (phase >= WARP_DEAD) {
+    if (lane == 0) atomicOr(a.err, ERR_TIMEOUT);
+    gend = 0;
+  }
   if (a.glist) {
     const long long G = group_count(a);
     if (G < gend) gend = G;
@@ -445,7 +446,8 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
     const long long i = group_at(a, g);
     if (!warp_rows_in(bar, phase, a.err, lane)) {
       phase = WARP_DEAD;
-      return;
+      gend = 0;  // (leaving by the loop's own end: a return from here cost the batched kernels 50 to 100 bytes of spills)
+      continue;
     }
     if (a.gskip && a.gskip[i]) {  // a group left untouched: pass its stage on
       __syncwarp();
