@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(1024) nl_step_kernel(const __grid_constant__ N
 // maxima (one warp reduction instruction each), the exponentials, and the lane's partial sums
 // to the table `part`, one row a sum; then a lane adds a row. Bound by issue: model 1 at
 // N = 65536, M = 128, L = 16 went from 806 us a step (10.9 k warp instructions a group, four warps
-// between barriers) to 322.
+// between barriers) to 313.
 // Shared memory of one warp, in floats.
 template <int D1, int D2>
 struct NLWarp {

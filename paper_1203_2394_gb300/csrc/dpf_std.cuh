@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(1024)
 // PPL consecutive inner particles in registers, every reduction and scan is a warp shuffle, the
 // local resampling takes the offspring ranges (no search), and the ancestor's rows of the next
 // group are bulk-copied into the warp's stage while this one's are used. A group takes 1.9 k warp instructions, not 6.9 k; the growth model's step (N = 65536,
-// M = 128) went from 581 to 197 us, 45% of the copy bandwidth; what bounds it now is the issue of
+// M = 128) went from 581 to 194 us, 46% of the copy bandwidth; what bounds it now is the issue of
 // the random numbers and the propagation at four warps a scheduler.
 // The component draw of x_t is made only where it is read (an x transition that depends
 // on z, or debug recording). The Gaussian form of the draw keeps the block kernel.

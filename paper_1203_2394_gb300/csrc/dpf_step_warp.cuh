@@ -446,7 +446,7 @@ __device__ __forceinline__ void warp_run(const MC<T, D1, D2, DY>& mc, const Step
     const long long i = group_at(a, g);
     if (!warp_rows_in(bar, phase, a.err, lane)) {
       phase = WARP_DEAD;
-      gend = 0;  // (leaving by the loop's own end: a return from here cost the batched kernels 50 to 100 bytes of spills)
+      gend = 0;  // (by the loop's own end: a return here cost the batched kernels 50 to 100 bytes of spills)
       continue;
     }
     if (a.gskip && a.gskip[i]) {  // a group left untouched: pass its stage on

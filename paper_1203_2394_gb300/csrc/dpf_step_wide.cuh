@@ -13,7 +13,8 @@
 // and what only one warp does (the next group's copies in, z_t's copies out, the outer weight) is
 // given to warps of the half that then waits for the other. Every sum that feeds a weight keeps the
 // block step's order, so the weights and every resampling decision keep their bits. Time steps of
-// the 64-state growth model, N = 32768, M = 256, L = 16: 5007 -> 3386 us a step; what bounds it now is shared
+// the 64-state growth model, N = 32768, M = 256, L = 16: 5007 -> 3343 us a step (the model read once a CTA from
+// the context's own copy; with it copied into a constant bank before every launch 3389); what bounds it now is shared
 // memory: the two projections read 56 rows of 8 weights for each particle (5 k cycles a group).
 #pragma once
 
